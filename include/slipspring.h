@@ -158,10 +158,10 @@ int ss_set_flow(ss_ctx* ctx, int elem, int64_t from_step, const double kappa[9])
 int ss_set_flow_table(ss_ctx* ctx, int n, const int32_t* elem, const int64_t* from_step, const double* kappa);
 
 /* Batched mode (support for many elements; not in the paper): when enabled,
- * ss_run advances all elements with one persistent launch per chunk of
- * chunk_steps steps, replayed from an explicitly built CUDA graph; CTAs take
- * (element, chain tile) work items from an atomic counter, longest chains
- * first.  Before the first batched launch an autotuner times the candidate lane
+ * ss_run advances all elements with one graph launch per chunk of chunk_steps
+ * steps, replayed from an explicitly built CUDA graph of one kernel per lane
+ * layout; each CTA runs one (element, chain tile) work item for the whole
+ * chunk, longest chains first.  Before the first batched launch an autotuner times the candidate lane
  * layouts of each chain length on a scratch ensemble and keeps the fastest (the
  * default layout unless another is at least 3% faster; results cached per
  * process).  Batched mode keeps the stress logs, not the

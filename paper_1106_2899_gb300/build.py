@@ -2,24 +2,28 @@
 
     python -m paper_1106_2899_gb300.build [--force] [--verbose]
 
-produces paper_1106_2899_gb300/libslipspring.so with one nvcc call (one
--gencode: arch=compute_103a,code=sm_103a).  No CPU fallback exists: without the
-library the Python binding raises.
+produces paper_1106_2899_gb300/libslipspring.so: one nvcc call per translation
+unit, in parallel (one -gencode: arch=compute_103a,code=sm_103a), then a link.
+No CPU fallback exists: without the library the Python binding raises.
 """
 import os
 import subprocess
 import sys
+import tempfile
+from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 LIB = os.path.join(PKG, "libslipspring.so")
-SOURCES = [os.path.join(CSRC, "ss_api.cu")]
-DEPS = SOURCES + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))] + [
+# the longest to compile first
+SOURCES = [os.path.join(CSRC, f) for f in ("ss_chunk_f64_flow.cu", "ss_chunk_f64.cu", "ss_chunk_f32_flow.cu",
+                                           "ss_chunk_f32.cu", "ss_batched.cu", "ss_adjoint.cu", "ss_api.cu")]
+DEPS = SOURCES + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h", ".inl"))] + [
     os.path.join(ROOT, "include", "slipspring.h")]
 
 NVCC_FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_103a,code=sm_103a", "-lineinfo",
-              "-Xcompiler", "-fPIC", "-shared", "--expt-relaxed-constexpr"]
+              "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr"]
 
 
 def nvcc():
@@ -33,13 +37,22 @@ def build(force: bool = False, verbose: bool = False) -> str:
     newest = max(os.path.getmtime(p) for p in DEPS)
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= newest:
         return LIB
-    tmp = LIB + ".tmp%d" % os.getpid()
-    cmd = [nvcc()] + NVCC_FLAGS + ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-o", tmp] + SOURCES
-    if verbose:
-        cmd.insert(1, "-Xptxas=-v")
-        print(" ".join(cmd))
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    flags = NVCC_FLAGS + ["-I", os.path.join(ROOT, "include"), "-I", CSRC] + (["-Xptxas=-v"] if verbose else [])
+    with tempfile.TemporaryDirectory(dir=PKG, prefix="_build_") as tmp:
+        objs = [os.path.join(tmp, os.path.basename(s) + ".o") for s in SOURCES]
+
+        def compile_one(src, obj):
+            cmd = [nvcc()] + flags + ["-c", "-o", obj, src]
+            if verbose:
+                print(" ".join(cmd))
+            subprocess.check_call(cmd)
+
+        with ThreadPoolExecutor(len(SOURCES)) as ex:
+            for f in [ex.submit(compile_one, s, o) for s, o in zip(SOURCES, objs)]:
+                f.result()
+        lib = os.path.join(tmp, "lib.so")
+        subprocess.check_call([nvcc(), "-shared", "-o", lib] + objs)
+        os.replace(lib, LIB)
     return LIB
 
 

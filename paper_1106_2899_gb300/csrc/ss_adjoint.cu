@@ -1,0 +1,25 @@
+// ss_adjoint.cu -- the reverse sweep of differentiation windows, by lane layout.
+#include "ss_adjoint.cuh"
+#include "ss_launch.h"
+
+namespace ssk {
+namespace {
+
+template <typename T>
+const void* adjoint_fn(int W, int B) {
+    switch (W * 16 + B) {
+        case 16 * 16 + 1: return (const void*)adjoint_kernel<T, 16, 1>;
+        case 16 * 16 + 2: return (const void*)adjoint_kernel<T, 16, 2>;
+        case 16 * 16 + 3: return (const void*)adjoint_kernel<T, 16, 3>;
+        case 16 * 16 + 4: return (const void*)adjoint_kernel<T, 16, 4>;
+        case 32 * 16 + 4: return (const void*)adjoint_kernel<T, 32, 4>;
+        default: return nullptr;
+    }
+}
+
+}  // namespace
+
+const void* adjoint_fn_f32(int W, int B) { return adjoint_fn<float>(W, B); }
+const void* adjoint_fn_f64(int W, int B) { return adjoint_fn<double>(W, B); }
+
+}  // namespace ssk

@@ -114,7 +114,7 @@ struct AdjArgs {
 };
 
 template <typename T, int W, int B>
-__global__ void __launch_bounds__(kChunkThreads, B == 1 ? SS_CTAS_PER_SM : SS_CTAS_PER_SM_MULTI)
+__global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
     adjoint_kernel(const AdjArgs a, const StepConst<T> c) {
     constexpr int SEGS = 32 / W;
     constexpr int NP = W * B;

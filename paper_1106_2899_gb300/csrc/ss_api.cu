@@ -20,6 +20,9 @@
 #include "slipspring.h"
 #include "ss_kernels.cuh"
 #include "ss_adjoint.cuh"
+#include "ss_corr.cuh"
+#include "ss_launch.h"
+#include "ss_state.cuh"
 
 namespace {
 
@@ -49,13 +52,11 @@ struct Elem {
     bool flow_dirty = true;
 };
 
-// one layout class of the batched launch: its items, counter and graph node
+// one layout class of the batched launch: its items and graph node
 struct BatchedClass {
     int k = 0;
     int2* items = nullptr;
-    int n_items = 0;
-    unsigned* next = nullptr;
-    int grid = 1, smem = 0;
+    int n_items = 0, smem = 0;
     cudaGraphNode_t node = nullptr;
 };
 
@@ -81,13 +82,12 @@ struct ss_ctx {
     long long launches = 0;
     bool timing = false;
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> events;  // chain-kernel launches while timing
-    // batched mode: one persistent launch per chunk over all elements
+    // batched mode: one graph launch per chunk over all elements
     bool batched = false;
     bool tuned = false;
     bool graph_dirty = true;
     ssk::ChunkArgs* d_elems = nullptr;
     int2* d_items = nullptr;
-    unsigned* d_next = nullptr;
     std::vector<BatchedClass> bclasses;
     cudaGraphExec_t gexec = nullptr;
     cudaGraph_t graph = nullptr;
@@ -173,28 +173,47 @@ void free_elem(Elem& e) {
     e.n_kap_d = 0;
 }
 
-// Chain layout for N beads: W lanes per chain, B beads per lane (NP = W*B).
-#ifndef SS_N32_LAYOUT_W32
-#define SS_N32_LAYOUT_W32 0
-#endif
-void layout_for(int N, int* W, int* B) {
-    if (N <= 16) {
-        *W = 16, *B = 1;
-    } else if (N <= 32) {
-        if (SS_N32_LAYOUT_W32)
-            *W = 32, *B = 1;
+// Chain layout for N beads: W lanes per chain, B beads per lane (W*B >= N).  Every
+// layout of the chain kernel rounds each sum over beads alike, so the choice is
+// free.  Eight lanes per chain leave fewer lanes idle at N <= 8 and 17..24 and share
+// the slot work and the reductions of a warp among four chains, but run half as
+// many warps: they win once the chip is full (us per step, 8 against 16 lanes:
+// N = 24: 1.70 / 1.46 at 4096 chains, 2.39 / 2.50 at 8192, 14.6 / 16.5 at 65536;
+// N = 16: 3.10 / 2.89 at 16384, 10.0 / 10.4 at 65536).  FP64 work is bound by the
+// FP64 pipe of the SM partitions a launch reaches, and takes the wider layouts.
+void layout_for(int M, int N, int prec, int integrator, int* W, int* B) {
+    const bool narrow = prec == SS_FP32 && integrator == SS_EULER;
+    if (N <= 8) {
+        *W = 8, *B = 1;
+    } else if (N <= 16) {
+        if (narrow && M >= 40000)
+            *W = 8, *B = 2;
         else
-            *W = 16, *B = 2;
+            *W = 16, *B = 1;
+    } else if (N <= 24 && narrow && M >= 8192) {
+        *W = 8, *B = 3;
+    } else if (N <= 32) {
+        *W = 16, *B = 2;
     } else if (N <= 48) {
         *W = 16, *B = 3;
     } else if (N <= 64) {
         *W = 16, *B = 4;
+    } else if (N <= 96) {
+        *W = 32, *B = 3;
     } else {
         *W = 32, *B = 4;
     }
 }
 
 int chains_per_cta(int W) { return kWarpsPerCta * (32 / W); }
+
+// the chain kernel of this precision (windows refuse a velocity gradient)
+template <typename T>
+const void* chunk_fn(int W, int B, int win, bool flow, bool heun, bool corr) {
+    if (sizeof(T) == 8)
+        return flow ? ssk::chunk_fn_f64_flow(W, B, win, heun, corr) : ssk::chunk_fn_f64(W, B, win, heun, corr);
+    return flow ? ssk::chunk_fn_f32_flow(W, B, win, heun, corr) : ssk::chunk_fn_f32(W, B, win, heun, corr);
+}
 
 // z_max by default: one slot per bead (Sec. 3.2), at most SS_MAX_SLOTS
 int default_zmax(int N) { return std::min(N, SS_MAX_SLOTS); }
@@ -288,7 +307,7 @@ bool flow_in_window(const Elem& e, long long t0, int nsteps) {
     return false;
 }
 
-template <typename T, int W, int B>
+template <typename T>
 int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
     NvtxRange range("chain kernel + correlator launch");
     const ss_params& p = c->P;
@@ -351,34 +370,27 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
         a.snap_t0 = c->opt_snap_t0;
         a.snap_steps = c->win.ce;
     }
-    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, W, B, a.nlog_chunk);
-    // differentiation windows run the instantiation with the window hooks; an
-    // FP32 launch without a velocity gradient, and a Heun launch without one in
-    // either precision, the one without the flow terms
-    const bool win = c->opt_tape_mode != 0 || c->opt_snap;
-    void (*kern)(const ssk::ChunkArgs, const ssk::StepConst<T>) =
-        win ? ssk::chunk_kernel<T, W, B, true, true> : ssk::chunk_kernel<T, W, B, false, true>;
-    if (c->P.integrator == SS_HEUN) {
-        kern = ssk::chunk_kernel<T, W, B, false, true, true>;  // windows refuse this integrator
-        if (!flow_in_window(e, t0, nsteps)) kern = ssk::chunk_kernel<T, W, B, false, false, true>;
-    } else if constexpr (std::is_same<T, float>::value) {
-        if (!flow_in_window(e, t0, nsteps))
-            kern = win ? ssk::chunk_kernel<T, W, B, true, false> : ssk::chunk_kernel<T, W, B, false, false>;
-    }
+    // differentiation windows run the instantiations with the window hooks (they
+    // refuse a velocity gradient), a launch without a velocity gradient the one
+    // without the flow terms
+    const int win = c->opt_tape_mode == 1 ? ssk::kWinRecord : (c->opt_tape_mode == 2 ? ssk::kWinReplay : ssk::kWinOff);
+    const void* kern = chunk_fn<T>(e.W, e.B, win, flow_in_window(e, t0, nsteps), c->P.integrator == SS_HEUN, corr);
+    if (!kern) return fail(c, SS_EINVAL, "no chain kernel for this layout");
+    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk);
     // the attribute belongs to the current device: set it on every launch that
     // needs more than the default 48 KiB (a host call per launch of many steps)
     if (plan.total > 48 * 1024)
         SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total));
-    const ssk::StepConst<T> sc = step_const<T>(c, e.N);
-    const int ctas = (e.M + chains_per_cta(W) - 1) / chains_per_cta(W);
+    ssk::StepConst<T> sc = step_const<T>(c, e.N);
+    const int cpc = chains_per_cta(e.W), ctas = (e.M + cpc - 1) / cpc;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (c->timing) {
         SS_CUDA(c, cudaEventCreate(&ev0));
         SS_CUDA(c, cudaEventCreate(&ev1));
         SS_CUDA(c, cudaEventRecord(ev0, c->stream));
     }
-    kern<<<ctas, kThreads, plan.total, c->stream>>>(a, sc);
-    SS_CUDA(c, cudaGetLastError());
+    void* args[] = {(void*)&a, (void*)&sc};
+    SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, c->stream));
     if (c->timing) {
         SS_CUDA(c, cudaEventRecord(ev1, c->stream));
         c->events.emplace_back(ev0, ev1);
@@ -393,17 +405,6 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
         c->launches += nl;
     }
     return SS_OK;
-}
-
-template <typename T>
-int dispatch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
-    if (e.W == 32) return e.B == 4 ? launch_chunk<T, 32, 4>(c, e, t0, nsteps) : launch_chunk<T, 32, 1>(c, e, t0, nsteps);
-    switch (e.B) {
-        case 1: return launch_chunk<T, 16, 1>(c, e, t0, nsteps);
-        case 2: return launch_chunk<T, 16, 2>(c, e, t0, nsteps);
-        case 3: return launch_chunk<T, 16, 3>(c, e, t0, nsteps);
-        default: return launch_chunk<T, 16, 4>(c, e, t0, nsteps);
-    }
 }
 
 template <typename T>
@@ -604,10 +605,10 @@ std::vector<int> group_sizes(const Elem& e) {
 }
 
 // ------------------------------------------------------------ batched ----
-// Lane layouts the batched path can use; one persistent kernel per layout.
-constexpr int kBatchedLayouts = 7;
-constexpr int kLayoutW[kBatchedLayouts] = {16, 16, 16, 32, 8, 16, 32};
-constexpr int kLayoutB[kBatchedLayouts] = {1, 2, 3, 1, 2, 4, 4};
+// Lane layouts the batched path can use; one kernel per layout.
+constexpr int kBatchedLayouts = 10;
+constexpr int kLayoutW[kBatchedLayouts] = {16, 16, 16, 16, 8, 8, 8, 32, 32, 32};
+constexpr int kLayoutB[kBatchedLayouts] = {1, 2, 3, 4, 1, 2, 3, 1, 3, 4};
 
 int layout_class(int W, int B) {
     for (int k = 0; k < kBatchedLayouts; ++k)
@@ -620,12 +621,10 @@ void free_batched(ss_ctx* c) {
     if (c->graph) cudaGraphDestroy(c->graph);
     if (c->d_elems) cudaFree(c->d_elems);
     if (c->d_items) cudaFree(c->d_items);
-    if (c->d_next) cudaFree(c->d_next);
     c->gexec = nullptr;
     c->graph = nullptr;
     c->d_elems = nullptr;
     c->d_items = nullptr;
-    c->d_next = nullptr;
     c->bclasses.clear();
     c->graph_dirty = true;
 }
@@ -679,22 +678,9 @@ std::vector<int2> make_items(const std::vector<Elem>& el, int W, int B) {
     return items;
 }
 
-template <typename T, int W, int B>
-const void* batched_fn() {
-    return (const void*)ssk::batched_kernel<T, W, B>;
-}
-
 template <typename T>
 const void* batched_fn_of(int k) {
-    switch (k) {
-        case 0: return batched_fn<T, 16, 1>();
-        case 1: return batched_fn<T, 16, 2>();
-        case 2: return batched_fn<T, 16, 3>();
-        case 3: return batched_fn<T, 32, 1>();
-        case 4: return batched_fn<T, 8, 2>();
-        case 5: return batched_fn<T, 16, 4>();
-        default: return batched_fn<T, 32, 4>();
-    }
+    return sizeof(T) == 8 ? ssk::batched_fn_f64(kLayoutW[k], kLayoutB[k]) : ssk::batched_fn_f32(kLayoutW[k], kLayoutB[k]);
 }
 
 template <typename T>
@@ -703,39 +689,26 @@ int batched_smem_bytes(const ss_ctx* c, int k) {
     return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog).total;
 }
 
-// persistent grid size of class k: resident CTAs per SM x SMs, at most one per item
-template <typename T>
-int batched_grid(ss_ctx* c, int k, int n_items, int smem, int* grid) {
-    const void* fn = batched_fn_of<T>(k);
-    SS_CUDA(c, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    int per_sm = 0, dev = 0, sms = 0;
-    SS_CUDA(c, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem));
-    SS_CUDA(c, cudaGetDevice(&dev));
-    SS_CUDA(c, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    *grid = std::max(1, std::min(n_items, std::max(1, per_sm) * sms));
-    return SS_OK;
-}
-
 template <typename T>
 int batched_launch_direct(ss_ctx* c, int k, const ssk::ChunkArgs* d_elems, const int2* d_items, int n_items,
-                          unsigned* d_next, long long t0, int ns, int grid, int smem) {
-    SS_CUDA(c, cudaMemsetAsync(d_next, 0, sizeof(unsigned), c->stream));
+                          long long t0, int ns, int smem) {
     ssk::RunInfo info{t0, ns, c->log_m0};
     ssk::StepConst<T> sc = step_const<T>(c, 32);
-    void* args[] = {(void*)&d_elems, (void*)&d_items, (void*)&n_items, (void*)&d_next, (void*)&info, (void*)&sc};
-    SS_CUDA(c, cudaLaunchKernel(batched_fn_of<T>(k), dim3(grid), dim3(kThreads), args, smem, c->stream));
+    void* args[] = {(void*)&d_elems, (void*)&d_items, (void*)&info, (void*)&sc};
+    SS_CUDA(c, cudaLaunchKernel(batched_fn_of<T>(k), dim3(n_items), dim3(kThreads), args, smem, c->stream));
     return SS_OK;
 }
 
-// Candidate lane layouts with the same padded stride NP as the default.
+// Candidate lane layouts of the batched kernel, the default first.
 std::vector<std::pair<int, int>> layout_candidates(int N) {
-    int W, B;
-    layout_for(N, &W, &B);
-    const int NP = W * B;
-    std::vector<std::pair<int, int>> cand = {{W, B}};
-    if (NP == 32) cand.push_back({32, 1});
-    if (NP == 16) cand.push_back({8, 2});
-    return cand;
+    if (N <= 8) return {{8, 1}};
+    if (N <= 16) return {{16, 1}, {8, 2}};
+    if (N <= 24) return {{16, 2}, {8, 3}, {32, 1}};
+    if (N <= 32) return {{16, 2}, {32, 1}};
+    if (N <= 48) return {{16, 3}};
+    if (N <= 64) return {{16, 4}};
+    if (N <= 96) return {{32, 3}};
+    return {{32, 4}};
 }
 
 // Project-written autotuner: for each chain length, time every candidate layout
@@ -765,14 +738,13 @@ int autotune(ss_ctx* c) {
                 for (const Elem& e : c->el)
                     if (e.N == N) total += e.M;
                 Elem t;
-                // enough chains that every candidate runs many work items per
-                // persistent CTA: the comparison is then one of steady throughput,
-                // not of the tail of a partly filled wave
+                // as many chains as the workload has, up to enough for many waves:
+                // the comparison is then one of steady throughput
                 t.M = (int)std::max<long long>(256, std::min<long long>(65536, total));
                 t.N = N;
                 t.W = bestW;
                 t.B = bestB;
-                t.NP = t.W * t.B;
+                t.NP = ssk::row_stride(N);
                 t.zmax = c->P.z_max > 0 ? std::min(c->P.z_max, N) : default_zmax(N);
                 t.slices = (t.M + ssk::kSliceChains - 1) / ssk::kSliceChains;
                 t.groups = 1;
@@ -787,11 +759,9 @@ int autotune(ss_ctx* c) {
                 if (rc == SS_OK) rc = upload_flow(c, t);
                 ssk::ChunkArgs* dd = nullptr;
                 int2* di = nullptr;
-                unsigned* dn = nullptr;
                 unsigned long long* dcnt = nullptr;  // the trials count into scratch, not the context
                 if (rc == SS_OK && (cudaMalloc(&dd, sizeof(ssk::ChunkArgs)) != cudaSuccess ||
-                                    cudaMalloc(&di, sizeof(int2) * ((t.M + 3) / 4 + 1)) != cudaSuccess ||
-                                    cudaMalloc(&dn, sizeof(unsigned)) != cudaSuccess ||
+                                    cudaMalloc(&di, sizeof(int2) * t.M) != cudaSuccess ||
                                     cudaMalloc(&dcnt, 16 * sizeof(unsigned long long)) != cudaSuccess))
                     rc = fail(c, SS_ENOMEM, "autotune: allocation failed");
                 const long long saved_m0 = c->log_m0;
@@ -813,19 +783,18 @@ int autotune(ss_ctx* c) {
                     ssk::ChunkArgs desc = make_desc(c, t);
                     desc.counters = dcnt;
                     desc.status = reinterpret_cast<int32_t*>(dcnt + 8);
-                    int grid = 1;
                     const int smem = batched_smem_bytes<T>(c, k);
-                    rc = batched_grid<T>(c, k, (int)items.size(), smem, &grid);
-                    if (rc != SS_OK) break;
+                    SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    smem));
                     SS_CUDA(c, cudaMemcpy(dd, &desc, sizeof(desc), cudaMemcpyHostToDevice));
                     SS_CUDA(c, cudaMemcpy(di, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice));
                     cudaEvent_t e0, e1;
                     SS_CUDA(c, cudaEventCreate(&e0));
                     SS_CUDA(c, cudaEventCreate(&e1));
-                    rc = batched_launch_direct<T>(c, k, dd, di, (int)items.size(), dn, 0, 32, grid, smem);
+                    rc = batched_launch_direct<T>(c, k, dd, di, (int)items.size(), 0, 32, smem);
                     cudaEventRecord(e0, c->stream);
                     if (rc == SS_OK)
-                        rc = batched_launch_direct<T>(c, k, dd, di, (int)items.size(), dn, 32, 256, grid, smem);
+                        rc = batched_launch_direct<T>(c, k, dd, di, (int)items.size(), 32, 256, smem);
                     cudaEventRecord(e1, c->stream);
                     cudaEventSynchronize(e1);
                     float ms = 0.f;
@@ -846,7 +815,6 @@ int autotune(ss_ctx* c) {
                 c->P.log_every = saved_log;
                 if (dd) cudaFree(dd);
                 if (di) cudaFree(di);
-                if (dn) cudaFree(dn);
                 if (dcnt) cudaFree(dcnt);
                 free_elem(t);
                 if (rc != SS_OK) return rc;
@@ -862,9 +830,8 @@ int autotune(ss_ctx* c) {
     return SS_OK;
 }
 
-// Descriptors, work items and the graph of one batched launch: per layout
-// class a counter reset and a persistent kernel, the classes on independent
-// branches so that they share the GPU.
+// Descriptors, work items and the graph of one batched launch: a kernel per
+// layout class, on independent branches so that they share the GPU.
 template <typename T>
 int batched_prepare(ss_ctx* c) {
     free_batched(c);
@@ -878,7 +845,6 @@ int batched_prepare(ss_ctx* c) {
     }
     SS_CUDA(c, cudaMalloc(&c->d_elems, sizeof(ssk::ChunkArgs) * descs.size()));
     SS_CUDA(c, cudaMalloc(&c->d_items, sizeof(int2) * std::max<size_t>(1, total)));
-    SS_CUDA(c, cudaMalloc(&c->d_next, sizeof(unsigned) * kBatchedLayouts));
     SS_CUDA(c, cudaMemcpy(c->d_elems, descs.data(), sizeof(ssk::ChunkArgs) * descs.size(), cudaMemcpyHostToDevice));
     SS_CUDA(c, cudaGraphCreate(&c->graph, 0));
     size_t off = 0;
@@ -889,29 +855,19 @@ int batched_prepare(ss_ctx* c) {
         bc.k = k;
         bc.items = c->d_items + off;
         bc.n_items = (int)cls[k].size();
-        bc.next = c->d_next + k;
         bc.smem = batched_smem_bytes<T>(c, k);
-        int rc = batched_grid<T>(c, k, bc.n_items, bc.smem, &bc.grid);
-        if (rc != SS_OK) return rc;
-        cudaMemsetParams mp{};
-        mp.dst = bc.next;
-        mp.value = 0;
-        mp.elementSize = sizeof(unsigned);
-        mp.width = 1;
-        mp.height = 1;
-        cudaGraphNode_t mnode;
-        SS_CUDA(c, cudaGraphAddMemsetNode(&mnode, c->graph, nullptr, 0, &mp));
+        SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, bc.smem));
         ssk::RunInfo info{0, 1, 0};
         ssk::StepConst<T> sc = step_const<T>(c, 32);
         const ssk::ChunkArgs* pe = c->d_elems;
-        void* args[] = {(void*)&pe, (void*)&bc.items, (void*)&bc.n_items, (void*)&bc.next, (void*)&info, (void*)&sc};
+        void* args[] = {(void*)&pe, (void*)&bc.items, (void*)&info, (void*)&sc};
         cudaKernelNodeParams kp{};
         kp.func = (void*)batched_fn_of<T>(k);
-        kp.gridDim = dim3(bc.grid);
+        kp.gridDim = dim3(bc.n_items);
         kp.blockDim = dim3(kThreads);
         kp.sharedMemBytes = bc.smem;
         kp.kernelParams = args;
-        SS_CUDA(c, cudaGraphAddKernelNode(&bc.node, c->graph, &mnode, 1, &kp));
+        SS_CUDA(c, cudaGraphAddKernelNode(&bc.node, c->graph, nullptr, 0, &kp));
         c->bclasses.push_back(bc);
         off += cls[k].size();
     }
@@ -928,10 +884,10 @@ int batched_chunk(ss_ctx* c, long long t0, int ns) {
     ssk::StepConst<T> sc = step_const<T>(c, 32);
     const ssk::ChunkArgs* pe = c->d_elems;
     for (BatchedClass& bc : c->bclasses) {
-        void* args[] = {(void*)&pe, (void*)&bc.items, (void*)&bc.n_items, (void*)&bc.next, (void*)&info, (void*)&sc};
+        void* args[] = {(void*)&pe, (void*)&bc.items, (void*)&info, (void*)&sc};
         cudaKernelNodeParams kp{};
         kp.func = (void*)batched_fn_of<T>(bc.k);
-        kp.gridDim = dim3(bc.grid);
+        kp.gridDim = dim3(bc.n_items);
         kp.blockDim = dim3(kThreads);
         kp.sharedMemBytes = bc.smem;
         kp.kernelParams = args;
@@ -989,7 +945,7 @@ int seg_len(const ss_ctx* c, int seg) {
     return (int)std::min<long long>(c->win.ce, left);
 }
 
-template <typename T, int W, int B>
+template <typename T>
 int launch_adjoint(ss_ctx* c, Elem& e, int seg) {
     auto& w = c->win;
     const size_t ts = sizeof(T);
@@ -1014,25 +970,18 @@ int launch_adjoint(ss_ctx* c, Elem& e, int seg) {
     a.destroy_new = c->P.destroy_new;
     a.create_mode = c->P.create_mode;
     a.zmax = e.zmax;
+    const int W = e.NP <= 64 ? 16 : 32, B = e.NP / W;  // snapshots and tape have the same columns in every layout
     const int smem = kWarpsPerCta * 32 * B * (int)(2 * sizeof(ssk::Pos<T>) + sizeof(ssk::SlotRec<T>) + 8);
+    const void* kern = sizeof(T) == 8 ? ssk::adjoint_fn_f64(W, B) : ssk::adjoint_fn_f32(W, B);
+    if (!kern) return fail(c, SS_EINVAL, "no adjoint kernel for this layout");
     if (smem > 48 * 1024)
-        SS_CUDA(c, cudaFuncSetAttribute(ssk::adjoint_kernel<T, W, B>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int ctas = (e.M + chains_per_cta(W) - 1) / chains_per_cta(W);
-    ssk::adjoint_kernel<T, W, B><<<ctas, kThreads, smem, c->stream>>>(a, step_const<T>(c, e.N));
-    SS_CUDA(c, cudaGetLastError());
+    ssk::StepConst<T> sc = step_const<T>(c, e.N);
+    void* args[] = {(void*)&a, (void*)&sc};
+    SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, smem, c->stream));
     c->launches++;
     return SS_OK;
-}
-
-template <typename T>
-int dispatch_adjoint(ss_ctx* c, Elem& e, int seg) {
-    if (e.W == 32) return e.B == 4 ? launch_adjoint<T, 32, 4>(c, e, seg) : launch_adjoint<T, 32, 1>(c, e, seg);
-    switch (e.B) {
-        case 1: return launch_adjoint<T, 16, 1>(c, e, seg);
-        case 2: return launch_adjoint<T, 16, 2>(c, e, seg);
-        case 3: return launch_adjoint<T, 16, 3>(c, e, seg);
-        default: return launch_adjoint<T, 16, 4>(c, e, seg);
-    }
 }
 
 template <typename T>
@@ -1099,12 +1048,12 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
         c->opt_snap = true;
         c->opt_corr_off = true;
         c->opt_snap_t0 = w.t_start + (long long)seg * w.ce;
-        rc = dispatch_chunk<T>(c, e, c->opt_snap_t0, seg_len(c, seg));
+        rc = launch_chunk<T>(c, e, c->opt_snap_t0, seg_len(c, seg));
         c->opt_tape_mode = 0;
         c->opt_snap = false;
         c->opt_corr_off = false;
         if (rc != SS_OK) return rc;
-        rc = dispatch_adjoint<T>(c, e, seg);
+        rc = launch_adjoint<T>(c, e, seg);
         if (rc != SS_OK) return rc;
     }
     // the live state is the window's final state again
@@ -1160,8 +1109,8 @@ int ss_create(ss_ctx** out, const ss_element* elems, int n_elems, int precision,
         Elem e;
         e.M = elems[i].n_chains;
         e.N = elems[i].n_beads;
-        layout_for(e.N, &e.W, &e.B);
-        e.NP = e.W * e.B;
+        layout_for(e.M, e.N, precision, SS_EULER, &e.W, &e.B);
+        e.NP = ssk::row_stride(e.N);
         e.chain_base = base;
         base += (uint32_t)e.M;
         c->el.push_back(e);
@@ -1221,6 +1170,7 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
     c->k_b = kb;
     c->k_s = ks;
     c->levels = p.corr_levels > 0 ? p.corr_levels : 0;
+    c->tuned = false;
     c->step = 0;
     c->initialized = false;
     // with the correlator on, a launch covers at most kCorrMaxSteps steps
@@ -1228,6 +1178,7 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
     const size_t ts = tsize(c);
     for (Elem& e : c->el) {
         e.zmax = p.z_max > 0 ? p.z_max : default_zmax(e.N);
+        layout_for(e.M, e.N, c->prec, p.integrator, &e.W, &e.B);
         e.slices = (e.M + ssk::kSliceChains - 1) / ssk::kSliceChains;
         e.groups = std::min(p.groups, e.slices);
         SS_CUDA(c, cudaMalloc(&e.R, (size_t)e.M * 3 * e.NP * ts));
@@ -1294,7 +1245,7 @@ int ss_set_batched(ss_ctx* c, int enable) {
     c->batched = enable != 0;
     c->graph_dirty = true;
     if (!c->batched) {  // back to the per-element kernels' layouts (same padded stride)
-        for (Elem& e : c->el) layout_for(e.N, &e.W, &e.B);
+        for (Elem& e : c->el) layout_for(e.M, e.N, c->prec, c->P.integrator, &e.W, &e.B);
         c->tuned = false;
     }
     return SS_OK;
@@ -1331,8 +1282,8 @@ int ss_run(ss_ctx* c, int64_t n_steps) {
     while (left > 0) {
         const int ns = (int)std::min<long long>(left, p.chunk_steps);
         for (Elem& e : c->el) {
-            int rc = c->prec == SS_FP64 ? dispatch_chunk<double>(c, e, c->step, ns)
-                                        : dispatch_chunk<float>(c, e, c->step, ns);
+            int rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, ns)
+                                        : launch_chunk<float>(c, e, c->step, ns);
             if (rc != SS_OK) return rc;
         }
         c->step += ns;
@@ -1757,7 +1708,7 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
         c->opt_tape_mode = replay ? 2 : 1;
         c->opt_series = true;
         const int len = seg_len(c, seg);
-        rc = c->prec == SS_FP64 ? dispatch_chunk<double>(c, e, c->step, len) : dispatch_chunk<float>(c, e, c->step, len);
+        rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, len) : launch_chunk<float>(c, e, c->step, len);
         c->opt_tape_mode = 0;
         c->opt_series = false;
         if (rc != SS_OK) return rc;
@@ -1839,11 +1790,11 @@ __global__ void noalloc_put_kappa_kernel(const KappaVal kv, double* __restrict__
     if (threadIdx.x < 9) dst[threadIdx.x] = kv.k[threadIdx.x];
 }
 
-template <typename T, int W, int B>
-int noalloc_launches(ss_ctx* c, const ss_params& p, int M, int N, int zmax, uint32_t chain_base, int64_t t0,
+template <typename T>
+int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, int zmax, uint32_t chain_base, int64_t t0,
                      int64_t n_steps, void* R, void* A, int32_t* S, int32_t* Z, unsigned char* scr,
                      size_t off_hist, size_t off_ser, size_t off_lev, int ser_cap, size_t off_acc64, size_t off_kap,
-                     size_t off_kfrom, size_t off_cnt, size_t off_status, cudaStream_t st) {
+                     size_t off_kfrom, size_t off_cnt, size_t off_status, bool flow, cudaStream_t st) {
     ssk::ChunkArgs a{};
     a.R = R;
     a.A = A;
@@ -1874,20 +1825,22 @@ int noalloc_launches(ss_ctx* c, const ss_params& p, int M, int N, int zmax, uint
         a.series = scr + off_ser;
         a.series_row0 = 0;
     }
+    const void* kern = chunk_fn<T>(W, B, ssk::kWinOff, flow, false, c->levels > 0);
+    if (!kern) return SS_EINVAL;
+    const int cpc = chains_per_cta(W);
     const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, W, B, 0);
-    if (plan.total > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(ssk::chunk_kernel<T, W, B, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             plan.total);
-        if (e != cudaSuccess) return SS_ECUDA;
-    }
-    const ssk::StepConst<T> sc = step_const<T>(c, N);
+    if (plan.total > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total) != cudaSuccess)
+        return SS_ECUDA;
+    ssk::StepConst<T> sc = step_const<T>(c, N);
+    void* args[] = {(void*)&a, (void*)&sc};
     int64_t done = 0;
     while (done < n_steps) {
         const int ns = (int)std::min<int64_t>(n_steps - done, c->levels > 0 ? ser_cap : p.chunk_steps);
         a.t0 = t0 + done;
         a.nsteps = ns;
-        ssk::chunk_kernel<T, W, B, false, true><<<(M + chains_per_cta(W) - 1) / chains_per_cta(W), kThreads, plan.total, st>>>(a, sc);
-        if (cudaGetLastError() != cudaSuccess) return SS_ECUDA;
+        if (cudaLaunchKernel(kern, dim3((M + cpc - 1) / cpc), dim3(kThreads), args, plan.total, st) != cudaSuccess)
+            return SS_ECUDA;
         if (c->levels > 0 &&
             corr_launches<T>(static_cast<const T*>(a.series), ns, M, c->levels, done,
                              reinterpret_cast<T*>(scr + off_hist), reinterpret_cast<double*>(scr + off_acc64), nullptr,
@@ -1921,8 +1874,8 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
     Elem e;
     e.M = n_chains;
     e.N = n_beads;
-    layout_for(n_beads, &e.W, &e.B);
-    e.NP = e.W * e.B;
+    layout_for(n_chains, n_beads, precision, SS_EULER, &e.W, &e.B);
+    e.NP = ssk::row_stride(e.N);
     c.el.push_back(e);
     {
         ss_params q = *params;
@@ -2000,27 +1953,14 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
     if (cudaMemsetAsync(scr, 0, off_ser, st) != cudaSuccess) return SS_ECUDA;
     KappaVal kv{};
     if (kappa) std::memcpy(kv.k, kappa, sizeof(kv.k));
+    const bool flow = std::any_of(kv.k, kv.k + 9, [](double k) { return k != 0.0; });
     noalloc_put_kappa_kernel<<<1, 32, 0, st>>>(kv, reinterpret_cast<double*>(scr + off_kap));
     if (cudaGetLastError() != cudaSuccess) return SS_ECUDA;
     const int zm = c.el[0].zmax;
 #define SS_NOALLOC_ARGS                                                                                          \
-    &c, c.P, n_chains, n_beads, zm, chain_base, t0, n_steps, R, A, S, Z, scr, off_hist, off_ser, off_lev,       \
-        ser_cap, off_acc64, off_kap, off_kfrom, off_cnt, off_status, st
-    if (precision == SS_FP64) {
-        if (e.W == 32 && e.B == 4) rc = noalloc_launches<double, 32, 4>(SS_NOALLOC_ARGS);
-        else if (e.W == 32) rc = noalloc_launches<double, 32, 1>(SS_NOALLOC_ARGS);
-        else if (e.B == 1) rc = noalloc_launches<double, 16, 1>(SS_NOALLOC_ARGS);
-        else if (e.B == 2) rc = noalloc_launches<double, 16, 2>(SS_NOALLOC_ARGS);
-        else if (e.B == 3) rc = noalloc_launches<double, 16, 3>(SS_NOALLOC_ARGS);
-        else rc = noalloc_launches<double, 16, 4>(SS_NOALLOC_ARGS);
-    } else {
-        if (e.W == 32 && e.B == 4) rc = noalloc_launches<float, 32, 4>(SS_NOALLOC_ARGS);
-        else if (e.W == 32) rc = noalloc_launches<float, 32, 1>(SS_NOALLOC_ARGS);
-        else if (e.B == 1) rc = noalloc_launches<float, 16, 1>(SS_NOALLOC_ARGS);
-        else if (e.B == 2) rc = noalloc_launches<float, 16, 2>(SS_NOALLOC_ARGS);
-        else if (e.B == 3) rc = noalloc_launches<float, 16, 3>(SS_NOALLOC_ARGS);
-        else rc = noalloc_launches<float, 16, 4>(SS_NOALLOC_ARGS);
-    }
+    &c, e.W, e.B, c.P, n_chains, n_beads, zm, chain_base, t0, n_steps, R, A, S, Z, scr, off_hist, off_ser, off_lev,       \
+        ser_cap, off_acc64, off_kap, off_kfrom, off_cnt, off_status, flow, st
+    rc = precision == SS_FP64 ? noalloc_launches<double>(SS_NOALLOC_ARGS) : noalloc_launches<float>(SS_NOALLOC_ARGS);
 #undef SS_NOALLOC_ARGS
     if (rc != SS_OK) return rc;
     if (corr_out && corr) {

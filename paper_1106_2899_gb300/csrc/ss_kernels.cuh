@@ -121,7 +121,14 @@ struct Mth;
 
 template <>
 struct Mth<float> {
-    static __device__ __forceinline__ float neg2log(float x) { return __log2f(x) * -1.3862943611198906f; }
+    // log2 of a normal x > 0 by the hardware approximation, without the scaling of
+    // subnormal arguments that __log2f carries (every argument here is >= 2^-24)
+    static __device__ __forceinline__ float log2(float x) {
+        float r;
+        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+        return r;
+    }
+    static __device__ __forceinline__ float neg2log(float x) { return log2(x) * -1.3862943611198906f; }
     // sqrt of x >= 0 by the hardware approximation (sqrt.approx); x = 0 gives 0
     static __device__ __forceinline__ float sqrt(float x) {
         float r;
@@ -132,6 +139,7 @@ struct Mth<float> {
     static __device__ __forceinline__ float exp(float x) { return __expf(x); }
     static __device__ __forceinline__ float div(float a, float b) { return __fdividef(a, b); }
     static __device__ __forceinline__ bool finite(float x) { return isfinite(x); }
+    static __device__ __forceinline__ float inf() { return __int_as_float(0x7f800000); }
 };
 
 template <>
@@ -142,6 +150,7 @@ struct Mth<double> {
     static __device__ __forceinline__ double exp(double x) { return ::exp(x); }
     static __device__ __forceinline__ double div(double a, double b) { return a / b; }
     static __device__ __forceinline__ bool finite(double x) { return isfinite(x); }
+    static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000ll); }
 };
 
 // pi / 2^23 in both precisions (a power-of-two scaling of pi)
@@ -187,7 +196,7 @@ __device__ __forceinline__ float2 pk(float a) { return make_float2(a, a); }
 __device__ __forceinline__ void box_muller_x2(uint32_t a0, uint32_t b0, uint32_t a1, uint32_t b1, float& c0,
                                               float& s0, float& c1, float& s1) {
     const float2 v = __fmul2_rn(pk(float((a0 >> 8) + 1u), float((a1 >> 8) + 1u)), pk(1.0f / 16777216.0f));
-    const float2 m = __fmul2_rn(pk(__log2f(v.x), __log2f(v.y)), pk(-1.3862943611198906f));
+    const float2 m = __fmul2_rn(pk(Mth<float>::log2(v.x), Mth<float>::log2(v.y)), pk(-1.3862943611198906f));
     const float2 r = pk(Mth<float>::sqrt(m.x), Mth<float>::sqrt(m.y));
     const float2 th = __fmul2_rn(pk(float(int(b0 >> 8) - (1 << 23)), float(int(b1 >> 8) - (1 << 23))),
                                  pk(3.14159265358979323846f / 8388608.0f));
@@ -267,8 +276,8 @@ struct ChunkArgs {
 // decision byte of one slot in one step (tape): hop, creation, destruction
 constexpr uint8_t kTapeUp = 1, kTapeDown = 2, kTapeNew0 = 4, kTapeNewN = 8, kTapeKillOld = 16, kTapeKillNew = 32;
 
-// One slip-spring slot as the force loop reads it from shared memory:
-// anchor and bead index (-1: empty slot), 16 bytes in FP32.
+// One slip-spring record in shared memory: a vector and an integer (the bead
+// index in the re-indexing, a flag in the spring tables), 16 bytes in FP32.
 template <typename T>
 struct __align__(16) SlotRec {
     T x, y, z;
@@ -281,36 +290,65 @@ struct __align__(16) Pos {
     T x, y, z, w;
 };
 
-// threads per CTA of the chunk kernel, and resident CTAs per SM it is compiled for
-constexpr int kChunkThreads = 128;
-#ifndef SS_CTAS_PER_SM
-#define SS_CTAS_PER_SM 6
-#endif
-#ifndef SS_CTAS_PER_SM_MULTI
-#define SS_CTAS_PER_SM_MULTI 5  // for layouts with several beads per lane
-#endif
-#ifndef SS_CTAS_PER_SM_BATCHED_MULTI
-#define SS_CTAS_PER_SM_BATCHED_MULTI 4  // the batched kernel with 3 or more beads per lane (it reads its
-#endif                                  // arguments through a pointer; 2 beads per lane fit 5 CTAs/SM)
+// Threads per CTA of the chain kernels: one warp, so that a small ensemble spreads
+// over the SMs and the last CTAs of a large one leave no warps waiting for their
+// CTA (against CTAs of four warps: 1.04-1.24x at N = 128 x 4096 chains and
+// N = 60 x 16384, 1.005x at N = 32 x 65536).
+constexpr int kChunkThreads = 32;
+// Resident warps per SM the kernels are compiled for.  Two beads per lane fit 96
+// registers; three or more need 128 (N = 40, 65536 chains: 26.4 us per step at 16
+// warps, 28.8 at 20 with the spills of 96 registers).
+constexpr int chunk_warps_per_sm(int B) { return B == 1 ? 24 : (B == 2 ? 20 : 16); }
+
+// Columns of a chain's row in device memory (R, A [3][NP], S, tape [NP]): a
+// property of the chain length alone, so layouts of fewer lanes x beads than
+// that (8 x 1, 8 x 3, 32 x 3) read and write the same arrays.
+__host__ __device__ constexpr int row_stride(int n) {
+    return n <= 64 ? (n + 15) / 16 * 16 : kMaxBeads;
+}
+// Slot sub-slots of a lane: slots above kMaxSlots never hold a spring.
+__host__ __device__ constexpr int slot_sub(int W, int B) { return W * B <= kMaxSlots ? B : kMaxSlots / W; }
 
 // shared memory carve-up (bytes), identical on host and device
 struct SmemPlan {
-    int off_tab, off_pos, off_bq, off_msk, off_log, total;
+    int off_rec, off_pos, off_bq, off_msk, off_red, off_kap, off_log, total;
 };
+
+// Stress samples are reduced in batches of kRedSteps steps (FP32): the six
+// per-lane parts of each step wait in shared memory, and then each lane adds up
+// whole rows (one value of one chain and step), five steps filling 60 of 64, 30
+// of 32 or 120 of 128 row slots of a warp.  (A shuffle reduction of every step,
+// with its selects and its five dependent rounds, took 12 instructions per
+// warp-step more.)
+constexpr int kRedSteps = 5;
+// Rows of W + 4 words, so that eight lanes reading 16 bytes of eight rows each
+// cover every bank once; the chains of a warp lie W words (mod 32) apart, so that
+// the 32 lanes writing one value of each do, too.
+__host__ __device__ constexpr int red_row(int W) { return W + 4; }
+__host__ __device__ constexpr int red_chain(int W) {
+    const int n = kRedSteps * 6 * red_row(W), pad = (W - n % 32 + 32) % 32;
+    return n + (W == 32 ? 0 : pad);
+}
 
 template <typename T>
 __host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_chunk) {
     SmemPlan p;
-    p.off_tab = 0;
-    // per chain NP slot records and one record of zeros that empty gathers read
-    int sz = warps * (32 / W) * (W * B + 1) * (int)sizeof(SlotRec<T>);
+    const int chains = warps * (32 / W), NL = W * B;
+    p.off_rec = 0;
+    // per chain 3 NL spring records: the first spring of each bead, the second, and by slot
+    int sz = chains * 3 * NL * (int)sizeof(SlotRec<T>);
     p.off_pos = (sz + 15) & ~15;
-    sz = p.off_pos + warps * 32 * B * (int)sizeof(Pos<T>);
+    // per chain NL positions between two guard entries
+    sz = p.off_pos + chains * (NL + 2) * (int)sizeof(Pos<T>);
     p.off_bq = (sz + 15) & ~15;
-    // per chain NP + 1 bond vectors: entry i + 1 holds bead i's, entry 0 zeros
-    sz = p.off_bq + warps * (32 / W) * (W * B + 1) * (int)sizeof(Pos<T>);
+    // per chain NL + 1 bond vectors: entry i + 1 holds bead i's, entry 0 zeros
+    sz = p.off_bq + chains * (NL + 1) * (int)sizeof(Pos<T>);
     p.off_msk = (sz + 15) & ~15;
-    sz = p.off_msk + warps * 32 * B * (int)sizeof(unsigned long long);
+    sz = p.off_msk + chains * NL * (int)(NL <= 32 ? sizeof(unsigned) : sizeof(unsigned long long));
+    p.off_red = (sz + 15) & ~15;
+    sz = p.off_red + (sizeof(T) == 4 ? chains * red_chain(W) * (int)sizeof(T) : 0);
+    p.off_kap = (sz + 15) & ~15;
+    sz = p.off_kap + warps * 3 * (int)sizeof(Pos<T>);
     p.off_log = (sz + 15) & ~15;
     sz = p.off_log + nlog_chunk * 14 * (int)sizeof(double);
     p.total = (sz + 15) & ~15;
@@ -345,7 +383,7 @@ __device__ __forceinline__ int seg6_value(int ll) {
     return ((ll & (W / 2)) ? 3 : 0) + comp;
 }
 template <typename T, int W>
-__device__ __forceinline__ T seg_reduce6(const T (&v)[8], int ll) {
+__device__ __forceinline__ T seg_reduce6(const T (&v)[6], int ll) {
     T w[3];
     {
         const bool hi = (ll & (W / 2)) != 0;
@@ -387,25 +425,12 @@ __device__ __forceinline__ T hop_prob(const StepConst<T>& c, T d_new, T d_old) {
     return w < T(0.5) ? w : T(0.5);
 }
 
-// FP32 form of the same probability: e^{2y} = 2^t with t = c2 (d_new - d_old)
-// (c2 = 2 chop log2 e) by ex2.approx, 2/(1+e^{2y}) by rcp.approx.  t is capped
-// at 80 log2 e (y <= 40), where the probability is still a normal float; below
-// y = -40 the expression already equals its limit 2 pref.
-template <typename T>
-__device__ __forceinline__ T hop_prob_fast(const StepConst<T>& c, T d_new, T d_old) {
-    return hop_prob<T>(c, d_new, d_old);
-}
-template <>
-__device__ __forceinline__ float hop_prob_fast<float>(const StepConst<float>& c, float d_new, float d_old) {
-    const float t = fminf(c.c2 * (d_new - d_old), 115.41560327111707f);
-    float e, r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-    return fminf(c.two_pref * r, 0.5f);
-}
-// The same for two moves from one slot (new squared lengths dnew.x, dnew.y),
-// with the additions and multiplications packed; each half is rounded as in
-// hop_prob_fast<float>.
+// FP32 form of the same probability for the two moves from one slot (new squared
+// lengths dnew.x, dnew.y): e^{2y} = 2^t with t = c2 (d_new - d_old) (c2 = 2 chop
+// log2 e) by ex2.approx, 2/(1+e^{2y}) by rcp.approx, the additions and
+// multiplications packed.  t is capped at 80 log2 e (y <= 40), where the
+// probability is still a normal float; below y = -40 the expression already
+// equals its limit 2 pref.
 __device__ __forceinline__ float2 hop_prob_x2(const StepConst<float>& c, float2 dnew, float d_old) {
     const float2 t = __fmul2_rn(pk(c.c2), __fadd2_rn(dnew, pk(-d_old)));
     float ea, eb, ra, rb;
@@ -420,12 +445,20 @@ __device__ __forceinline__ float2 hop_prob_x2(const StepConst<float>& c, float2 
 
 // ---------------------------------------------------------- chunk kernel ----
 // W lanes per chain, B beads per lane: bead i and slot i of a chain live on
-// lane i % W as its sub-slot i / W (NP = W*B >= N beads and slots).
+// lane i % W as its sub-slot i / W (NL = W*B >= N beads; slots only up to
+// kMaxSlots, SB sub-slots of a lane).  NP is the row stride in device memory.
+//
+// The spring forces of a step read, per bead, the vectors of up to two springs
+// from two tables that the slot lanes keep up to date (rec).  A third spring on
+// one bead is rare and handled in a branch.  (A gather by bit scans of the
+// masks spends 24 instructions on every bead, most of which carry no spring.)
+constexpr int kWinOff = 0, kWinRecord = 1, kWinReplay = 2;  // differentiation-window hooks
+
 // State of one chain before a step, for the recompute of a differentiation window.
-template <typename T, int W, int B>
-__device__ __forceinline__ void snapshot_store(const ChunkArgs& a, long long row, int mm, int ll, const T (&R)[B][3],
-                                               const T (&A)[B][3], const int (&S)[B], int Z) {
-    constexpr int NP = W * B;
+template <typename T, int W, int B, int SB, typename Args>
+__device__ __forceinline__ void snapshot_store(const Args& a, long long row, int mm, int ll, const T (&R)[B][3],
+                                               const T (&A)[SB][3], const int (&S)[SB], int Z) {
+    constexpr int NP = row_stride(W * B);
     T* sR = static_cast<T*>(a.snapR) + ((size_t)row * a.M + mm) * 3 * NP;
     T* sA = static_cast<T*>(a.snapA) + ((size_t)row * a.M + mm) * 3 * NP;
     int32_t* sS = a.snapS + ((size_t)row * a.M + mm) * NP;
@@ -435,27 +468,67 @@ __device__ __forceinline__ void snapshot_store(const ChunkArgs& a, long long row
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             sR[d * NP + i] = R[b][d];
-            sA[d * NP + i] = i < Z ? A[b][d] : T(0);
+            sA[d * NP + i] = b < SB && i < Z ? A[b < SB ? b : 0][d] : T(0);
         }
-        sS[i] = i < Z ? S[b] : -1;
+        sS[i] = b < SB && i < Z ? S[b < SB ? b : 0] : -1;
     }
     if (ll == 0) a.snapZ[(size_t)row * a.M + mm] = Z;
 }
 
+constexpr int kNever = 0x7fffffff;
+// absolute step as an offset from t0 (kNever: beyond any launch)
+__device__ __forceinline__ int rel_step(long long t_abs, long long t0) {
+    const long long r = t_abs - t0;
+    return r > (long long)kNever ? kNever : (int)r;
+}
+
+// Place in the velocity-gradient schedule: entry, offset of the next entry in
+// this launch, whether the entry is non-zero.
+struct KappaState {
+    int ki, next_from;
+    bool nz;
+};
+// The entry of the schedule for step t0 + s (from entry ki on), its matrix in
+// the rows kap.  All lanes of the warp call this together.  The loads are __ldg:
+// through pointers that come from memory, plain ones might read shared memory for
+// all the compiler knows, and cost the batched kernel 27 us per step instead of 18
+// (N = 32, 65536 chains).
+template <typename T, typename Args>
+__device__ __forceinline__ KappaState kappa_at(Args& a, int ki, long long t0, int s, Pos<T>* kap) {
+    const int lane = threadIdx.x & 31;
+    const int n = a.n_kap;
+    const double* const k = a.kap;
+    const long long* const from = a.kap_from;
+    while (ki + 1 < n && t0 + s >= __ldg(from + ki + 1)) ++ki;
+    const T v = lane < 9 ? T(__ldg(k + ki * 9 + lane)) : T(0);
+    if (lane < 9) reinterpret_cast<T*>(kap + lane / 3)[lane % 3] = v;
+    KappaState r;
+    r.ki = ki;
+    r.next_from = ki + 1 < n ? rel_step(__ldg(from + ki + 1), t0) : kNever;
+    r.nz = __any_sync(kFull, v != T(0));
+    __syncwarp();
+    return r;
+}
 // The chains of one CTA: chains cta_first .. cta_first + chains per CTA - 1 of
 // the element described by `a` (all warps of the CTA call this together).
 // FLOW: the velocity-gradient terms are compiled in (without them the launch
-// must have kappa = 0 throughout; recentring is then never needed).
-template <typename T, int W, int B, bool WIN, bool FLOW, bool HEUN = false>
-__device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T>& c, const int cta_first,
+// must have kappa = 0 throughout; recentring is then never needed).  CORR: the
+// stress series is compiled in.  VL = 2: eight lanes do the work of sixteen.
+// Sub-slots of even and of odd b are the beads of lanes l and l + 8 of a 16-lane
+// segment; summing them apart and adding the two is the first round of that
+// segment's reduction, so every sum over beads is rounded as there.
+template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, int VL, typename Args>
+__device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const int cta_first,
                                            const T NkT, const long long t0_, const int nsteps_,
                                            const long long log_m0_, const int nlog_) {
     constexpr int SEGS = 32 / W;
-    constexpr int NP = W * B;
-    constexpr int G8 = W / 8;        // lanes per value group after seg_reduce6
-    constexpr bool PK = std::is_same<T, float>::value && (B % 2) == 0;  // packed FP32x2 bead pairs
-    // per-bead slot masks: 32 bits cover every slot when NP <= 32
-    using Mask = typename std::conditional<(NP <= 32), unsigned, unsigned long long>::type;
+    constexpr int NL = W * B;               // beads of a chain's lanes
+    constexpr int NP = row_stride(NL);      // columns of a chain's rows in device memory
+    constexpr int SB = slot_sub(W, B);      // slot sub-slots
+    constexpr int G8 = W / 8;               // lanes per value group after seg_reduce6
+    constexpr int BP = std::is_same<T, float>::value ? B / 2 * 2 : 0;  // beads in packed FP32x2 pairs
+    // per-bead slot masks: 32 bits cover every slot when NL <= 32
+    using Mask = typename std::conditional<(NL <= 32), unsigned, unsigned long long>::type;
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nwarps = blockDim.x >> 5;
@@ -467,133 +540,240 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
     const int mm = live ? m : 0;
     const uint32_t chain_id = a.chain_base + (uint32_t)mm;
     const int N = a.N;
-    const int tmode = WIN ? a.tape_mode : 0;  // differentiation windows only
     const unsigned segmask = (W == 32) ? kFull : (((1u << W) - 1u) << (seg * W));
     const unsigned lt = ((1u << lane) - 1u) & segmask;  // lanes of this segment below this one
 
     extern __shared__ __align__(16) unsigned char smem[];
     const SmemPlan plan = smem_plan<T>(nwarps, W, B, nlog_);
-    SlotRec<T>* tab = reinterpret_cast<SlotRec<T>*>(smem + plan.off_tab) + (warp * SEGS + seg) * (NP + 1);
-    Pos<T>* pos = reinterpret_cast<Pos<T>*>(smem + plan.off_pos) + (warp * SEGS + seg) * NP;
+    // spring records of this chain: [0, NL) the first spring of each bead, [NL, 2 NL)
+    // the second (zeros where there is none), [2 NL, 3 NL) by slot: springs beyond
+    // the second of a bead, and scratch of the re-indexing
+    SlotRec<T>* rec = reinterpret_cast<SlotRec<T>*>(smem + plan.off_rec) + cslot * 3 * NL;
+    SlotRec<T>* tab = rec + 2 * NL;
+    // positions, with a guard entry on either side (read for a hop beyond an end,
+    // whose probability is then replaced by 0)
+    Pos<T>* pos = reinterpret_cast<Pos<T>*>(smem + plan.off_pos) + cslot * (NL + 2) + 1;
     // bond vectors Q_i = R_{i+1} - R_i of the current state, one entry up:
     // bq[i + 1] = Q_i, bq[0] = 0 (bead 0 has no left bond)
-    Pos<T>* bq = reinterpret_cast<Pos<T>*>(smem + plan.off_bq) + (warp * SEGS + seg) * (NP + 1);
-    Mask* msk = reinterpret_cast<Mask*>(smem + plan.off_msk) + (warp * SEGS + seg) * NP;
+    Pos<T>* bq = reinterpret_cast<Pos<T>*>(smem + plan.off_bq) + cslot * (NL + 1);
+    Mask* msk = reinterpret_cast<Mask*>(smem + plan.off_msk) + cslot * NL;
+    [[maybe_unused]] T* const red = reinterpret_cast<T*>(smem + plan.off_red) + warp * SEGS * red_chain(W);
     double* slog = reinterpret_cast<double*>(smem + plan.off_log);
 
     for (int i = threadIdx.x; i < nlog_ * 14; i += blockDim.x) slog[i] = 0.0;
 
+    // ---- flow schedule, as step offsets in this launch
+    const int never = kNever;
+    // The velocity gradient waits in shared memory, row by row (three 16-byte
+    // broadcast loads a step): nine registers for the whole launch would spill.
+    KappaState ks{0, never, false};
+    [[maybe_unused]] Pos<T>* const kap = reinterpret_cast<Pos<T>*>(smem + plan.off_kap) + warp * 3;
+    auto kx = [&](int d) { return kap[d].x; };
+    auto ky = [&](int d) { return kap[d].y; };
+    auto kz = [&](int d) { return kap[d].z; };
+    auto load_kappa = [&](int s) {
+        ks = kappa_at<T>(a, ks.ki, t0_, s, kap);
+    };
+    if constexpr (FLOW) load_kappa(0);
+
     // ---- load state
     const T* Rg = static_cast<const T*>(a.R);
     const T* Ag = static_cast<const T*>(a.A);
-    T R[B][3], A[B][3];
-    int S[B];
+    T R[B][3], A[SB][3];
+    int S[SB];
     int Z = live ? a.Z[mm] : 0;
+    SlotRec<T> zrec;
+    zrec.x = zrec.y = zrec.z = T(0);
+    zrec.s = 0;
+    Pos<T> zpos;
+    zpos.x = zpos.y = zpos.z = zpos.w = T(0);
+    auto store_pos = [&](const T (&X)[B][3]) {
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
+        for (int b = 0; b < B; ++b) {
+            Pos<T> p;
+            p.x = X[b][0];
+            p.y = X[b][1];
+            p.z = X[b][2];
+            p.w = T(0);
+            pos[ll + b * W] = p;
+        }
+    };
+#pragma unroll
+    for (int b = 0; b < SB; ++b) {
         const int i = ll + b * W;
         S[b] = (live && i < Z) ? a.S[(size_t)mm * NP + i] : 0;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            R[b][d] = (live && i < N) ? Rg[((size_t)mm * 3 + d) * NP + i] : T(0);
-            A[b][d] = (live && i < Z) ? Ag[((size_t)mm * 3 + d) * NP + i] : T(0);
-        }
-        Pos<T> p0;
-        p0.x = R[b][0];
-        p0.y = R[b][1];
-        p0.z = R[b][2];
-        p0.w = T(0);
-        pos[i] = p0;
+        for (int d = 0; d < 3; ++d) A[b][d] = (live && i < Z) ? Ag[((size_t)mm * 3 + d) * NP + i] : T(0);
+    }
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+        const int i = ll + b * W;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) R[b][d] = (live && i < N) ? Rg[((size_t)mm * 3 + d) * NP + i] : T(0);
+        rec[i] = zrec;
+        rec[NL + i] = zrec;
+        msk[i] = Mask(0);
+    }
+    store_pos(R);
+    if (ll == 0) {
+        pos[-1] = zpos;
+        pos[NL] = zpos;
+        bq[0] = zpos;
     }
 
-    // Values that change only with Z, kept from one change to the next: the
-    // creation attempts of substep 3a (slots first = Z .. c_last - 1, each
-    // creating with probability p_c(K = c_last - Z) at either end; c_drop: an
-    // attempt dropped at the cap, counted on lane 0) and the largest Z of this
-    // warp's chains (sub-slots at or above it hold no spring).
-    int c_last = Z;
-    T c_pc2 = T(0);  // 2 p_c
+    // Values that change only with Z, kept from one change to the next: per
+    // sub-slot the bound on u below which it creates a spring (2 p_c on the
+    // creation attempts of substep 3a, slots Z .. c_last - 1; 0 elsewhere) and the
+    // bound on n3 below which a spring at an end is destroyed (cd on occupied
+    // slots, -inf elsewhere) and its stiffness in the stress (0 on empty slots); an
+    // attempt dropped at the cap, counted on lane 0; and
+    // the largest Z of this warp's chains (sub-slots at or above it hold no spring).
+    T thr_c[SB];
     int z_w = 0;
     bool c_drop = false;
+    auto attempts_end = [&]() { return Z < a.zmax ? ((a.create_mode == 0) ? a.zmax : Z + 1) : Z; };
     auto set_create = [&]() {
         c_drop = Z >= a.zmax && a.create_mode == 1 && ll == 0 && live;
         z_w = (int)__reduce_max_sync(kFull, (unsigned)Z);
-        c_last = Z < a.zmax ? ((a.create_mode == 0) ? a.zmax : Z + 1) : Z;
-        c_pc2 = T(2) * c.pc[c_last - Z];
+        const int c_last = attempts_end();
+        const T pc2 = T(2) * c.pc[c_last - Z];
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            const int i = ll + b * W;
+            thr_c[b] = (i >= Z && i < c_last) ? pc2 : T(0);
+        }
     };
     set_create();
 
     // stress series of this launch (the correlator reads it afterwards)
     T* const ser = static_cast<T*>(a.series);
-    const bool corr_on = ser != nullptr;
+    const bool corr_on = CORR && ser != nullptr;
     const int gq = seg6_value<W>(ll);  // value this lane holds after seg_reduce6
     // one writer per value: the lowest lane of its group (yz is held twice over)
-    T* const ser_m = (corr_on && live && (ll % G8) == 0 && !((gq % 3) == 2 && (ll & (W / 4))))
+    [[maybe_unused]] T* const ser_m = (corr_on && live && (ll % G8) == 0 && !((gq % 3) == 2 && (ll & (W / 4))))
                          ? ser + ((size_t)a.series_row0 * a.M + mm) * 6 + gq
                          : nullptr;
     const size_t ser_step = (size_t)a.M * 6;
+    // Batched reduction (FP32): value q of step n of a batch is row 6 n + q of its
+    // chain, W lane parts summed in pairs as the butterflies of seg_reduce6 pair
+    // the lanes.
+    [[maybe_unused]] int red_n = 0;  // steps waiting
+    [[maybe_unused]] T* red_w = red + seg * red_chain(W) + ll;
+    [[maybe_unused]] auto red_put = [&](const T (&v)[6]) {
+#pragma unroll
+        for (int q = 0; q < 6; ++q) red_w[q * red_row(W)] = v[q];
+        red_w += 6 * red_row(W);
+    };
+    [[maybe_unused]] auto red_flush = [&](int s_end) {
+        const int rows = 6 * red_n;  // of each chain
+        for (int r = lane; r < rows * SEGS; r += 32) {
+            const int ch = SEGS == 1 ? 0 : r / rows, rr = r - ch * rows;
+            const float4* row = reinterpret_cast<const float4*>(red + ch * red_chain(W) + rr * red_row(W));
+            float4 x[W / 4];
+#pragma unroll
+            for (int k = 0; k < W / 4; ++k) x[k] = row[k];
+#pragma unroll
+            for (int h = W / 8; h > 0; h >>= 1) {
+#pragma unroll
+                for (int k = 0; k < h; ++k) {
+                    x[k].x += x[k + h].x;
+                    x[k].y += x[k + h].y;
+                    x[k].z += x[k + h].z;
+                    x[k].w += x[k + h].w;
+                }
+            }
+            const float sum = (x[0].x + x[0].z) + (x[0].y + x[0].w);
+            const int st = rr / 6, q = rr - 6 * st, m = cta_first + warp * SEGS + ch;
+            if (m < a.M) ser[((size_t)(a.series_row0 + s_end - red_n + st) * a.M + m) * 6 + q] = sum;
+        }
+        red_n = 0;
+        red_w = red + seg * red_chain(W) + ll;
+    };
     if (nlog_ > 0)
         __syncthreads();  // the CTA's stress-log buffer is zeroed
     else
         __syncwarp();
 
-    // ---- flow schedule and periodic events, as step offsets in this launch
-    const int never = 0x7fffffff;
-    auto rel = [&](long long t_abs) -> int {
-        const long long r = t_abs - t0_;
-        return r > (long long)never ? never : (int)r;
-    };
-    int ki = 0;
-    T kap[9];
-    bool kap_nz = false;
-    int next_from = never;
-    if constexpr (FLOW) {
-        while (ki + 1 < a.n_kap && t0_ >= a.kap_from[ki + 1]) ++ki;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            kap[i] = T(a.kap[ki * 9 + i]);
-            kap_nz |= (kap[i] != T(0));
-        }
-        next_from = (ki + 1 < a.n_kap) ? rel(a.kap_from[ki + 1]) : never;
-    }
-    int next_log = a.log_every > 0 ? rel((t0_ / a.log_every + 1) * a.log_every - 1) : never;
-    int next_rc = a.recenter_every > 0 ? rel((t0_ / a.recenter_every + 1) * a.recenter_every - 1) : never;
+    // ---- periodic events, as step offsets in this launch
+    int next_log = a.log_every > 0 ? rel_step((t0_ / a.log_every + 1) * a.log_every - 1, t0_) : never;
+    int next_rc = a.recenter_every > 0 ? rel_step((t0_ / a.recenter_every + 1) * a.recenter_every - 1, t0_) : never;
     int log_slot = 0;
     const uint32_t t0lo = (uint32_t)t0_;
 
     unsigned cnt_up = 0, cnt_dn = 0, cnt_cr = 0, cnt_de = 0, cnt_drop = 0;
 
-    // slot table: the spring vector d_j = R_{S_j} - A_j of every occupied slot
-    // j, written at the end of each step for the next step's spring forces; a
-    // recentring step rewrites it from the shifted coordinates, as a launch
-    // computes it here at its start.  The re-indexing below also uses the
-    // table as scratch.  Record NP is zero: an empty slot mask reads it.
-    __syncwarp();  // positions of this warp's chains are in the table
+    __syncwarp();  // positions, zeroed records and masks of this warp's chains are in place
+
+    // Spring vectors d_j = R_{S_j} - A_j into the tables the forces of the next
+    // step read: the first slot to enter its bit in the bead's mask takes the
+    // bead's first record, the next one the second (their sum is the same either
+    // way), any other its own slot's record; the record names its slot, so that a
+    // bead of three or more can add them in slot order.  The masks and the records
+    // of beads 0 .. NL - 1 are zero before: each slot clears what it wrote before
+    // it moves.  loc: this slot's record; more3: some bead of the warp has three.
+    // The slots of an idle lane (no spring) do the same work without a branch: a
+    // stale S is a valid bead, and their record is their own slot's, which nothing
+    // reads.  Sub-slots at or above every Z of the warp are skipped (the first
+    // never is).
+    int loc[SB];
+    bool more3 = false;
+    auto skip = [&](int b, int z) { return b > 0 && b * W >= z; };
+    auto register_springs = [&](const T (&d)[SB][3]) {
+        bool third = false;
 #pragma unroll
-    for (int b = 0; b < B; ++b) {
-        const int i = ll + b * W;
-        if (i < Z) {
-            const Pos<T> ps = pos[S[b]];
-            SlotRec<T> rec;
-            rec.x = ps.x - A[b][0];
-            rec.y = ps.y - A[b][1];
-            rec.z = ps.z - A[b][2];
-            rec.s = S[b];
-            tab[i] = rec;
+        for (int b = 0; b < SB; ++b) {
+            const int i = ll + b * W;
+            if (!skip(b, z_w)) {
+                const bool occ = i < Z;
+                Mask old = ~Mask(0);
+                if (occ) old = atomicOr(&msk[S[b]], Mask(1) << i);
+                const bool late = (old & (old - Mask(1))) != Mask(0);  // two or more before it, or no spring
+                third |= occ && late;
+                int l = old != Mask(0) ? NL + S[b] : S[b];
+                l = late ? 2 * NL + i : l;
+                loc[b] = l;
+                SlotRec<T> r;
+                r.x = d[b][0];
+                r.y = d[b][1];
+                r.z = d[b][2];
+                r.s = i;
+                rec[l] = r;
+            }
         }
+        more3 = __any_sync(kFull, third);
+    };
+    auto spring_vectors = [&](T (&d)[SB][3]) {
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            if (!skip(b, z_w)) {
+                const Pos<T> ps = pos[S[b]];
+                d[b][0] = ps.x - A[b][0];
+                d[b][1] = ps.y - A[b][1];
+                d[b][2] = ps.z - A[b][2];
+            }
+        }
+    };
+    // the vectors again, from shifted or predicted coordinates, in the same records
+    auto rewrite_springs = [&]() {
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            if (!skip(b, z_w)) {
+                const Pos<T> ps = pos[S[b]];
+                SlotRec<T>& r = rec[loc[b]];
+                r.x = ps.x - A[b][0];
+                r.y = ps.y - A[b][1];
+                r.z = ps.z - A[b][2];
+            }
+        }
+    };
+    {
+        T d[SB][3];
+        spring_vectors(d);
+        register_springs(d);
     }
     PhiloxPre ppre[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) ppre[b] = philox_pre((uint32_t)(ll + b * W), kPurposeStep, chain_id, c.rk0, c.rk1);
-    if (ll == 0) {
-        SlotRec<T> zero;
-        zero.x = zero.y = zero.z = T(0);
-        zero.s = -1;
-        tab[NP] = zero;
-        Pos<T> z4;
-        z4.x = z4.y = z4.z = z4.w = T(0);
-        bq[0] = z4;
-    }
     // Bond vectors of the current positions (the position table holds them):
     // the stress of a step and the bond forces of the next step both use
     // them.  The last bead and padding beads read themselves: Q = 0.
@@ -621,71 +801,65 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
     // at its end, where their integer work interleaves with the stress.
     auto draw = [&](const uint32_t tt, T (&nrm)[B][4], T (&u)[B]) {
         const unsigned long long p_shared = philox_step_shared(tt, kPurposeStep, c.rk0);
-        if constexpr (PK) {
 #pragma unroll
-            for (int b = 0; b < B; b += 2) {
-                const uint4 w0 = philox_step(ppre[b], p_shared, c.rk0, c.rk1);
-                const uint4 w1 = philox_step(ppre[b + 1], p_shared, c.rk0, c.rk1);
+        for (int b = 0; b < BP; b += 2) {
+            const uint4 w0 = philox_step(ppre[b], p_shared, c.rk0, c.rk1);
+            const uint4 w1 = philox_step(ppre[b + 1], p_shared, c.rk0, c.rk1);
+            if constexpr (std::is_same<T, float>::value) {
                 box_muller_x2(w0.x, w0.y, w1.x, w1.y, nrm[b][0], nrm[b][1], nrm[b + 1][0], nrm[b + 1][1]);
                 box_muller_x2(w0.z, w0.w, w1.z, w1.w, nrm[b][2], nrm[b][3], nrm[b + 1][2], nrm[b + 1][3]);
                 const float2 uu = __fmul2_rn(pk(float(lo24_bits(w0)), float(lo24_bits(w1))), pk(1.0f / 16777216.0f));
                 u[b] = uu.x;
                 u[b + 1] = uu.y;
             }
-        } else if constexpr (std::is_same<T, float>::value) {
+        }
 #pragma unroll
-            for (int b = 0; b < B; ++b) {  // the bead's two Box-Muller pairs packed
-                const uint4 w = philox_step(ppre[b], p_shared, c.rk0, c.rk1);
+        for (int b = BP; b < B; ++b) {
+            const uint4 w = philox_step(ppre[b], p_shared, c.rk0, c.rk1);
+            if constexpr (std::is_same<T, float>::value) {  // the bead's two Box-Muller pairs packed
                 box_muller_x2(w.x, w.y, w.z, w.w, nrm[b][0], nrm[b][1], nrm[b][2], nrm[b][3]);
-                u[b] = uniform_lo24<T>(w);
-            }
-        } else {
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const uint4 w = philox_step(ppre[b], p_shared, c.rk0, c.rk1);
+            } else {
                 box_muller<T>(w.x, w.y, nrm[b][0], nrm[b][1]);
                 box_muller<T>(w.z, w.w, nrm[b][2], nrm[b][3]);
-                u[b] = uniform_lo24<T>(w);
             }
+            u[b] = uniform_lo24<T>(w);
         }
     };
-    T nrm[B][4], u[B];
-    draw(t0lo, nrm, u);
-    for (int s = 0; s < nsteps_; ++s) {
+    // decisions of a replayed step, loaded one step ahead
+    auto tape_at = [&](int s, int b) -> uint8_t {
+        const long long row = (long long)t0_ + s - a.tape_t0;
+        return (live && s < nsteps_ && row >= 0 && row < a.tape_rows)
+                   ? a.tape[((size_t)row * a.M + mm) * NP + ll + b * W]
+                   : (uint8_t)0;
+    };
+    [[maybe_unused]] uint8_t tape_next[SB];
+    if constexpr (WIN == kWinReplay) {
+#pragma unroll
+        for (int b = 0; b < SB; ++b) tape_next[b] = tape_at(0, b);
+    }
+    int s = 0;
+    for (;;) {  // stretches of one velocity gradient
+    const int s_end = FLOW ? min(nsteps_, ks.next_from) : nsteps_;
+    for (; s < s_end; ++s) {
         const uint32_t t = t0lo + (uint32_t)s;
-        if (FLOW && s >= next_from) {
-            while (ki + 1 < a.n_kap && t0_ + s >= a.kap_from[ki + 1]) ++ki;
-            kap_nz = false;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) {
-                kap[i] = T(a.kap[ki * 9 + i]);
-                kap_nz |= (kap[i] != T(0));
-            }
-            next_from = (ki + 1 < a.n_kap) ? rel(a.kap_from[ki + 1]) : never;
-        }
-        if (WIN && a.snapR != nullptr && live) {
+        if (WIN == kWinReplay && a.snapR != nullptr && live) {
             const long long sr = (long long)t0_ + s - a.snap_t0;
-            if (sr >= 0 && sr <= a.snap_steps) snapshot_store<T, W, B>(a, sr, mm, ll, R, A, S, Z);
+            if (sr >= 0 && sr <= a.snap_steps) snapshot_store<T, W, B, SB>(a, sr, mm, ll, R, A, S, Z);
         }
-        const long long trow = (long long)t0_ + s - a.tape_t0;
-        const bool tape_row = WIN && tmode != 0 && live && trow >= 0 && trow < a.tape_rows;
-        uint8_t tb[B];
+        [[maybe_unused]] uint8_t tb[SB];
+        if constexpr (WIN != kWinOff) {
 #pragma unroll
-        for (int b = 0; b < B; ++b)
-            tb[b] = (tmode == 2 && tape_row) ? a.tape[((size_t)trow * a.M + mm) * NP + ll + b * W] : (uint8_t)0;
-        // ---- per-bead slot masks for this step's spring forces
-#pragma unroll
-        for (int b = 0; b < B; ++b) msk[ll + b * W] = Mask(0);
-        __syncwarp();
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-            if (i < Z) atomicOr(&msk[S[b]], Mask(1) << i);
+            for (int b = 0; b < SB; ++b) {
+                tb[b] = WIN == kWinReplay ? tape_next[b] : (uint8_t)0;
+                if (WIN == kWinReplay) tape_next[b] = tape_at(s + 1, b);
+            }
         }
 
+        T nrm[B][4], u[B];
+        draw(t, nrm, u);
         // ---- substep 1: forces at time t, Euler-Maruyama, anchor advection.
         // Forces on positions Ro (this lane's beads; the other beads from the
-        // position table) with the spring vectors of the slot table: bonds
+        // position table) with the spring vectors of the tables: bonds
         // k_b (R_{i-1} + R_{i+1} - 2 R_i), springs -k_s sum_{j: S_j = i} d_j.
         // With bonds_from_q the bond forces come from the bond vectors of the
         // state (this lane's Q and the left neighbour's from the table):
@@ -711,43 +885,46 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
                     for (int d = 0; d < 3; ++d) Fo[b][d] = c.k_b * (Rl[d] - Ro[b][d]) + c.k_b * (Rr[d] - Ro[b][d]);
                 }
             }
-            __syncwarp();
-            bool more = false;
-            Mask mrest[B];
+            // springs on this bead: -k_s sum_j d_j, slots in ascending order
+            // (zero records where there is none)
+            T sp[B][3];
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                // springs on this bead: -k_s sum_j d_j, slots in ascending order
-                // (an empty mask reads the zero record at NP)
-                const Mask m0 = msk[ll + b * W];
-                const Mask m1 = m0 & (m0 - Mask(1));
-                const int j0 = m0 ? mask_ffs(m0) - 1 : NP;
-                const int j1 = m1 ? mask_ffs(m1) - 1 : NP;
-                const SlotRec<T> r0 = tab[j0], r1 = tab[j1];
-                const Mask mb = m1 & (m1 - Mask(1));
-                mrest[b] = mb;
-                more |= mb != Mask(0);
-                Fo[b][0] -= c.k_s * (r0.x + r1.x);
-                Fo[b][1] -= c.k_s * (r0.y + r1.y);
-                Fo[b][2] -= c.k_s * (r0.z + r1.z);
+                const SlotRec<T> r0 = rec[ll + b * W], r1 = rec[NL + ll + b * W];
+                sp[b][0] = r0.x + r1.x;
+                sp[b][1] = r0.y + r1.y;
+                sp[b][2] = r0.z + r1.z;
             }
-            if (__any_sync(kFull, more)) {  // a third spring on one bead: rare
+            if (more3) {  // a third spring on one bead of the warp: rare
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
-                    // the first two slots were added already; add the rest in order
-                    Mask mb = mrest[b];
-                    T sx = T(0), sy = T(0), sz = T(0);
-                    while (mb) {
-                        const SlotRec<T> r = tab[mask_ffs(mb) - 1];
-                        mb &= mb - Mask(1);
-                        sx += r.x;
-                        sy += r.y;
-                        sz += r.z;
+                    Mask mb = msk[ll + b * W];
+                    if (mask_popc(mb) > 2) {
+                        // the springs of the mask in slot order: the first two, then the rest
+                        const int j0 = rec[ll + b * W].s, j1 = rec[NL + ll + b * W].s;
+                        auto take = [&]() {
+                            const int j = mask_ffs(mb) - 1;
+                            mb &= mb - Mask(1);
+                            return rec[j == j0 ? ll + b * W : (j == j1 ? NL + ll + b * W : 2 * NL + j)];
+                        };
+                        const SlotRec<T> q0 = take(), q1 = take();
+                        Fo[b][0] -= c.k_s * (q0.x + q1.x);
+                        Fo[b][1] -= c.k_s * (q0.y + q1.y);
+                        Fo[b][2] -= c.k_s * (q0.z + q1.z);
+                        sp[b][0] = sp[b][1] = sp[b][2] = T(0);
+                        while (mb) {
+                            const SlotRec<T> q = take();
+                            sp[b][0] += q.x;
+                            sp[b][1] += q.y;
+                            sp[b][2] += q.z;
+                        }
                     }
-                    Fo[b][0] -= c.k_s * sx;
-                    Fo[b][1] -= c.k_s * sy;
-                    Fo[b][2] -= c.k_s * sz;
                 }
             }
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) Fo[b][d] -= c.k_s * sp[b][d];
         };
         T F[B][3];
         forces(F, R, true);
@@ -755,71 +932,84 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
         // vectors are zero, they exert no force, carry no spring, enter no
         // stress and are never stored.
         T Rn[B][3];
-        [[maybe_unused]] T A0[B][3];
+        [[maybe_unused]] T A0[SB][3];
         if constexpr (HEUN) {
 #pragma unroll
-            for (int b = 0; b < B; ++b)
+            for (int b = 0; b < SB; ++b)
 #pragma unroll
                 for (int d = 0; d < 3; ++d) A0[b][d] = A[b][d];
         }
 #pragma unroll
         for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-            if (kap_nz) {
-                if constexpr (PK) {
-                    // beads b and b + 1 together; the same operations as the FP32 form below
-                    if ((b & 1) == 0) {
-                        const float2 r0 = pk(R[b][0], R[b + 1][0]), r1 = pk(R[b][1], R[b + 1][1]),
-                                     r2 = pk(R[b][2], R[b + 1][2]);
+            if (ks.nz) {
+                if constexpr (std::is_same<T, float>::value) {
+                    if (b < BP) {
+                        // beads b and b + 1 together; the same operations as the scalar form below
+                        if ((b & 1) == 0) {
+                            const int b1 = b + 1 < B ? b + 1 : b;
+                            const float2 r0 = pk(R[b][0], R[b1][0]), r1 = pk(R[b][1], R[b1][1]),
+                                         r2 = pk(R[b][2], R[b1][2]);
+#pragma unroll
+                            for (int d = 0; d < 3; ++d) {
+                                const float2 flow = __ffma2_rn(pk(kz(d)), r2,
+                                                               __ffma2_rn(pk(ky(d)), r1,
+                                                                          __fmul2_rn(pk(kx(d)), r0)));
+                                const float2 e = __ffma2_rn(
+                                    pk(c.amp), pk(nrm[b][d], nrm[b1][d]),
+                                    __ffma2_rn(pk(c.dt), flow,
+                                               __ffma2_rn(pk(c.mob), pk(F[b][d], F[b1][d]), pk(R[b][d], R[b1][d]))));
+                                Rn[b][d] = e.x;
+                                Rn[b1][d] = e.y;
+                            }
+                        }
+                    } else {
 #pragma unroll
                         for (int d = 0; d < 3; ++d) {
-                            const float2 flow = __ffma2_rn(pk(kap[3 * d + 2]), r2,
-                                                           __ffma2_rn(pk(kap[3 * d + 1]), r1,
-                                                                      __fmul2_rn(pk(kap[3 * d]), r0)));
-                            const float2 e = __ffma2_rn(
-                                pk(c.amp), pk(nrm[b][d], nrm[b + 1][d]),
-                                __ffma2_rn(pk(c.dt), flow,
-                                           __ffma2_rn(pk(c.mob), pk(F[b][d], F[b + 1][d]), pk(R[b][d], R[b + 1][d]))));
-                            Rn[b][d] = e.x;
-                            Rn[b + 1][d] = e.y;
+                            const float flow = __fmaf_rn(
+                                kz(d), R[b][2],
+                                __fmaf_rn(ky(d), R[b][1], __fmul_rn(kx(d), R[b][0])));
+                            Rn[b][d] =
+                                __fmaf_rn(c.amp, nrm[b][d], __fmaf_rn(c.dt, flow, __fmaf_rn(c.mob, F[b][d], R[b][d])));
                         }
-                    }
-                } else if constexpr (std::is_same<T, float>::value) {
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const float flow = __fmaf_rn(kap[3 * d + 2], R[b][2],
-                                                     __fmaf_rn(kap[3 * d + 1], R[b][1], __fmul_rn(kap[3 * d], R[b][0])));
-                        Rn[b][d] = __fmaf_rn(c.amp, nrm[b][d], __fmaf_rn(c.dt, flow, __fmaf_rn(c.mob, F[b][d], R[b][d])));
                     }
                 } else {
 #pragma unroll
                     for (int d = 0; d < 3; ++d) {
-                        const T flow = kap[3 * d] * R[b][0] + kap[3 * d + 1] * R[b][1] + kap[3 * d + 2] * R[b][2];
+                        const T flow = kx(d) * R[b][0] + ky(d) * R[b][1] + kz(d) * R[b][2];
                         Rn[b][d] = R[b][d] + c.mob * F[b][d] + c.dt * flow + c.amp * nrm[b][d];
                     }
                 }
-            } else if constexpr (PK) {
-                if ((b & 1) == 0) {  // beads b and b + 1 together
+            } else if (b < BP) {
+                if constexpr (std::is_same<T, float>::value) {
+                    if ((b & 1) == 0) {  // beads b and b + 1 together
+                        const int b1 = b + 1 < B ? b + 1 : b;
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        const float2 e = __ffma2_rn(pk(c.amp), pk(nrm[b][d], nrm[b + 1][d]),
-                                                    __ffma2_rn(pk(c.mob), pk(F[b][d], F[b + 1][d]),
-                                                               pk(R[b][d], R[b + 1][d])));
-                        Rn[b][d] = e.x;
-                        Rn[b + 1][d] = e.y;
+                        for (int d = 0; d < 3; ++d) {
+                            const float2 e = __ffma2_rn(pk(c.amp), pk(nrm[b][d], nrm[b1][d]),
+                                                        __ffma2_rn(pk(c.mob), pk(F[b][d], F[b1][d]),
+                                                                   pk(R[b][d], R[b1][d])));
+                            Rn[b][d] = e.x;
+                            Rn[b1][d] = e.y;
+                        }
                     }
                 }
             } else {
 #pragma unroll
                 for (int d = 0; d < 3; ++d) Rn[b][d] = R[b][d] + c.mob * F[b][d] + c.amp * nrm[b][d];
             }
-            if (kap_nz && i < Z) {
-                T An[3];
+        }
+        if (ks.nz) {
 #pragma unroll
-                for (int d = 0; d < 3; ++d)
-                    An[d] = A[b][d] + c.dt * (kap[3 * d] * A[b][0] + kap[3 * d + 1] * A[b][1] + kap[3 * d + 2] * A[b][2]);
+            for (int b = 0; b < SB; ++b) {
+                if (ll + b * W < Z) {
+                    T An[3];
 #pragma unroll
-                for (int d = 0; d < 3; ++d) A[b][d] = An[d];
+                    for (int d = 0; d < 3; ++d)
+                        An[d] = A[b][d] +
+                                c.dt * (kx(d) * A[b][0] + ky(d) * A[b][1] + kz(d) * A[b][2]);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) A[b][d] = An[d];
+                }
             }
         }
         if constexpr (HEUN && !FLOW) {
@@ -828,15 +1018,7 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
             // predicted positions is the step's spring force less
             // k_s n_i (Rn_i - R_i), n_i the number of springs on bead i (the
             // same sum, reordered); only the bond forces are recomputed.
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                Pos<T> pn;
-                pn.x = Rn[b][0];
-                pn.y = Rn[b][1];
-                pn.z = Rn[b][2];
-                pn.w = T(0);
-                pos[ll + b * W] = pn;
-            }
+            store_pos(Rn);
             __syncwarp();
 #pragma unroll
             for (int b = 0; b < B; ++b) {
@@ -864,53 +1046,35 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
             // (predicted anchors A under a flow), with the springs and the
             // noise of this step.
             __syncwarp();
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                Pos<T> pn;
-                pn.x = Rn[b][0];
-                pn.y = Rn[b][1];
-                pn.z = Rn[b][2];
-                pn.w = T(0);
-                pos[ll + b * W] = pn;
-            }
+            store_pos(Rn);
             __syncwarp();
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int i = ll + b * W;
-                if (i < Z) {
-                    const Pos<T> ps = pos[S[b]];
-                    SlotRec<T> rec;
-                    rec.x = ps.x - A[b][0];
-                    rec.y = ps.y - A[b][1];
-                    rec.z = ps.z - A[b][2];
-                    rec.s = S[b];
-                    tab[i] = rec;
-                }
-            }
+            rewrite_springs();
             __syncwarp();
             T F2[B][3];
             forces(F2, Rn, false);
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                const int i = ll + b * W;
                 T fl[3] = {T(0), T(0), T(0)};
-                if (kap_nz) {
+                if (ks.nz) {
 #pragma unroll
                     for (int d = 0; d < 3; ++d)
-                        fl[d] = (kap[3 * d] * R[b][0] + kap[3 * d + 1] * R[b][1] + kap[3 * d + 2] * R[b][2]) +
-                                (kap[3 * d] * Rn[b][0] + kap[3 * d + 1] * Rn[b][1] + kap[3 * d + 2] * Rn[b][2]);
+                        fl[d] = (kx(d) * R[b][0] + ky(d) * R[b][1] + kz(d) * R[b][2]) +
+                                (kx(d) * Rn[b][0] + ky(d) * Rn[b][1] + kz(d) * Rn[b][2]);
                 }
 #pragma unroll
                 for (int d = 0; d < 3; ++d)
                     Rn[b][d] = R[b][d] + c.hmob * (F[b][d] + F2[b][d]) + c.hdt * fl[d] + c.amp * nrm[b][d];
-                if (kap_nz && i < Z) {
+            }
+#pragma unroll
+            for (int b = 0; b < SB; ++b) {
+                if (ks.nz && ll + b * W < Z) {
                     T An[3];
 #pragma unroll
                     for (int d = 0; d < 3; ++d)
-                        An[d] = A0[b][d] + c.hdt * ((kap[3 * d] * A0[b][0] + kap[3 * d + 1] * A0[b][1] +
-                                                     kap[3 * d + 2] * A0[b][2]) +
-                                                    (kap[3 * d] * A[b][0] + kap[3 * d + 1] * A[b][1] +
-                                                     kap[3 * d + 2] * A[b][2]));
+                        An[d] = A0[b][d] + c.hdt * ((kx(d) * A0[b][0] + ky(d) * A0[b][1] +
+                                                     kz(d) * A0[b][2]) +
+                                                    (kx(d) * A[b][0] + ky(d) * A[b][1] +
+                                                     kz(d) * A[b][2]));
 #pragma unroll
                     for (int d = 0; d < 3; ++d) A[b][d] = An[d];
                 }
@@ -921,218 +1085,214 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
         // of the position table lie behind the barriers of the slot masks and
         // of the forces already
         if constexpr (HEUN) __syncwarp();
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            Pos<T> pn;
-            pn.x = Rn[b][0];
-            pn.y = Rn[b][1];
-            pn.z = Rn[b][2];
-            pn.w = T(0);
-            pos[ll + b * W] = pn;
-        }
+        store_pos(Rn);
         __syncwarp();
 
         // ---- substep 2: hops on the new positions, one uniform per spring;
-        // sub-slots above every chain's Z in this warp are skipped
+        // sub-slots above every chain's Z in this warp are skipped.  Each slot
+        // clears its record and its bead's mask (the forces have read them) and
+        // keeps the spring vector dd after the move.
         const int zw = z_w;
+        T dd[SB][3];
+        bool cand = false;
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            if (b * W >= zw) break;
-            const int i = ll + b * W;
-            const bool occ = i < Z;
-            const int si = S[b];  // a valid bead index in every slot, occupied or not
-            const int sm = si > 0 ? si - 1 : 0;
-            const int sp = si < N - 1 ? si + 1 : N - 1;
-            const Pos<T> q0 = pos[si], qp = pos[sp], qm = pos[sm];
-            const T r0[3] = {q0.x - A[b][0], q0.y - A[b][1], q0.z - A[b][2]};
-            const T rp[3] = {qp.x - A[b][0], qp.y - A[b][1], qp.z - A[b][2]};
-            const T rm[3] = {qm.x - A[b][0], qm.y - A[b][1], qm.z - A[b][2]};
-            const T d0 = r0[0] * r0[0] + r0[1] * r0[1] + r0[2] * r0[2];
-            T pp, pm;
-            if constexpr (std::is_same<T, float>::value) {
-                // the moves up and down as one packed pair
-                const float2 dpm = __ffma2_rn(pk(rp[2], rm[2]), pk(rp[2], rm[2]),
-                                              __ffma2_rn(pk(rp[1], rm[1]), pk(rp[1], rm[1]),
-                                                         __fmul2_rn(pk(rp[0], rm[0]), pk(rp[0], rm[0]))));
-                const float2 ppm = hop_prob_x2(c, dpm, d0);
-                pp = (si < N - 1) ? ppm.x : T(0);
-                pm = (si > 0) ? ppm.y : T(0);
-            } else {
-                const T dp = rp[0] * rp[0] + rp[1] * rp[1] + rp[2] * rp[2];
-                const T dm = rm[0] * rm[0] + rm[1] * rm[1] + rm[2] * rm[2];
-                pp = (si < N - 1) ? hop_prob_fast<T>(c, dp, d0) : T(0);
-                pm = (si > 0) ? hop_prob_fast<T>(c, dm, d0) : T(0);
+        for (int b = 0; b < SB; ++b) {
+            if (!skip(b, zw)) {
+                const int i = ll + b * W;
+                const bool occ = i < Z;
+                const int si = S[b];  // a valid bead index in every slot, occupied or not
+                rec[loc[b]] = zrec;
+                msk[si] = Mask(0);
+                bool up, dn;
+                if constexpr (WIN == kWinReplay) {
+                    // (a tape recorded from another state must not move a spring off the chain)
+                    up = occ && (tb[b] & kTapeUp) && si < N - 1;
+                    dn = occ && (tb[b] & kTapeDown) && si > 0;
+                    S[b] = up ? si + 1 : (dn ? si - 1 : si);
+                    const Pos<T> ps = pos[S[b]];
+                    dd[b][0] = ps.x - A[b][0];
+                    dd[b][1] = ps.y - A[b][1];
+                    dd[b][2] = ps.z - A[b][2];
+                } else {
+                    const Pos<T> q0 = pos[si], qp = pos[si + 1], qm = pos[si - 1];
+                    const T r0[3] = {q0.x - A[b][0], q0.y - A[b][1], q0.z - A[b][2]};
+                    const T rp[3] = {qp.x - A[b][0], qp.y - A[b][1], qp.z - A[b][2]};
+                    const T rm[3] = {qm.x - A[b][0], qm.y - A[b][1], qm.z - A[b][2]};
+                    const T d0 = r0[0] * r0[0] + r0[1] * r0[1] + r0[2] * r0[2];
+                    const T dp = fma(rp[2], rp[2], fma(rp[1], rp[1], rp[0] * rp[0]));
+                    const T dm = fma(rm[2], rm[2], fma(rm[1], rm[1], rm[0] * rm[0]));
+                    T pp, pm;
+                    if constexpr (std::is_same<T, float>::value) {
+                        const float2 ppm = hop_prob_x2(c, make_float2(dp, dm), d0);
+                        pp = (si < N - 1) ? ppm.x : T(0);
+                        pm = (si > 0) ? ppm.y : T(0);
+                    } else {
+                        pp = (si < N - 1) ? hop_prob<T>(c, dp, d0) : T(0);
+                        pm = (si > 0) ? hop_prob<T>(c, dm, d0) : T(0);
+                    }
+                    up = occ && (u[b] < pp);
+                    dn = occ && !up && (u[b] < pp + pm);
+                    if constexpr (WIN == kWinRecord) tb[b] = (up ? kTapeUp : 0) | (dn ? kTapeDown : 0);
+                    S[b] = up ? si + 1 : (dn ? si - 1 : si);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) dd[b][d] = up ? rp[d] : (dn ? rm[d] : r0[d]);
+                }
+                cnt_up += up ? 1u : 0u;
+                cnt_dn += dn ? 1u : 0u;
+                if constexpr (WIN != kWinReplay)
+                    cand |= occ && (nrm[b][3] < c.cd) && ((unsigned)(S[b] - 1) >= (unsigned)(N - 2));
             }
-            bool up = occ && (u[b] < pp);
-            bool dn = occ && !up && (u[b] < pp + pm);
-            if (tmode == 2) {
-                up = occ && (tb[b] & kTapeUp);
-                dn = occ && (tb[b] & kTapeDown);
-            }
-            if (tmode == 1) tb[b] |= (up ? kTapeUp : 0) | (dn ? kTapeDown : 0);
-            S[b] = up ? si + 1 : (dn ? si - 1 : S[b]);
-            cnt_up += up ? 1u : 0u;
-            cnt_dn += dn ? 1u : 0u;
         }
 
         // ---- substep 3a: creation, K attempts at both ends
-        const int Zc = Z;
-        const int first = Zc, last = c_last;
         if (c_drop) ++cnt_drop;
-        const T pc = T(0.5) * c_pc2;
         // a slot can change only if it may create (u < 2 p_c on an attempt) or
         // sits at an end with a destruction hit: the detailed work below runs
         // only when some slot of the warp can
-        bool cand = WIN;
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-            cand |= ((i >= first) && (i < last) && (u[b] < c_pc2)) ||
-                    ((i < Zc) && (S[b] == 0 || S[b] == N - 1) && (nrm[b][3] < c.cd));
+        for (int b = 0; b < SB; ++b) {
+            if constexpr (WIN == kWinReplay)
+                cand |= (tb[b] & (kTapeNew0 | kTapeNewN | kTapeKillOld | kTapeKillNew)) != 0;
+            else  // S = 0 or S = N - 1: S - 1 >= N - 2 as unsigned numbers
+                cand |= u[b] < thr_c[b];
         }
         if (__any_sync(kFull, cand)) {
-        int end_new[B];
-        bool any_new = false;
+            // ---- substeps 3a and 3b in detail, then the re-indexing: survivors in
+            // slot order (sub-slot major, then lane), new springs at bead 1 in
+            // attempt order, new springs at bead N
+            const int Zc = Z, last = attempts_end();
+            const T pc = c.pc[last - Zc], pc2 = T(2) * pc;
+            int end_new[SB];  // the end a spring is created at by this slot's attempt, -1 none
+            bool gone[SB];    // an old spring destroyed
+            bool any_new = false, any_gone = false;
 #pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-            const bool att = (i >= first) && (i < last);
-            end_new[b] = !att ? -1 : (u[b] < pc ? 0 : (u[b] < c_pc2 ? N - 1 : -1));
-            if (tmode == 2) end_new[b] = !att ? -1 : ((tb[b] & kTapeNew0) ? 0 : ((tb[b] & kTapeNewN) ? N - 1 : -1));
-            if (tmode == 1) tb[b] |= end_new[b] == 0 ? kTapeNew0 : (end_new[b] > 0 ? kTapeNewN : 0);
-            any_new |= end_new[b] >= 0;
-        }
-        T Anew[B][3];
-#pragma unroll
-        for (int b = 0; b < B; ++b) Anew[b][0] = Anew[b][1] = Anew[b][2] = T(0);
-        const bool some_new = __any_sync(kFull, any_new);
-        if (some_new) {
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                if (end_new[b] >= 0) {
-                    const Pos<T> pe = pos[end_new[b]];
-                    const uint4 wc = philox4x32_10_rk((uint32_t)(ll + b * W), t, kPurposeCreate, chain_id, c.rk0,
-                                                      c.rk1);
-                    T n3[4];
-                    box_muller<T>(wc.x, wc.y, n3[0], n3[1]);
-                    box_muller<T>(wc.z, wc.w, n3[2], n3[3]);
-                    Anew[b][0] = pe.x + c.sa * n3[0];
-                    Anew[b][1] = pe.y + c.sa * n3[1];
-                    Anew[b][2] = pe.z + c.sa * n3[2];
-                    ++cnt_cr;
-                }
-            }
-        }
-
-        // ---- substep 3b: destruction at the ends, then re-indexing
-        bool alive_old[B], alive_new[B];
-        bool any_change = false;
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-            const bool hit = nrm[b][3] < c.cd;
-            bool kill_old = (i < Zc) && (S[b] == 0 || S[b] == N - 1) && hit;
-            bool kill_new = (end_new[b] >= 0) && a.destroy_new && hit;
-            if (tmode == 2) {
-                kill_old = (i < Zc) && (tb[b] & kTapeKillOld);
-                kill_new = (end_new[b] >= 0) && (tb[b] & kTapeKillNew);
-            }
-            if (tmode == 1) {
-                tb[b] |= (kill_old ? kTapeKillOld : 0) | (kill_new ? kTapeKillNew : 0);
-                if (tape_row) a.tape[((size_t)trow * a.M + mm) * NP + ll + b * W] = tb[b];
-            }
-            alive_old[b] = (i < Zc) && !kill_old;
-            alive_new[b] = (end_new[b] >= 0) && !kill_new;
-            cnt_de += (kill_old ? 1u : 0u) + (kill_new ? 1u : 0u);
-            any_change |= kill_old || (end_new[b] >= 0);
-        }
-        if (__any_sync(kFull, any_change)) {
-            // slot order: sub-slot major, then lane; survivors, then new springs at
-            // bead 1 in attempt order, then new springs at bead N
-            int dest[B];
-            int base = 0;
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const unsigned kb = __ballot_sync(kFull, alive_old[b]) & segmask;
-                dest[b] = alive_old[b] ? base + __popc(kb & lt) : -1;
-                base += __popc(kb);
-            }
-            if (some_new) {  // new springs in this warp: at bead 1, then at bead N
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const bool e0 = alive_new[b] && end_new[b] == 0;
-                const unsigned nb = __ballot_sync(kFull, e0) & segmask;
-                if (e0) dest[b] = base + __popc(nb & lt);
-                base += __popc(nb);
-            }
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const bool eN = alive_new[b] && end_new[b] == N - 1;
-                const unsigned nb = __ballot_sync(kFull, eN) & segmask;
-                if (eN) dest[b] = base + __popc(nb & lt);
-                base += __popc(nb);
-            }
-            }
-            const int Znew = base;
-            __syncwarp();
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                if (dest[b] >= 0) {
-                    SlotRec<T> rec;
-                    rec.x = alive_old[b] ? A[b][0] : Anew[b][0];
-                    rec.y = alive_old[b] ? A[b][1] : Anew[b][1];
-                    rec.z = alive_old[b] ? A[b][2] : Anew[b][2];
-                    rec.s = alive_old[b] ? S[b] : end_new[b];
-                    tab[dest[b]] = rec;
-                }
-            }
-            __syncwarp();
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
+            for (int b = 0; b < SB; ++b) {
                 const int i = ll + b * W;
-                if (i < Znew) {
-                    const SlotRec<T> rec = tab[i];
-                    S[b] = rec.s;
-                    A[b][0] = rec.x;
-                    A[b][1] = rec.y;
-                    A[b][2] = rec.z;
+                const bool hit = nrm[b][3] < c.cd;
+                const bool att = i >= Zc && i < last;
+                if constexpr (WIN == kWinReplay) {
+                    end_new[b] = !att ? -1 : ((tb[b] & kTapeNew0) ? 0 : ((tb[b] & kTapeNewN) ? N - 1 : -1));
+                    gone[b] = i < Zc && (tb[b] & kTapeKillOld);
+                } else {
+                    end_new[b] = !att ? -1 : (u[b] < pc ? 0 : (u[b] < pc2 ? N - 1 : -1));
+                    gone[b] = i < Zc && hit && (S[b] == 0 || S[b] == N - 1);
+                }
+                const bool made = end_new[b] >= 0;
+                const bool undone =  // created and destroyed within the step
+                    made && (WIN == kWinReplay ? (tb[b] & kTapeKillNew) != 0 : a.destroy_new && hit);
+                if constexpr (WIN == kWinRecord)
+                    tb[b] |= (made ? (end_new[b] == 0 ? kTapeNew0 : kTapeNewN) : 0) | (gone[b] ? kTapeKillOld : 0) |
+                             (undone ? kTapeKillNew : 0);
+                cnt_cr += made ? 1u : 0u;
+                cnt_de += (gone[b] ? 1u : 0u) + (undone ? 1u : 0u);
+                if (undone) end_new[b] = -1;
+                any_new |= end_new[b] >= 0;
+                any_gone |= gone[b];
+            }
+            int base = Zc;  // springs placed so far
+            if (__any_sync(kFull, any_gone)) {
+                int dest[SB];
+                base = 0;
+#pragma unroll
+                for (int b = 0; b < SB; ++b) {
+                    const bool stays = ll + b * W < Zc && !gone[b];
+                    const unsigned kb = __ballot_sync(kFull, stays) & segmask;
+                    dest[b] = stays ? base + __popc(kb & lt) : -1;
+                    base += __popc(kb);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int b = 0; b < SB; ++b) {
+                    if (dest[b] >= 0) {
+                        SlotRec<T> r;
+                        r.x = A[b][0];
+                        r.y = A[b][1];
+                        r.z = A[b][2];
+                        r.s = S[b];
+                        tab[dest[b]] = r;
+                    }
+                }
+            }
+            int Znew = base;
+            if (__any_sync(kFull, any_new)) {
+                int dest[SB];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+#pragma unroll
+                    for (int b = 0; b < SB; ++b) {
+                        const bool here = end_new[b] == (e == 0 ? 0 : N - 1);
+                        const unsigned nb = __ballot_sync(kFull, here) & segmask;
+                        if (here) dest[b] = Znew + __popc(nb & lt);
+                        Znew += __popc(nb);
+                    }
+                }
+                __syncwarp();
+#pragma unroll
+                for (int b = 0; b < SB; ++b) {
+                    if (end_new[b] >= 0) {
+                        const Pos<T> pe = pos[end_new[b]];
+                        const uint4 wc = philox4x32_10_rk((uint32_t)(ll + b * W), t, kPurposeCreate, chain_id, c.rk0,
+                                                          c.rk1);
+                        T n3[4];
+                        box_muller<T>(wc.x, wc.y, n3[0], n3[1]);
+                        box_muller<T>(wc.z, wc.w, n3[2], n3[3]);
+                        SlotRec<T> r;
+                        r.x = pe.x + c.sa * n3[0];
+                        r.y = pe.y + c.sa * n3[1];
+                        r.z = pe.z + c.sa * n3[2];
+                        r.s = end_new[b];
+                        tab[dest[b]] = r;
+                    }
+                }
+            }
+            __syncwarp();
+            // slots whose content moved: all of a chain that lost a spring, else the new ones
+#pragma unroll
+            for (int b = 0; b < SB; ++b) {
+                const int i = ll + b * W;
+                if (i < Znew && (base != Zc || i >= Zc)) {
+                    const SlotRec<T> r = tab[i];
+                    S[b] = r.s;
+                    A[b][0] = r.x;
+                    A[b][1] = r.y;
+                    A[b][2] = r.z;
                 }
             }
             __syncwarp();
             Z = Znew;
             set_create();
+            spring_vectors(dd);
         }
-        }  // candidates
-        draw(t + 1u, nrm, u);  // the next step's random numbers
+        if constexpr (WIN == kWinRecord) {
+            const long long row = (long long)t0_ + s - a.tape_t0;
+            if (live && row >= 0 && row < a.tape_rows) {
+#pragma unroll
+                for (int b = 0; b < SB; ++b) a.tape[((size_t)row * a.M + mm) * NP + ll + b * W] = tb[b];
+            }
+        }
+        // ---- spring vectors of the new state: this step's stress (with a stiffness
+        // of 0 in an empty slot), the next step's spring forces
+        __syncwarp();  // every slot has cleared its record and mask
+        register_springs(dd);
+        const int zn = z_w;
+        T sv[VL][3];  // this lane's parts of sigma^(v)_xy, xz, yz
+#pragma unroll
+        for (int v = 0; v < VL; ++v) sv[v][0] = sv[v][1] = sv[v][2] = T(0);
+#pragma unroll
+        for (int b = 0; b < SB; ++b) {
+            T(&x)[3] = sv[b % VL];
+            if (!skip(b, zn)) {
+                const T ks_b = ll + b * W < Z ? c.k_s : T(0);
+                const T kd0 = ks_b * dd[b][0], kd1 = ks_b * dd[b][1];
+                x[0] = fma(kd0, dd[b][1], x[0]);
+                x[1] = fma(kd0, dd[b][2], x[1]);
+                x[2] = fma(kd1, dd[b][2], x[2]);
+            }
+        }
 #pragma unroll
         for (int b = 0; b < B; ++b)
 #pragma unroll
             for (int d = 0; d < 3; ++d) R[b][d] = Rn[b][d];
-
-        // ---- spring vectors of the new state, d_j = R_{S_j} - A_j (0 for an
-        // empty slot): next step's spring forces and this step's stress;
-        // sub-slots above every chain's Z in this warp hold none
-        const int zn = z_w;
-        T dd[B][3];
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            dd[b][0] = dd[b][1] = dd[b][2] = T(0);
-            if (b * W < zn) {
-                const int i = ll + b * W;
-                const Pos<T> ps = pos[i < Z ? S[b] : 0];
-                if (i < Z) {
-                    dd[b][0] = ps.x - A[b][0];
-                    dd[b][1] = ps.y - A[b][1];
-                    dd[b][2] = ps.z - A[b][2];
-                    SlotRec<T> rec;
-                    rec.x = dd[b][0];
-                    rec.y = dd[b][1];
-                    rec.z = dd[b][2];
-                    rec.s = S[b];
-                    tab[i] = rec;
-                }
-            }
-        }
 
         // ---- bond vectors of the new state: this step's stress, the next
         // step's bond forces
@@ -1141,72 +1301,63 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
         // ---- stress of the new state (Eq. stress_tensor_single_chain, App. B)
         const bool do_log = (s == next_log);
         if (do_log) next_log += a.log_every;
-        const bool do_rc = (s == next_rc) && kap_nz;
+        const bool do_rc = (s == next_rc) && ks.nz;
         if (s == next_rc) next_rc += a.recenter_every;
         // per-lane parts of the off-diagonal sigma_ab (bonds) and sigma_ab +
         // sigma^(v)_ab (v[0..5]), and with `diag` the bond part of sigma_aa
-        auto stress_parts = [&](T (&v)[8], T (&dgp)[3], const bool diag) {
+        auto stress_parts = [&](T (&vs)[6], T (&dgs)[3], const bool diag) {
+            T v[VL][3], dgp[VL][3];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) v[k] = T(0);
-            dgp[0] = dgp[1] = dgp[2] = T(0);
+            for (int p = 0; p < VL; ++p)
+#pragma unroll
+                for (int k = 0; k < 3; ++k) v[p][k] = dgp[p][k] = T(0);
 #pragma unroll
             for (int b = 0; b < B; ++b) {
-                const T (&q)[3] = Q[b];  // the last bead's is 0
-                T kq0, kq1;
-                if constexpr (std::is_same<T, float>::value) {  // (xy, xz) as a packed pair
-                    const float2 kq = __fmul2_rn(pk(c.k_b), pk(q[0], q[1]));
-                    kq0 = kq.x;
-                    kq1 = kq.y;
-                    const float2 v01 = __ffma2_rn(pk(kq0), pk(q[1], q[2]), pk(v[0], v[1]));
-                    v[0] = v01.x;
-                    v[1] = v01.y;
-                    v[2] += kq1 * q[2];
-                    if (b * W < zn) {  // springs (an empty slot's d is 0)
-                        const float2 kd = __fmul2_rn(pk(c.k_s), pk(dd[b][0], dd[b][1]));
-                        const float2 v34 = __ffma2_rn(pk(kd.x), pk(dd[b][1], dd[b][2]), pk(v[3], v[4]));
-                        v[3] = v34.x;
-                        v[4] = v34.y;
-                        v[5] += kd.y * dd[b][2];
-                    }
-                } else {
-                    kq0 = c.k_b * q[0];
-                    kq1 = c.k_b * q[1];
-                    v[0] += kq0 * q[1];
-                    v[1] += kq0 * q[2];
-                    v[2] += kq1 * q[2];
-                    if (b * W < zn) {  // springs (an empty slot's d is 0)
-                        const T kd0 = c.k_s * dd[b][0], kd1 = c.k_s * dd[b][1];
-                        v[3] += kd0 * dd[b][1];
-                        v[4] += kd0 * dd[b][2];
-                        v[5] += kd1 * dd[b][2];
-                    }
-                }
+                const T(&q)[3] = Q[b];  // the last bead's is 0
+                T(&x)[3] = v[b % VL];
+                T(&dg)[3] = dgp[b % VL];
+                const T kq0 = c.k_b * q[0], kq1 = c.k_b * q[1];
+                x[0] = fma(kq0, q[1], x[0]);
+                x[1] = fma(kq0, q[2], x[1]);
+                x[2] = fma(kq1, q[2], x[2]);
                 if (diag) {
-                    dgp[0] += kq0 * q[0];
-                    dgp[1] += kq1 * q[1];
-                    dgp[2] += c.k_b * q[2] * q[2];
+                    dg[0] += kq0 * q[0];
+                    dg[1] += kq1 * q[1];
+                    dg[2] += c.k_b * q[2] * q[2];
                 }
             }
-            v[3] += v[0];
-            v[4] += v[1];
-            v[5] += v[2];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                vs[k] = v[0][k];
+                vs[3 + k] = sv[0][k] + v[0][k];
+                dgs[k] = dgp[0][k];
+                if constexpr (VL == 2) {
+                    vs[k] += v[VL - 1][k];
+                    vs[3 + k] += sv[VL - 1][k] + v[VL - 1][k];
+                    dgs[k] += dgp[VL - 1][k];
+                }
+            }
         };
         if (corr_on) {  // every step: the correlator's input
-            T v[8], dgp[3];
+            T v[6], dgp[3];
             stress_parts(v, dgp, false);
-            const T red = seg_reduce6<T, W>(v, ll);
-            if (ser_m != nullptr) ser_m[(size_t)s * ser_step] = red;
+            if constexpr (sizeof(T) == 4) {
+                red_put(v);
+            } else {
+                const T r = seg_reduce6<T, W>(v, ll);
+                if (ser_m != nullptr) ser_m[(size_t)s * ser_step] = r;
+            }
         }
         if (do_log) {
             // a log step (warp-uniform, every log_every steps): the stress
             // again with its diagonal, kept out of the every-step path
-            T v[8], dgp[3];
+            T v[6], dgp[3];
             stress_parts(v, dgp, true);
-            const T red = seg_reduce6<T, W>(v, ll);
+            const T r6 = seg_reduce6<T, W>(v, ll);
             T sig[3], dg[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                sig[d] = shfl(red, d == 0 ? 0 : (d == 1 ? W / 4 : W / 8), W);
+                sig[d] = shfl(r6, d == 0 ? 0 : (d == 1 ? W / 4 : W / 8), W);
                 dg[d] = seg_sum<T, W>(dgp[d]) - NkT;
             }
             const int slot = log_slot++;
@@ -1224,55 +1375,53 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
             }
         }
         if (do_rc) {
-            T csum[3] = {T(0), T(0), T(0)};
+            T csum[VL][3];
+#pragma unroll
+            for (int p = 0; p < VL; ++p) csum[p][0] = csum[p][1] = csum[p][2] = T(0);
 #pragma unroll
             for (int b = 0; b < B; ++b)
 #pragma unroll
-                for (int d = 0; d < 3; ++d) csum[d] += (ll + b * W < N) ? R[b][d] : T(0);
+                for (int d = 0; d < 3; ++d) csum[b % VL][d] += (ll + b * W < N) ? R[b][d] : T(0);
             T com[3];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) com[d] = seg_sum<T, W>(csum[d]) / T(N);
+            for (int d = 0; d < 3; ++d) {
+                if constexpr (VL == 2) csum[0][d] += csum[VL - 1][d];
+                com[d] = seg_sum<T, W>(csum[0][d]) / T(N);
+            }
             __syncwarp();
 #pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int i = ll + b * W;
+            for (int b = 0; b < B; ++b)
 #pragma unroll
-                for (int d = 0; d < 3; ++d) {
-                    if (i < N) R[b][d] -= com[d];
-                    if (i < Z) A[b][d] -= com[d];
-                }
-                Pos<T> pn;
-                pn.x = R[b][0];
-                pn.y = R[b][1];
-                pn.z = R[b][2];
-                pn.w = T(0);
-                pos[i] = pn;
-            }
+                for (int d = 0; d < 3; ++d)
+                    if (ll + b * W < N) R[b][d] -= com[d];
+#pragma unroll
+            for (int b = 0; b < SB; ++b)
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    if (ll + b * W < Z) A[b][d] -= com[d];
+            store_pos(R);
             // the spring and bond vectors from the shifted coordinates, as a
             // launch starting here computes them: results do not depend on
             // where the launches end
             __syncwarp();
             bond_vectors();
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int i = ll + b * W;
-                if (i < Z) {
-                    const Pos<T> ps = pos[S[b]];
-                    SlotRec<T> rec;
-                    rec.x = ps.x - A[b][0];
-                    rec.y = ps.y - A[b][1];
-                    rec.z = ps.z - A[b][2];
-                    rec.s = S[b];
-                    tab[i] = rec;
-                }
-            }
+            rewrite_springs();
         }
         __syncwarp();
+        if constexpr (sizeof(T) == 4) {
+            if (corr_on && ++red_n == kRedSteps) red_flush(s + 1);
+        }
+    }
+    if (!FLOW || s >= nsteps_) break;
+    load_kappa(s);
+    }
+    if constexpr (sizeof(T) == 4) {
+        if (corr_on) red_flush(nsteps_);
     }
 
-    if (WIN && a.snapR != nullptr && live) {
+    if (WIN == kWinReplay && a.snapR != nullptr && live) {
         const long long sr = (long long)t0_ + nsteps_ - a.snap_t0;
-        if (sr >= 0 && sr <= a.snap_steps) snapshot_store<T, W, B>(a, sr, mm, ll, R, A, S, Z);
+        if (sr >= 0 && sr <= a.snap_steps) snapshot_store<T, W, B, SB>(a, sr, mm, ll, R, A, S, Z);
     }
 
     // ---- store state
@@ -1285,16 +1434,24 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             const int i = ll + b * W;
-            a.S[(size_t)mm * NP + i] = (i < Z) ? S[b] : -1;
-            broken |= (i < Z) && (S[b] < 0 || S[b] >= N);
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 if (i < N) {
                     Rw[((size_t)mm * 3 + d) * NP + i] = R[b][d];
                     bad |= !Mth<T>::finite(R[b][d]);
                 }
-                Aw[((size_t)mm * 3 + d) * NP + i] = (i < Z) ? A[b][d] : T(0);
             }
+        }
+#pragma unroll
+        for (int i0 = 0; i0 < NP; i0 += W) {  // every column: slots above this layout's are empty
+            const int i = i0 + ll, b = i0 / W;
+            const int sj = b < SB ? S[b < SB ? b : 0] : 0;
+            const bool occ = b < SB && i < Z;
+            a.S[(size_t)mm * NP + i] = occ ? sj : -1;
+            broken |= occ && (sj < 0 || sj >= N);
+#pragma unroll
+            for (int d = 0; d < 3; ++d)
+                Aw[((size_t)mm * 3 + d) * NP + i] = occ ? A[b < SB ? b : 0][d] : T(0);
         }
     }
     if (__any_sync(kFull, bad) && lane == 0) {
@@ -1335,25 +1492,25 @@ __device__ __forceinline__ void run_chains(const ChunkArgs& a, const StepConst<T
     }
 }
 
-// WIN: the differentiation-window hooks (decision tape, snapshots, stress
-// series) are compiled in; the plain kernel carries none of them.  FLOW: the
+// WIN: the differentiation-window hooks are compiled in (kWinRecord,
+// kWinReplay); the plain kernel (kWinOff) carries none of them.  FLOW: the
 // velocity-gradient terms are compiled in (launches with kappa = 0 throughout
 // may use the instantiation without them).  HEUN: the stochastic Heun
-// integrator instead of Euler-Maruyama for substep 1.
-template <typename T, int W, int B, bool WIN, bool FLOW, bool HEUN = false>
-__global__ void __launch_bounds__(kChunkThreads, B == 1 ? SS_CTAS_PER_SM : (B >= 4 ? 4 : SS_CTAS_PER_SM_MULTI))
+// integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
+// be written (without one, its registers are free).
+template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm(B))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
-    run_chains<T, W, B, WIN, FLOW, HEUN>(a, c, blockIdx.x * (kChunkThreads / W), c.NkT, a.t0, a.nsteps, a.log_m0,
+    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, blockIdx.x * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
                                          a.nlog_chunk);
 }
 
 // ------------------------------------------------------ batched kernel ------
-// Many elements in one persistent launch per lane layout: each CTA takes work
-// items (element, first chain of a CTA tile) of its layout class from an
-// atomic counter until the list is exhausted, and runs the tile for all steps
-// of the launch.  The counter is only ever incremented: no CTA waits for
-// another.  Each element's arguments (state pointers, sizes, flow schedule,
-// log buffers) live in a device array and are read in place.
+// Many elements in one launch per lane layout: CTA k runs work item k (element,
+// first chain of a CTA tile) of its layout class for all steps of the launch.  The
+// items are ordered longest first and the hardware starts CTAs in order, as slots
+// free up.  Each element's arguments (state pointers, sizes, flow schedule, log
+// buffers) live in a device array; a CTA reads them from shared memory.
 struct RunInfo {
     long long t0;     // first step of this launch
     int nsteps;
@@ -1361,403 +1518,23 @@ struct RunInfo {
 };
 
 template <typename T, int W, int B>
-__global__ void __launch_bounds__(kChunkThreads, B == 1 ? SS_CTAS_PER_SM : (B == 2 ? SS_CTAS_PER_SM_MULTI : SS_CTAS_PER_SM_BATCHED_MULTI))
-    batched_kernel(const ChunkArgs* __restrict__ elems, const int2* __restrict__ items, int n_items,
-                   unsigned* __restrict__ next_item, const RunInfo info, const StepConst<T> c) {
-    __shared__ int item_s;
-    for (;;) {
-        __syncthreads();
-        if (threadIdx.x == 0) item_s = (int)atomicAdd(next_item, 1u);
-        __syncthreads();
-        const int it = item_s;
-        if (it >= n_items) break;
-        const int2 wi = items[it];
-        const ChunkArgs& a = elems[wi.x];
-        const int nlog = a.log_every > 0 ? (int)((info.t0 + info.nsteps) / a.log_every - info.t0 / a.log_every) : 0;
-        run_chains<T, W, B, false, true>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps, info.log_m0, nlog);
-    }
-}
-
-// ----------------------------------------------------- correlator kernels ----
-// Multiple-tau lag products of one launch's stress series (Eq.
-// relaxation_modulus_tensor_green_kubo_form, App. B).  Level 0 holds the raw
-// samples; level l >= 1 the means of two consecutive level-(l-1) samples, i.e.
-// of blocks of 2^l raw samples aligned to the absolute sample index.  At level
-// l, lag k (0..15 at level 0, 8..15 above) adds x_l(j) y_l(j - k) for every
-// sample j completed in this launch, with x = sigma_off (the later value) and
-// y = sigma_off (AUTO channel) or (sigma + sigma^(v))_off (TOTAL channel).
-//
-// One thread per (chain, series row q): q = 0..2 are sigma_off (xy, xz, yz),
-// q = 3..5 (sigma + sigma^(v))_off; a warp holds 5 chains x 6 rows, and the
-// later value x of row q is row q % 3 of the same chain, taken by a shuffle.
-// Samples of a level are [j][M][6] arrays (the chain kernel's series for
-// level 0).  hist [M][L][6][16] keeps the newest 16 samples of every level
-// and row (oldest first, zero after a reset): the lags reach back into
-// earlier launches through a 16-entry register ring; each level's pass
-// writes its own history when it ends.  A CTA covers one slice of
-// kSliceChains chains and adds its chains' sums of this launch, in chain
-// order, to the slice's FP64 sums acc64 [slices][L][3][32] (component,
-// channel * 16 + lag).  With TT the rows of sigma + sigma^(v) also take their
-// own samples as the later value (channel TT, acc64tt [slices][L][3][16]).
-constexpr int kCorrChainsPerWarp = 5;
-constexpr int kCorrWarps = (kSliceChains + kCorrChainsPerWarp - 1) / kCorrChainsPerWarp;  // 13
-constexpr int kCorrThreads = kCorrWarps * 32;
-constexpr int kCorrMaxSteps = 1024;  // samples per launch (the level-sample buffers hold half)
-
-// This slice's FP32 sums of one level (each thread's lags k0..15 of its row),
-// folded in chain order into FP64.
-// Channel TT of the rows q >= 3, folded the same way into out [3][16].
-// Sum of column i over the kSliceChains rows of red (row stride `stride`), in
-// chain order, in FP64.  FP32 rows go in blocks of eight: a block is summed in
-// FP32 while the rounding error of every addition is kept exactly (TwoSum,
-// Knuth) and summed beside it, then the block's sum and error are added in
-// FP64.  The result has FP64 accuracy with a quarter of the FP64 conversions
-// and additions (the FP64 pipe runs at a small fraction of the FP32 rate).
-template <typename T>
-__device__ __forceinline__ double slice_column_sum(const T* red, int stride, int i) {
-    static_assert(kSliceChains % 8 == 0, "blocks of eight chains");
-    double sum = 0.0;
-    if constexpr (sizeof(T) == 4) {
-        for (int c0 = 0; c0 < kSliceChains; c0 += 8) {
-            float s = red[(size_t)c0 * stride + i], e = 0.0f;
-#pragma unroll
-            for (int c = 1; c < 8; ++c) {
-                const float x = red[(size_t)(c0 + c) * stride + i];
-                const float t = s + x;
-                const float bp = t - s;
-                e += (s - (t - bp)) + (x - bp);
-                s = t;
-            }
-            sum += (double)s;
-            sum += (double)e;
-        }
-    } else {
-        for (int c = 0; c < kSliceChains; ++c) sum += (double)red[(size_t)c * stride + i];
-    }
-    return sum;
-}
-
-template <typename T>
-__device__ __forceinline__ void corr_fold_slice_tt(const T (&acc2)[16], int k0, bool live, int slot, int q,
-                                                   double* __restrict__ out, T* red) {
-    __syncthreads();  // the first fold has read red
-    if (slot < kSliceChains && q >= 3) {
-        T* row = red + (size_t)slot * 48 + (q - 3) * kP;
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (k >= k0) row[k] = live ? acc2[k] : T(0);
-    }
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm(B))
+    batched_kernel(const ChunkArgs* __restrict__ elems, const int2* __restrict__ items, const RunInfo info,
+                   const StepConst<T> c) {
+    static_assert(sizeof(ChunkArgs) % 8 == 0, "copied in 8-byte words");
+    __shared__ unsigned long long args_s[sizeof(ChunkArgs) / 8];
+    // volatile: read where they are used (most of them in rare branches), not kept
+    // in registers for the whole launch
+    const volatile ChunkArgs& a = *reinterpret_cast<const volatile ChunkArgs*>(args_s);
+    const int2 wi = items[blockIdx.x];
+    for (int i = threadIdx.x; i < (int)(sizeof(ChunkArgs) / 8); i += blockDim.x)
+        args_s[i] = reinterpret_cast<const unsigned long long*>(elems + wi.x)[i];
     __syncthreads();
-    for (int i = threadIdx.x; i < 48; i += blockDim.x) {
-        if (i % kP < k0) continue;
-        out[i] += slice_column_sum(red, 48, i);
-    }
-}
-
-template <typename T>
-__device__ __forceinline__ void corr_fold_slice(const T (&acc)[16], int k0, bool live, int slot, int q,
-                                                double* __restrict__ out, T* red) {
-    // red: [kSliceChains][96] T in shared memory, free once every thread is here
-    __syncthreads();
-    if (slot < kSliceChains) {
-        T* row = red + (size_t)slot * 96 + (q % 3) * kCells + (q / 3) * kP;
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (k >= k0) row[k] = live ? acc[k] : T(0);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 96; i += blockDim.x) {
-        const int lag = i % kP;
-        if (lag < k0) continue;
-        out[i] += slice_column_sum(red, 96, i);
-    }
-}
-
-// Ring of the newest 16 samples of one row: r[i] holds sample base + i - 16
-// when the next sample to enter is sample base (i.e. after a whole number of
-// 16-sample blocks).  Products of n new samples, sample j given by get(j) (a
-// load), each later value x taken from lane src_lane; emit(j, y) sees every
-// sample in order (the pair means of the level above are formed there).  nr
-// returns the ring position of the next sample (the number of samples in the
-// last partial block).  With TT, acc2 also takes the row's own sample as the
-// later value (for the rows of sigma + sigma^(v): channel TT).
-template <typename T, int K0, bool TT, typename Get, typename Emit>
-__device__ __forceinline__ void corr_ring_products(T (&r)[16], T (&acc)[16], T (&acc2)[16], Get get, Emit emit,
-                                                   int n, int src_lane, int& nr) {
-    int j = 0;
-    for (; j + 16 <= n; j += 16) {
-        T yv[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) yv[u] = get(j + u);  // independent loads first
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            emit(j + u, yv[u]);
-            const T xv = __shfl_sync(kFull, yv[u], src_lane);
-            r[u] = yv[u];
-#pragma unroll
-            for (int k = K0; k < 16; ++k) acc[k] += xv * r[(u - k) & 15];
-            if constexpr (TT) {
-#pragma unroll
-                for (int k = K0; k < 16; ++k) acc2[k] += yv[u] * r[(u - k) & 15];
-            }
-        }
-    }
-    const int rem = n - j;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-        if (u < rem) {
-            const T yv = get(j + u);
-            emit(j + u, yv);
-            const T xv = __shfl_sync(kFull, yv, src_lane);
-            r[u] = yv;
-#pragma unroll
-            for (int k = K0; k < 16; ++k) acc[k] += xv * r[(u - k) & 15];
-            if constexpr (TT) {
-#pragma unroll
-                for (int k = K0; k < 16; ++k) acc2[k] += yv * r[(u - k) & 15];
-            }
-        }
-    }
-    nr = rem;
-}
-
-// The newest 16 samples in ring order after `nr` samples of a partial block:
-// out[i] = r[(nr + i) & 15].
-template <typename T>
-__device__ __forceinline__ void corr_ring_newest(const T (&r)[16], int nr, T* out) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        T v = r[0];
-#pragma unroll
-        for (int s2 = 1; s2 < 16; ++s2)
-            if (((nr + i) & 15) == s2) v = r[s2];
-        out[i] = v;
-    }
-}
-
-// All levels of one launch in one kernel.  Level l's pass reads the level-l
-// samples of this launch (the series rows for level 0, else the samples the
-// pass below stored), adds their products, and, as the samples stream by,
-// stores the pairwise means that are the level-(l+1) samples into one of the
-// ping-pong buffers lev (lev_half elements each).  A mean may pair the newest
-// level-l sample of the previous launch (the last entry of the level's
-// history) with the first new one.  Every thread reads only rows it wrote
-// itself (its chain and series row); the block synchronises only for the
-// slice folds.
-template <typename T, bool TT>
-__global__ void __launch_bounds__(kCorrThreads, (sizeof(T) == 4 && !TT) ? 2 : 1)
-    corr_kernel(const T* __restrict__ ser, int ns, long long n0, int M, int L, T* __restrict__ hist,
-                T* __restrict__ lev, size_t lev_half, double* __restrict__ acc64, double* __restrict__ acc64tt) {
-    __shared__ T red[kSliceChains * 96];
-    const int lane = threadIdx.x & 31;
-    const int cc = lane / 6, q = lane % 6;
-    const int slot = (threadIdx.x >> 5) * kCorrChainsPerWarp + cc;  // chain within the slice
-    const int fslot = lane < 30 ? slot : kSliceChains;
-    const int m = blockIdx.x * kSliceChains + slot;
-    const bool live = lane < 30 && slot < kSliceChains && m < M;
-    const int mm = live ? m : 0;
-    const int src_lane = min(cc * 6 + q % 3, 31);
-    const size_t stride = (size_t)M * 6;
-    auto cl_of = [&](int l) { return (int)(((n0 + ns) >> l) - (n0 >> l)); };
-
-    const T* yin = ser;  // level-l samples of this launch
-    int cl = ns;
-    for (int l = 0; l < L && cl > 0; ++l) {
-        const int k0 = l == 0 ? 0 : kP / 2;
-        T* h = hist + (((size_t)mm * L + l) * 6 + q) * 16;
-        T r[16], acc[16], acc2[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            r[i] = live ? h[i] : T(0);
-            acc[i] = T(0);
-            acc2[i] = T(0);
-        }
-        // level-(l+1) sample J is the mean of level-l samples off + 2J and
-        // off + 2J + 1 of this launch; sample -1 is the newest before it
-        const int cn = l + 1 < L ? cl_of(l + 1) : 0;
-        const int off = (int)(2 * (n0 >> (l + 1)) - (n0 >> l));  // -1 or 0
-        T* const yout = lev + (size_t)(l & 1) * lev_half;
-        T* const orow = yout + (size_t)mm * 6 + q;
-        T prev = r[15];
-        auto emit = [&](int a, T y) {
-            const int J = (a - off - 1) >> 1;
-            if (((a - off - 1) & 1) == 0 && J < cn && live) orow[(size_t)J * stride] = T(0.5) * (prev + y);
-            prev = y;
-        };
-        const T* yrow = yin + (size_t)mm * 6 + q;
-        int nr = 0;
-        if (l == 0)
-            corr_ring_products<T, 0, TT>(r, acc, acc2, [&](int j) { return yrow[(size_t)j * stride]; }, emit, cl,
-                                         src_lane, nr);
-        else
-            corr_ring_products<T, kP / 2, TT>(r, acc, acc2, [&](int j) { return yrow[(size_t)j * stride]; }, emit,
-                                              cl, src_lane, nr);
-        corr_fold_slice(acc, k0, live, fslot, q, acc64 + ((size_t)blockIdx.x * L + l) * 96, red);
-        if constexpr (TT) corr_fold_slice_tt(acc2, k0, live, fslot, q, acc64tt + ((size_t)blockIdx.x * L + l) * 48, red);
-        if (live) {
-            T nh[16];
-            corr_ring_newest(r, nr, nh);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) h[i] = nh[i];
-        }
-        yin = yout;
-        cl = cn;
-    }
-}
-
-// ------------------------------------------------------- state upload ------
-// A caller's state in the host layout (R [M][N][3], A [M][zm][3] double;
-// S [M][zm], Z [M] int32), staged on the device as it is, checked and then
-// converted to the device layout.  One thread per (chain, bead or slot i).
-// bad: bit 1 Z out of 0..zm, 2 S out of 0..N-1, 4 A not finite, 8 R not finite.
-__global__ void state_check_kernel(const double* __restrict__ R, const double* __restrict__ A,
-                                   const int32_t* __restrict__ S, const int32_t* __restrict__ Z, int M, int N,
-                                   int zm, int width, int* __restrict__ bad) {
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (long long)M * width) return;
-    const int m = (int)(id / width), i = (int)(id % width);
-    const int z = Z[m];
-    int f = 0;
-    if (i == 0 && (z < 0 || z > zm)) f |= 1;
-    if (i < N)
-        for (int d = 0; d < 3; ++d)
-            if (!isfinite(R[((size_t)m * N + i) * 3 + d])) f |= 8;
-    if (i < zm && i < z) {
-        const int sj = S[(size_t)m * zm + i];
-        if (sj < 0 || sj >= N) f |= 2;
-        for (int d = 0; d < 3; ++d)
-            if (!isfinite(A[((size_t)m * zm + i) * 3 + d])) f |= 4;
-    }
-    if (f) atomicOr(bad, f);
-}
-
-template <typename T>
-__global__ void state_convert_kernel(const double* __restrict__ Rh, const double* __restrict__ Ah,
-                                     const int32_t* __restrict__ Sh, const int32_t* __restrict__ Zh, int M, int N,
-                                     int zm, int NP, T* __restrict__ R, T* __restrict__ A, int32_t* __restrict__ S,
-                                     int32_t* __restrict__ Z) {
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (long long)M * NP) return;
-    const int m = (int)(id / NP), i = (int)(id % NP);
-    const int z = Zh[m];
-    if (i == 0) Z[m] = z;
-    for (int d = 0; d < 3; ++d) {
-        R[((size_t)m * 3 + d) * NP + i] = i < N ? T(Rh[((size_t)m * N + i) * 3 + d]) : T(0);
-        A[((size_t)m * 3 + d) * NP + i] = i < z ? T(Ah[((size_t)m * zm + i) * 3 + d]) : T(0);
-    }
-    S[(size_t)m * NP + i] = i < z ? Sh[(size_t)m * zm + i] : -1;
-}
-
-// The state in the caller's layout (R [M][N][3], A [M][zm][3] double; S
-// [M][zm] int32 with -1 for empty slots, Z [M]) from the device layout, into
-// caller-owned device arrays (any may be null).  One thread per (chain, i).
-template <typename T>
-__global__ void state_export_kernel(const T* __restrict__ R, const T* __restrict__ A, const int32_t* __restrict__ S,
-                                    const int32_t* __restrict__ Z, int M, int N, int zm, int NP, double* __restrict__ Ro,
-                                    double* __restrict__ Ao, int32_t* __restrict__ So, int32_t* __restrict__ Zo) {
-    const int width = N > zm ? N : zm;
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (long long)M * width) return;
-    const int m = (int)(id / width), i = (int)(id % width);
-    const int z = Z[m];
-    if (i == 0 && Zo) Zo[m] = z;
-    if (i < N && Ro)
-        for (int d = 0; d < 3; ++d) Ro[((size_t)m * N + i) * 3 + d] = (double)R[((size_t)m * 3 + d) * NP + i];
-    if (i < zm) {
-        const bool occ = i < z;
-        if (So) So[(size_t)m * zm + i] = occ ? S[(size_t)m * NP + i] : -1;
-        if (Ao)
-            for (int d = 0; d < 3; ++d)
-                Ao[((size_t)m * zm + i) * 3 + d] = occ ? (double)A[((size_t)m * 3 + d) * NP + i] : 0.0;
-    }
-}
-
-// Histogram of the slip-spring numbers Z of M chains: hist[z] += number of
-// chains with Z = z, z = 0..nb-1 (nb <= kMaxSlots + 1), bins per CTA in shared
-// memory.  A Z outside 0..nb-1 (never produced by the step) is counted in bin
-// nb, the overflow bin.
-__global__ void zhist_kernel(const int32_t* __restrict__ Z, int M, int nb, unsigned long long* __restrict__ hist) {
-    __shared__ unsigned int h[kMaxSlots + 2];
-    for (int i = threadIdx.x; i <= nb; i += blockDim.x) h[i] = 0u;
-    __syncthreads();
-    for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < M; m += gridDim.x * blockDim.x) {
-        const int z = Z[m];
-        atomicAdd(&h[(z >= 0 && z < nb) ? z : nb], 1u);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i <= nb; i += blockDim.x)
-        if (h[i]) atomicAdd(hist + i, (unsigned long long)h[i]);
-}
-
-// Correlator group sums from the slice sums: out[g][l][lag][ch][d] (the layout
-// of ss_corr_sums) = sum over the slices of group g, in slice order, of
-// acc64[s][l][d * 32 + ch * 16 + lag].  One thread per (g, l, cell).
-__global__ void corr_group_kernel(const double* __restrict__ acc64, int slices, int groups, int L,
-                                  double* __restrict__ out) {
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= groups * L * 96) return;
-    const int g = id / (L * 96), l = (id / 96) % L, i = id % 96;
-    const int d = i / 32, ch = (i % 32) / 16, lag = i % 16;
-    // slices of group g: s with floor(s * groups / slices) == g
-    const int s0 = (int)(((long long)g * slices + groups - 1) / groups);
-    const int s1 = (int)(((long long)(g + 1) * slices + groups - 1) / groups);
-    double sum = 0.0;
-    for (int sl = s0; sl < s1; ++sl) sum += acc64[((size_t)sl * L + l) * 96 + i];
-    out[((((size_t)g * L + l) * 16 + lag) * 2 + ch) * 3 + d] = sum;
-}
-
-// ------------------------------------------------------------ init kernel ----
-// Equilibrium initial state (Sec. 3.1 sampling): ideal-chain bonds with
-// variance kT/k_b per component, Z ~ Poisson(N/N0) by inverse CDF on a 53-bit
-// uniform (capped at z_max), S uniform on the beads, anchors Gaussian around
-// their bead with variance kT/k_s.  One thread per chain, FP64 arithmetic.
-template <typename T, int NP>
-__global__ void init_kernel(T* R, T* A, int32_t* S, int32_t* Z, int M, int N, int zmax, double sb,
-                            double sa, double lam, uint32_t key0, uint32_t key1, uint32_t chain_base) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= M) return;
-    const uint32_t cid = chain_base + (uint32_t)m;
-    double r[kMaxBeads][3];
-    r[0][0] = r[0][1] = r[0][2] = 0.0;
-    for (int i = 0; i + 1 < N; ++i) {
-        const uint4 w = philox4x32_10((uint32_t)i, 0u, kPurposeInitBond, cid, key0, key1);
-        double n[4];
-        box_muller<double>(w.x, w.y, n[0], n[1]);
-        box_muller<double>(w.z, w.w, n[2], n[3]);
-        for (int d = 0; d < 3; ++d) r[i + 1][d] = r[i][d] + sb * n[d];
-    }
-    for (int i = 0; i < NP; ++i)
-        for (int d = 0; d < 3; ++d) R[((size_t)m * 3 + d) * NP + i] = i < N ? T(r[i][d]) : T(0);
-    int z = zmax;
-    {
-        const uint4 w = philox4x32_10(0u, 0u, kPurposeInitZ, cid, key0, key1);
-        const double u53 = ((double)(w.x >> 5) * 67108864.0 + (double)(w.y >> 6)) / 9007199254740992.0;
-        double pmf = exp(-lam), cdf = pmf;
-        for (int k = 0; k < zmax; ++k) {
-            if (u53 < cdf) {
-                z = k;
-                break;
-            }
-            pmf *= lam / (double)(k + 1);
-            cdf += pmf;
-        }
-    }
-    Z[m] = z;
-    for (int j = 0; j < NP; ++j) {
-        int sj = -1;
-        double an[3] = {0.0, 0.0, 0.0};
-        if (j < z) {
-            const uint4 ws = philox4x32_10((uint32_t)j, 0u, kPurposeInitS, cid, key0, key1);
-            sj = (int)(((unsigned long long)ws.x * (unsigned long long)N) >> 32);
-            const uint4 wa = philox4x32_10((uint32_t)j, 0u, kPurposeInitA, cid, key0, key1);
-            double n[4];
-            box_muller<double>(wa.x, wa.y, n[0], n[1]);
-            box_muller<double>(wa.z, wa.w, n[2], n[3]);
-            for (int d = 0; d < 3; ++d) an[d] = r[sj][d] + sa * n[d];
-        }
-        S[(size_t)m * NP + j] = sj;
-        for (int d = 0; d < 3; ++d) A[((size_t)m * 3 + d) * NP + j] = T(an[d]);
-    }
+    const int nlog = a.log_every > 0 ? (int)((info.t0 + info.nsteps) / a.log_every - info.t0 / a.log_every) : 0;
+    // the 8 x 2 layout sums its lanes' two beads first, as its own layout
+    constexpr int VL = W == 8 && B != 2 ? 2 : 1;
+    run_chains<T, W, B, kWinOff, true, false, false, VL>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
+                                                     info.log_m0, nlog);
 }
 
 }  // namespace ssk
