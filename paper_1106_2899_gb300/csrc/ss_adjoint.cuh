@@ -381,8 +381,8 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                         const uint4 wc = philox4x32_10_rk((uint32_t)(ll + b * W), tt, kPurposeCreate, chain_id,
                                                           c.rk0, c.rk1);
                         T n3[4];
-                        box_muller<T>(wc.x, wc.y, n3[0], n3[1]);
-                        box_muller<T>(wc.z, wc.w, n3[2], n3[3]);
+                        draw_pair<T>(wc.x, wc.y, n3[0], n3[1]);
+                        draw_pair<T>(wc.z, wc.w, n3[2], n3[3]);
                         // d sqrt(kT/k_s) / d k_s = -sqrt(kT/k_s) / (2 k_s)
                         gks += -(double)c.sa / (2.0 * (double)ks) *
                                (double)(anew[b][0] * n3[0] + anew[b][1] * n3[1] + anew[b][2] * n3[2]);
@@ -456,8 +456,8 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 // noise of this bead in this step
                 const uint4 w = philox_step(ppre[b], philox_step_shared(tt, kPurposeStep, c.rk0), c.rk0, c.rk1);
                 T nrm[4];
-                box_muller<T>(w.x, w.y, nrm[0], nrm[1]);
-                box_muller<T>(w.z, w.w, nrm[2], nrm[3]);
+                draw_pair<T>(w.x, w.y, nrm[0], nrm[1]);
+                draw_pair<T>(w.z, w.w, nrm[2], nrm[3]);
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
                     T fbk = T(0), lap = T(0);  // bond force / k_b, Laplacian of the adjoint

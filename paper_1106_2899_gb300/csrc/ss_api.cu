@@ -33,15 +33,16 @@ struct Elem {
     int M = 0, N = 0, W = 16, B = 2, NP = 32, zmax = 0;
     uint32_t chain_base = 0;
     int slices = 0, groups = 0;
+    int parts = 1;            // correlator CTAs per slice
     void* R = nullptr;
     void* A = nullptr;
     int32_t* S = nullptr;
     int32_t* Z = nullptr;
     void* hist = nullptr;    // [M][L][6][16] T: newest 16 samples per correlator level and series row
-    double* acc64 = nullptr;  // [slices][L][96] FP64 sums
-    double* acc64tt = nullptr;  // [slices][L][48] FP64 sums of channel TT (optional)
+    double* acc64 = nullptr;  // [slices * parts][L][96] FP64 sums
+    double* acc64tt = nullptr;  // [slices * parts][L][48] FP64 sums of channel TT (optional)
     void* ser = nullptr;     // [ser_cap][M][6] T: stress series of one launch
-    void* lev = nullptr;     // [2][ser_cap / 2 + 1][M][6] T: correlator level samples (ping-pong)
+    void* lev = nullptr;     // [2][ser_cap / 4 + 1][M][6] T: correlator level samples (ping-pong)
     int ser_cap = 0;
     double* logs = nullptr;
     double* kap_d = nullptr;
@@ -75,7 +76,7 @@ struct ss_ctx {
     long long step = 0;
     long long nsamp = 0;
     long long log_m0 = 0;
-    unsigned long long* counters = nullptr;  // [8]
+    unsigned long long* counters = nullptr;  // [kCounterCopies][8]
     int32_t* status = nullptr;
     void* stage = nullptr;  // device staging for state uploads and correlator readout
     size_t stage_bytes = 0;
@@ -259,6 +260,8 @@ ssk::StepConst<T> step_const(const ss_ctx* c, int N) {
     }
     s.two_pref = T(2.0 * p.dt * p.kT / p.zeta_s);
     s.c2 = T(2.0 * (c->k_s / (4.0 * p.kT)) * 1.4426950408889634);
+    s.c2_f = (float)(2.0 * (c->k_s / (4.0 * p.kT)) * 1.4426950408889634);
+    s.two_pref_f = (float)(2.0 * p.dt * p.kT / p.zeta_s);
     s.hmob = T(0.5 * (p.dt / p.zeta));
     s.hdt = T(0.5 * p.dt);
     uint32_t k0 = (uint32_t)c->seed, k1 = (uint32_t)(c->seed >> 32);
@@ -272,24 +275,40 @@ ssk::StepConst<T> step_const(const ss_ctx* c, int N) {
 }
 
 // The correlator kernel of one launch: all levels over the launch's series
-// (ns rows of [M][6]); each CTA folds its slice's sums into acc64.  n0:
+// (ns rows of [M][6]); each CTA folds its chains' sums into acc64.  n0:
 // samples before the launch; lev: two level-sample buffers of lev_half
 // elements.  Returns the number of kernels launched, or -1.
+// chains: those of one FP64 sum (a part of a slice, or a whole one).
 template <typename T, bool TT>
-int corr_launches_t(const T* ser, int ns, int M, int L, long long n0, T* hist, double* acc64, double* acc64tt,
-                    T* lev, size_t lev_half, cudaStream_t st) {
-    const int grid = (M + ssk::kSliceChains - 1) / ssk::kSliceChains;
-    ssk::corr_kernel<T, TT><<<grid, ssk::kCorrThreads, 0, st>>>(ser, ns, n0, M, L, hist, lev, lev_half, acc64,
-                                                                acc64tt);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+int corr_launches_t(const T* ser, int chains, int ns, int M, int L, long long n0, T* hist, double* acc64,
+                    double* acc64tt, T* lev, size_t lev_half, cudaStream_t st) {
+    // one sum per slice: the FP32 kernel takes whole slices, the FP64 one (more
+    // registers) half of every slice at a time
+    constexpr bool whole = sizeof(T) == 4 && !TT;
+    int launched = 0;
+    const int part = std::min(chains, whole ? ssk::kSliceChains : ssk::kCorrPartChains);
+    const dim3 grid((M + chains - 1) / chains), block(ssk::corr_threads(part));
+    for (int first = 0; first < chains && first < M; first += part) {
+        if (whole && part > ssk::kCorrPartChains) {
+            if constexpr (whole)
+                ssk::corr_kernel<T, TT, ssk::kSliceChains>
+                    <<<grid, block, 0, st>>>(ser, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
+        } else {
+            ssk::corr_kernel<T, TT, ssk::kCorrPartChains>
+                <<<grid, block, 0, st>>>(ser, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
+        }
+        if (cudaGetLastError() != cudaSuccess) return -1;
+        ++launched;
+    }
+    return launched;
 }
 
 // acc64tt null: channel TT off
 template <typename T>
-int corr_launches(const T* ser, int ns, int M, int L, long long n0, T* hist, double* acc64, double* acc64tt, T* lev,
-                  size_t lev_half, cudaStream_t st) {
-    return acc64tt ? corr_launches_t<T, true>(ser, ns, M, L, n0, hist, acc64, acc64tt, lev, lev_half, st)
-                   : corr_launches_t<T, false>(ser, ns, M, L, n0, hist, acc64, nullptr, lev, lev_half, st);
+int corr_launches(const T* ser, int chains, int ns, int M, int L, long long n0, T* hist, double* acc64,
+                  double* acc64tt, T* lev, size_t lev_half, cudaStream_t st) {
+    return acc64tt ? corr_launches_t<T, true>(ser, chains, ns, M, L, n0, hist, acc64, acc64tt, lev, lev_half, st)
+                   : corr_launches_t<T, false>(ser, chains, ns, M, L, n0, hist, acc64, nullptr, lev, lev_half, st);
 }
 
 // Whether element e has a nonzero velocity gradient at any step of t0 ..
@@ -318,6 +337,7 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
     a.Z = e.Z;
     a.logs = e.logs;
     a.counters = c->counters;
+    a.cnt_mask = ssk::kCounterCopies - 1;
     a.status = c->status;
     a.kap = e.kap_d;
     a.kap_from = e.kfrom_d;
@@ -398,8 +418,8 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
     c->launches++;
     if (corr) {
         const T* ser = static_cast<const T*>(a.series) + (size_t)a.series_row0 * e.M * 6;
-        const int nl = corr_launches<T>(ser, nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
-                                        e.acc64tt, static_cast<T*>(e.lev), (size_t)(e.ser_cap / 2 + 1) * e.M * 6,
+        const int nl = corr_launches<T>(ser, ssk::corr_chains(e.M), nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
+                                        e.acc64tt, static_cast<T*>(e.lev), (size_t)(e.ser_cap / 4 + 1) * e.M * 6,
                                         c->stream);
         if (nl < 0) return fail(c, SS_ECUDA, "correlator kernel launch failed");
         c->launches += nl;
@@ -465,9 +485,11 @@ int zero_observables(ss_ctx* c) {
     for (Elem& e : c->el) {
         if (e.hist) SS_CUDA(c, cudaMemsetAsync(e.hist, 0, (size_t)e.M * c->levels * 96 * ts, c->stream));
         if (e.acc64)
-            SS_CUDA(c, cudaMemsetAsync(e.acc64, 0, (size_t)e.slices * c->levels * 96 * sizeof(double), c->stream));
+            SS_CUDA(c, cudaMemsetAsync(e.acc64, 0, (size_t)e.slices * e.parts * c->levels * 96 * sizeof(double),
+                                       c->stream));
         if (e.acc64tt)
-            SS_CUDA(c, cudaMemsetAsync(e.acc64tt, 0, (size_t)e.slices * c->levels * 48 * sizeof(double), c->stream));
+            SS_CUDA(c, cudaMemsetAsync(e.acc64tt, 0, (size_t)e.slices * e.parts * c->levels * 48 * sizeof(double),
+                                       c->stream));
         if (e.logs && c->P.max_logs > 0)
             SS_CUDA(c, cudaMemsetAsync(e.logs, 0, (size_t)c->P.max_logs * e.groups * 14 * sizeof(double),
                                        c->stream));
@@ -564,31 +586,16 @@ int check_convert_state(ss_ctx* c, Elem& e, const double* dR, const double* dA, 
     return SS_OK;
 }
 
-// channel TT per group: out[G][L][16][3]
-int group_corr_tt(ss_ctx* c, Elem& e, std::vector<double>& out) {
+// group sums [G][L][16][2][3] (W = 96) or, of channel TT, [G][L][16][3] (W = 48)
+// from the device sums of the parts, summed on the device
+template <int W>
+int group_corr(ss_ctx* c, Elem& e, const double* acc, std::vector<double>& out) {
     const int L = c->levels;
-    std::vector<double> sl((size_t)e.slices * L * 48);
-    SS_CUDA(c, cudaMemcpyAsync(sl.data(), e.acc64tt, sl.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    SS_CUDA(c, cudaStreamSynchronize(c->stream));
-    out.assign((size_t)e.groups * L * 16 * 3, 0.0);
-    for (int s = 0; s < e.slices; ++s) {
-        const int g = (int)(((long long)s * e.groups) / e.slices);
-        for (int l = 0; l < L; ++l)
-            for (int d = 0; d < 3; ++d)
-                for (int lag = 0; lag < 16; ++lag)
-                    out[(((size_t)g * L + l) * 16 + lag) * 3 + d] += sl[((size_t)s * L + l) * 48 + d * 16 + lag];
-    }
-    return SS_OK;
-}
-
-// group sums [G][L][16][2][3] from the per-slice device sums, summed on the device
-int group_corr(ss_ctx* c, Elem& e, std::vector<double>& out) {
-    const int L = c->levels;
-    const size_t n = (size_t)e.groups * L * 96;
+    const size_t n = (size_t)e.groups * L * W;
     int rc = stage_at_least(c, n * sizeof(double));
     if (rc != SS_OK) return rc;
     double* d = static_cast<double*>(c->stage);
-    ssk::corr_group_kernel<<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(e.acc64, e.slices, e.groups, L, d);
+    ssk::corr_group_kernel<W><<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(acc, e.slices, e.parts, e.groups, L, d);
     SS_CUDA(c, cudaGetLastError());
     out.resize(n);
     SS_CUDA(c, cudaMemcpyAsync(out.data(), d, n * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -639,6 +646,7 @@ ssk::ChunkArgs make_desc(const ss_ctx* c, const Elem& e) {
     a.Z = e.Z;
     a.logs = e.logs;
     a.counters = c->counters;
+    a.cnt_mask = ssk::kCounterCopies - 1;
     a.status = c->status;
     a.kap = e.kap_d;
     a.kap_from = e.kfrom_d;
@@ -762,7 +770,7 @@ int autotune(ss_ctx* c) {
                 unsigned long long* dcnt = nullptr;  // the trials count into scratch, not the context
                 if (rc == SS_OK && (cudaMalloc(&dd, sizeof(ssk::ChunkArgs)) != cudaSuccess ||
                                     cudaMalloc(&di, sizeof(int2) * t.M) != cudaSuccess ||
-                                    cudaMalloc(&dcnt, 16 * sizeof(unsigned long long)) != cudaSuccess))
+                                    cudaMalloc(&dcnt, (ssk::kCounterCopies + 1) * 8 * sizeof(unsigned long long)) != cudaSuccess))
                     rc = fail(c, SS_ENOMEM, "autotune: allocation failed");
                 const long long saved_m0 = c->log_m0;
                 const int saved_log = c->P.log_every;
@@ -782,7 +790,7 @@ int autotune(ss_ctx* c) {
                     std::vector<int2> items = make_items(one, t.W, t.B);
                     ssk::ChunkArgs desc = make_desc(c, t);
                     desc.counters = dcnt;
-                    desc.status = reinterpret_cast<int32_t*>(dcnt + 8);
+                    desc.status = reinterpret_cast<int32_t*>(dcnt + 8 * ssk::kCounterCopies);
                     const int smem = batched_smem_bytes<T>(c, k);
                     SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                     smem));
@@ -1115,12 +1123,12 @@ int ss_create(ss_ctx** out, const ss_element* elems, int n_elems, int precision,
         base += (uint32_t)e.M;
         c->el.push_back(e);
     }
-    if (cudaMalloc(&c->counters, 8 * sizeof(unsigned long long)) != cudaSuccess ||
+    if (cudaMalloc(&c->counters, ssk::kCounterCopies * 8 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMalloc(&c->status, sizeof(int32_t)) != cudaSuccess) {
         ss_destroy(c);
         return SS_ECUDA;
     }
-    cudaMemset(c->counters, 0, 8 * sizeof(unsigned long long));
+    cudaMemset(c->counters, 0, ssk::kCounterCopies * 8 * sizeof(unsigned long long));
     cudaMemset(c->status, 0, sizeof(int32_t));
     *out = c;
     return SS_OK;
@@ -1181,6 +1189,7 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
         layout_for(e.M, e.N, c->prec, p.integrator, &e.W, &e.B);
         e.slices = (e.M + ssk::kSliceChains - 1) / ssk::kSliceChains;
         e.groups = std::min(p.groups, e.slices);
+        e.parts = ssk::corr_parts(e.M);
         SS_CUDA(c, cudaMalloc(&e.R, (size_t)e.M * 3 * e.NP * ts));
         SS_CUDA(c, cudaMalloc(&e.A, (size_t)e.M * 3 * e.NP * ts));
         SS_CUDA(c, cudaMalloc(&e.S, (size_t)e.M * e.NP * sizeof(int32_t)));
@@ -1190,14 +1199,15 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
             SS_CUDA(c, cudaMalloc(&e.hist, (size_t)e.M * c->levels * 96 * ts));
             e.ser_cap = c->P.chunk_steps;
             SS_CUDA(c, cudaMalloc(&e.ser, (size_t)e.M * 6 * e.ser_cap * ts));
-            SS_CUDA(c, cudaMalloc(&e.lev, (size_t)2 * (e.ser_cap / 2 + 1) * e.M * 6 * ts));
-            SS_CUDA(c, cudaMalloc(&e.acc64, (size_t)e.slices * c->levels * 96 * sizeof(double)));
-            if (p.corr_tt) SS_CUDA(c, cudaMalloc(&e.acc64tt, (size_t)e.slices * c->levels * 48 * sizeof(double)));
+            SS_CUDA(c, cudaMalloc(&e.lev, (size_t)2 * (e.ser_cap / 4 + 1) * e.M * 6 * ts));
+            SS_CUDA(c, cudaMalloc(&e.acc64, (size_t)e.slices * e.parts * c->levels * 96 * sizeof(double)));
+            if (p.corr_tt)
+                SS_CUDA(c, cudaMalloc(&e.acc64tt, (size_t)e.slices * e.parts * c->levels * 48 * sizeof(double)));
         }
         if (p.max_logs > 0) SS_CUDA(c, cudaMalloc(&e.logs, (size_t)p.max_logs * e.groups * 14 * sizeof(double)));
         e.flow_dirty = true;
     }
-    SS_CUDA(c, cudaMemsetAsync(c->counters, 0, 8 * sizeof(unsigned long long), c->stream));
+    SS_CUDA(c, cudaMemsetAsync(c->counters, 0, ssk::kCounterCopies * 8 * sizeof(unsigned long long), c->stream));
     SS_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream));
     c->launches = 0;
     int rc = zero_observables(c);
@@ -1341,10 +1351,10 @@ int ss_correlator(ss_ctx* c, int elem, int channel, double* t, double* G, double
     if (n_out) *n_out = n_slots;
     if (cap == 0 || (!t && !G && !sem)) return SS_OK;  // a size query reads nothing from the device
     std::vector<double> acc, acc_tt;
-    int rc = group_corr(c, *e, acc);
+    int rc = group_corr<96>(c, *e, e->acc64, acc);
     if (rc != SS_OK) return rc;
     if (tt) {
-        rc = group_corr_tt(c, *e, acc_tt);
+        rc = group_corr<48>(c, *e, e->acc64tt, acc_tt);
         if (rc != SS_OK) return rc;
     }
     const std::vector<int> gsz = group_sizes(*e);
@@ -1548,7 +1558,7 @@ int ss_corr_sums(ss_ctx* c, int elem, double* acc, int* n_groups, int64_t* n_sam
     if (!e) return fail(c, SS_EINVAL, "bad element");
     if (!c->have_params || c->levels <= 0) return fail(c, SS_ESTATE, "correlator not enabled");
     std::vector<double> g;
-    int rc = group_corr(c, *e, g);
+    int rc = group_corr<96>(c, *e, e->acc64, g);
     if (rc != SS_OK) return rc;
     if (acc) std::memcpy(acc, g.data(), g.size() * sizeof(double));
     if (n_groups) *n_groups = e->groups;
@@ -1561,7 +1571,7 @@ int ss_corr_sums_tt(ss_ctx* c, int elem, double* acc_tt, int* n_groups, int64_t*
     if (!e) return fail(c, SS_EINVAL, "bad element");
     if (!c->have_params || c->levels <= 0 || !e->acc64tt) return fail(c, SS_ESTATE, "channel TT not enabled");
     std::vector<double> g;
-    int rc = group_corr_tt(c, *e, g);
+    int rc = group_corr<48>(c, *e, e->acc64tt, g);
     if (rc != SS_OK) return rc;
     if (acc_tt) std::memcpy(acc_tt, g.data(), g.size() * sizeof(double));
     if (n_groups) *n_groups = e->groups;
@@ -1590,9 +1600,11 @@ int ss_log_sums(ss_ctx* c, int elem, int64_t* log_step, double* sums, int cap, i
 
 int ss_counters(ss_ctx* c, int64_t out[8]) {
     if (!c || !out) return SS_EINVAL;
-    unsigned long long h[8] = {0};
-    SS_CUDA(c, cudaMemcpyAsync(h, c->counters, sizeof(h), cudaMemcpyDeviceToHost, c->stream));
+    unsigned long long all[ssk::kCounterCopies][8], h[8] = {0};
+    SS_CUDA(c, cudaMemcpyAsync(all, c->counters, sizeof(all), cudaMemcpyDeviceToHost, c->stream));
     SS_CUDA(c, cudaStreamSynchronize(c->stream));
+    for (const auto& copy : all)
+        for (int i = 0; i < 8; ++i) h[i] += copy[i];
     for (int i = 0; i < 5; ++i) out[i] = (int64_t)h[i];
     out[5] = c->launches;
     out[6] = (int64_t)h[6];
@@ -1842,7 +1854,7 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
         if (cudaLaunchKernel(kern, dim3((M + cpc - 1) / cpc), dim3(kThreads), args, plan.total, st) != cudaSuccess)
             return SS_ECUDA;
         if (c->levels > 0 &&
-            corr_launches<T>(static_cast<const T*>(a.series), ns, M, c->levels, done,
+            corr_launches<T>(static_cast<const T*>(a.series), ssk::kSliceChains, ns, M, c->levels, done,
                              reinterpret_cast<T*>(scr + off_hist), reinterpret_cast<double*>(scr + off_acc64), nullptr,
                              reinterpret_cast<T*>(scr + off_lev), (size_t)(ser_cap / 2 + 1) * M * 6, st) < 0)
             return SS_ECUDA;

@@ -14,238 +14,267 @@ namespace ssk {
 // y = sigma_off (AUTO channel) or (sigma + sigma^(v))_off (TOTAL channel).
 //
 // One thread per (chain, series row q): q = 0..2 are sigma_off (xy, xz, yz),
-// q = 3..5 (sigma + sigma^(v))_off; a warp holds 5 chains x 6 rows, and the
-// later value x of row q is row q % 3 of the same chain, taken by a shuffle.
-// Samples of a level are [j][M][6] arrays (the chain kernel's series for
-// level 0).  hist [M][L][6][16] keeps the newest 16 samples of every level
-// and row (oldest first, zero after a reset): the lags reach back into
-// earlier launches through a 16-entry register ring; each level's pass
-// writes its own history when it ends.  A CTA covers one slice of
-// kSliceChains chains and adds its chains' sums of this launch, in chain
-// order, to the slice's FP64 sums acc64 [slices][L][3][32] (component,
-// channel * 16 + lag).  With TT the rows of sigma + sigma^(v) also take their
-// own samples as the later value (channel TT, acc64tt [slices][L][3][16]).
-constexpr int kCorrChainsPerWarp = 5;
-constexpr int kCorrWarps = (kSliceChains + kCorrChainsPerWarp - 1) / kCorrChainsPerWarp;  // 13
-constexpr int kCorrThreads = kCorrWarps * 32;
+// q = 3..5 (sigma + sigma^(v))_off; a warp holds 5 chains x 6 rows, and the later
+// value x of row q is row q % 3 of the same chain, taken by a shuffle.  A pass takes two levels: the samples of level l stream by from
+// memory (the chain kernel's series for level 0, else what the pass below stored),
+// their pair means are the samples of level l + 1 and never leave the registers,
+// and the pair means of those are stored as the samples of level l + 2.  So the
+// sample traffic is 1.7 times the series and there are half as many passes as
+// levels.  (One level per pass moved 3 times the series through memory.)
+// hist [M][L][6][16] keeps the newest 16 samples of every level and row (oldest
+// first, zero after a reset): the lags reach back into earlier launches through a
+// 16-entry register ring.  A CTA covers one part of a slice of kSliceChains chains
+// and adds its chains' sums of this launch to the part's FP64 sums acc64
+// [parts][L][3][32] (component, channel * 16 + lag).  With TT the rows of
+// sigma + sigma^(v) also take their own samples as the later value (channel TT,
+// acc64tt [parts][L][3][16]).
 constexpr int kCorrMaxSteps = 1024;  // samples per launch (the level-sample buffers hold half)
+constexpr int kCorrPartChains = 32;  // chains per CTA at most, but for callers that keep one sum per slice
 
-// This slice's FP32 sums of one level (each thread's lags k0..15 of its row),
-// folded in chain order into FP64.
-// Channel TT of the rows q >= 3, folded the same way into out [3][16].
-// Sum of column i over the kSliceChains rows of red (row stride `stride`), in
-// chain order, in FP64.  FP32 rows go in blocks of eight: a block is summed in
-// FP32 while the rounding error of every addition is kept exactly (TwoSum,
-// Knuth) and summed beside it, then the block's sum and error are added in
-// FP64.  The result has FP64 accuracy with a quarter of the FP64 conversions
-// and additions (the FP64 pipe runs at a small fraction of the FP32 rate).
+// Chains per CTA: 32 in seven warps, or, in ensembles too small to fill the chip
+// with those, 16 in four warps, over twice the SMs.
+__host__ __device__ constexpr int corr_chains(int M) { return M >= 8192 ? 32 : 16; }
+__host__ __device__ constexpr int corr_parts(int M) {  // parts of a slice
+    return kSliceChains / corr_chains(M);
+}
+constexpr int kCorrChainsPerWarp = 5;
+__host__ __device__ constexpr int corr_threads(int chains) {
+    return (chains + kCorrChainsPerWarp - 1) / kCorrChainsPerWarp * 32;
+}
+
+// Sums of column i of red over the eight chains from c0 on, in FP64.  FP32 values
+// are summed in FP32 while the rounding error of every addition is kept exactly
+// (TwoSum, Knuth) and summed beside them.  The result has FP64 accuracy with a
+// quarter of the FP64 conversions and additions.
 template <typename T>
-__device__ __forceinline__ double slice_column_sum(const T* red, int stride, int i) {
-    static_assert(kSliceChains % 8 == 0, "blocks of eight chains");
-    double sum = 0.0;
+__device__ __forceinline__ double corr_eight_chains(const T* red, int stride, int c0, int i) {
     if constexpr (sizeof(T) == 4) {
-        for (int c0 = 0; c0 < kSliceChains; c0 += 8) {
-            float s = red[(size_t)c0 * stride + i], e = 0.0f;
+        float s = red[(size_t)c0 * stride + i], e = 0.0f;
 #pragma unroll
-            for (int c = 1; c < 8; ++c) {
-                const float x = red[(size_t)(c0 + c) * stride + i];
-                const float t = s + x;
-                const float bp = t - s;
-                e += (s - (t - bp)) + (x - bp);
-                s = t;
-            }
-            sum += (double)s;
-            sum += (double)e;
+        for (int c = 1; c < 8; ++c) {
+            const float x = red[(size_t)(c0 + c) * stride + i];
+            const float t = s + x;
+            const float bp = t - s;
+            e += (s - (t - bp)) + (x - bp);
+            s = t;
         }
+        return (double)s + (double)e;
     } else {
-        for (int c = 0; c < kSliceChains; ++c) sum += (double)red[(size_t)c * stride + i];
-    }
-    return sum;
-}
-
-template <typename T>
-__device__ __forceinline__ void corr_fold_slice_tt(const T (&acc2)[16], int k0, bool live, int slot, int q,
-                                                   double* __restrict__ out, T* red) {
-    __syncthreads();  // the first fold has read red
-    if (slot < kSliceChains && q >= 3) {
-        T* row = red + (size_t)slot * 48 + (q - 3) * kP;
+        double s = 0.0;
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-            if (k >= k0) row[k] = live ? acc2[k] : T(0);
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < 48; i += blockDim.x) {
-        if (i % kP < k0) continue;
-        out[i] += slice_column_sum(red, 48, i);
+        for (int c = 0; c < 8; ++c) s += red[(size_t)(c0 + c) * stride + i];
+        return s;
     }
 }
 
-template <typename T>
-__device__ __forceinline__ void corr_fold_slice(const T (&acc)[16], int k0, bool live, int slot, int q,
-                                                double* __restrict__ out, T* red) {
-    // red: [kSliceChains][96] T in shared memory, free once every thread is here
-    __syncthreads();
-    if (slot < kSliceChains) {
-        T* row = red + (size_t)slot * 96 + (q % 3) * kCells + (q / 3) * kP;
+// This CTA's sums of one level (each thread's lags k0..15 of its row, column col0
+// + lag of W columns), folded into out [W]; mine: this thread owns a row.
+template <typename T, int W>
+__device__ __forceinline__ void corr_fold(const T (&acc)[16], int k0, bool live, bool mine, int c, int col0, int chains,
+                                          double* __restrict__ out, T* red) {
+    __syncthreads();  // the last fold has read red
+    if (mine) {
+        T* row = red + (size_t)c * W + col0;
 #pragma unroll
         for (int k = 0; k < 16; ++k)
             if (k >= k0) row[k] = live ? acc[k] : T(0);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < 96; i += blockDim.x) {
-        const int lag = i % kP;
-        if (lag < k0) continue;
-        out[i] += slice_column_sum(red, 96, i);
+    const int tasks = W * (chains / 8);  // at most two per thread
+    double p[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        const int i = threadIdx.x + k * blockDim.x;
+        p[k] = i < tasks && i % kP >= k0 ? corr_eight_chains(red, W, i / W * 8, i % W) : 0.0;
+    }
+    __syncthreads();
+    double* part = reinterpret_cast<double*>(red);
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+        if ((int)(threadIdx.x + k * blockDim.x) < tasks) part[threadIdx.x + k * blockDim.x] = p[k];
+    __syncthreads();
+    for (int i = threadIdx.x; i < W; i += blockDim.x) {
+        if (i % kP < k0) continue;
+        double s = part[i];
+        for (int b = 1; b < chains / 8; ++b) s += part[b * W + i];
+        out[i] += s;
     }
 }
 
-// Ring of the newest 16 samples of one row: r[i] holds sample base + i - 16
-// when the next sample to enter is sample base (i.e. after a whole number of
-// 16-sample blocks).  Products of n new samples, sample j given by get(j) (a
-// load), each later value x taken from lane src_lane; emit(j, y) sees every
-// sample in order (the pair means of the level above are formed there).  nr
-// returns the ring position of the next sample (the number of samples in the
-// last partial block).  With TT, acc2 also takes the row's own sample as the
-// later value (for the rows of sigma + sigma^(v): channel TT).
-template <typename T, int K0, bool TT, typename Get, typename Emit>
-__device__ __forceinline__ void corr_ring_products(T (&r)[16], T (&acc)[16], T (&acc2)[16], Get get, Emit emit,
-                                                   int n, int src_lane, int& nr) {
-    int j = 0;
-    for (; j + 16 <= n; j += 16) {
-        T yv[16];
-#pragma unroll
-        for (int u = 0; u < 16; ++u) yv[u] = get(j + u);  // independent loads first
-#pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            emit(j + u, yv[u]);
-            const T xv = __shfl_sync(kFull, yv[u], src_lane);
-            r[u] = yv[u];
-#pragma unroll
-            for (int k = K0; k < 16; ++k) acc[k] += xv * r[(u - k) & 15];
-            if constexpr (TT) {
-#pragma unroll
-                for (int k = K0; k < 16; ++k) acc2[k] += yv[u] * r[(u - k) & 15];
-            }
-        }
-    }
-    const int rem = n - j;
-#pragma unroll
-    for (int u = 0; u < 16; ++u) {
-        if (u < rem) {
-            const T yv = get(j + u);
-            emit(j + u, yv);
-            const T xv = __shfl_sync(kFull, yv, src_lane);
-            r[u] = yv;
-#pragma unroll
-            for (int k = K0; k < 16; ++k) acc[k] += xv * r[(u - k) & 15];
-            if constexpr (TT) {
-#pragma unroll
-                for (int k = K0; k < 16; ++k) acc2[k] += yv * r[(u - k) & 15];
-            }
-        }
-    }
-    nr = rem;
-}
-
-// The newest 16 samples in ring order after `nr` samples of a partial block:
-// out[i] = r[(nr + i) & 15].
+// Sixteen samples of one row's history.
 template <typename T>
-__device__ __forceinline__ void corr_ring_newest(const T (&r)[16], int nr, T* out) {
+__device__ __forceinline__ void corr_hist_load(const T* __restrict__ h, T (&r)[16]) {
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int n = 16 / (sizeof(V) / sizeof(T));
 #pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        T v = r[0];
+    for (int i = 0; i < n; ++i) reinterpret_cast<V*>(r)[i] = reinterpret_cast<const V*>(h)[i];
+}
+// The newest 16 samples, oldest first, after n samples in the ring: r rotated left
+// by n mod 16 (four conditional rotations), stored.
+template <typename T>
+__device__ __forceinline__ void corr_hist_store(T* __restrict__ h, T (&r)[16], int n) {
 #pragma unroll
-        for (int s2 = 1; s2 < 16; ++s2)
-            if (((nr + i) & 15) == s2) v = r[s2];
-        out[i] = v;
+    for (int s = 8; s > 0; s >>= 1) {
+        if (n & s) {
+            T x[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) x[i] = r[(i + s) & 15];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) r[i] = x[i];
+        }
+    }
+    using V = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
+    constexpr int m = 16 / (sizeof(V) / sizeof(T));
+#pragma unroll
+    for (int i = 0; i < m; ++i) reinterpret_cast<V*>(h)[i] = reinterpret_cast<const V*>(r)[i];
+}
+
+// The two levels of one pass for one thread: rings (ring position of a sample: its
+// index in this launch mod 16), sums, the newest sample of each level.
+template <typename T>
+struct CorrPass {
+    alignas(16) T rA[16], rB[16];
+    T accA[16], accB[16], ttA[16], ttB[16];
+    T py, pz;
+};
+
+// Up to 32 samples of level l from sample j0 on (all 32 unless TAIL): products of
+// lags K0..15, and of lags 8..15 of the pair means.  ODD: the first sample of the
+// launch completes a pair with the newest one before it.
+template <typename T, int K0, bool ODD, bool TT, bool TAIL>
+__device__ __forceinline__ void corr_block(CorrPass<T>& s, const T* yrow, int src, size_t stride, int j0, int n,
+                                           bool has_b, bool odd_b, T* out, bool emit) {
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+        asm volatile("" ::: "memory");  // one group of loads at a time: all 32 at once would spill
+        T yv[8];
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {  // independent loads first
+            const int u = h * 8 + v;
+            if (!TAIL || u < n) yv[v] = yrow[(size_t)(j0 + u) * stride];
+        }
+#pragma unroll
+        for (int v = 0; v < 8; ++v) {
+            const int u = h * 8 + v;
+            if (!TAIL || u < n) {
+                const T y = yv[v], x = __shfl_sync(kFull, y, src);
+                s.rA[u & 15] = y;
+#pragma unroll
+                for (int k = K0; k < 16; ++k) s.accA[k] += x * s.rA[(u - k) & 15];
+                if constexpr (TT) {
+#pragma unroll
+                    for (int k = K0; k < 16; ++k) s.ttA[k] += y * s.rA[(u - k) & 15];
+                }
+                if (has_b && (u & 1) == (ODD ? 0 : 1)) {
+                    const int j = u >> 1;  // sample j0 / 2 + j of level l + 1
+                    const T z = T(0.5) * (s.py + y), zx = __shfl_sync(kFull, z, src);
+                    s.rB[j & 15] = z;
+#pragma unroll
+                    for (int k = kP / 2; k < 16; ++k) s.accB[k] += zx * s.rB[(j - k) & 15];
+                    if constexpr (TT) {
+#pragma unroll
+                        for (int k = kP / 2; k < 16; ++k) s.ttB[k] += z * s.rB[(j - k) & 15];
+                    }
+                    if (emit && (j & 1) == (odd_b ? 0 : 1)) out[(size_t)((j0 / 2 + j) >> 1) * stride] = T(0.5) * (s.pz + z);
+                    s.pz = z;
+                }
+                s.py = y;
+            }
+        }
     }
 }
 
-// All levels of one launch in one kernel.  Level l's pass reads the level-l
-// samples of this launch (the series rows for level 0, else the samples the
-// pass below stored), adds their products, and, as the samples stream by,
-// stores the pairwise means that are the level-(l+1) samples into one of the
-// ping-pong buffers lev (lev_half elements each).  A mean may pair the newest
-// level-l sample of the previous launch (the last entry of the level's
-// history) with the first new one.  Every thread reads only rows it wrote
-// itself (its chain and series row); the block synchronises only for the
-// slice folds.
-template <typename T, bool TT>
-__global__ void __launch_bounds__(kCorrThreads, (sizeof(T) == 4 && !TT) ? 2 : 1)
-    corr_kernel(const T* __restrict__ ser, int ns, long long n0, int M, int L, T* __restrict__ hist,
-                T* __restrict__ lev, size_t lev_half, double* __restrict__ acc64, double* __restrict__ acc64tt) {
-    __shared__ T red[kSliceChains * 96];
-    const int lane = threadIdx.x & 31;
-    const int cc = lane / 6, q = lane % 6;
-    const int slot = (threadIdx.x >> 5) * kCorrChainsPerWarp + cc;  // chain within the slice
-    const int fslot = lane < 30 ? slot : kSliceChains;
-    const int m = blockIdx.x * kSliceChains + slot;
-    const bool live = lane < 30 && slot < kSliceChains && m < M;
+template <typename T, int K0, bool ODD, bool TT>
+__device__ __forceinline__ void corr_levels(CorrPass<T>& s, const T* yrow, int src, size_t stride, int n,
+                                            bool has_b, bool odd_b, T* out, bool emit) {
+    int j = 0;
+    for (; j + 32 <= n; j += 32)
+        corr_block<T, K0, ODD, TT, false>(s, yrow, src, stride, j, 32, has_b, odd_b, out, emit);
+    if (j < n) corr_block<T, K0, ODD, TT, true>(s, yrow, src, stride, j, n - j, has_b, odd_b, out, emit);
+}
+
+// All levels of one launch: ns samples after n0 earlier ones.  CTA b has the
+// `chains` <= CHAINS chains from b * span + first on and the sums of part b.  lev: two buffers of lev_half elements for the samples the
+// passes store.  A pair may join the newest sample of the previous launch (the last
+// entry of the level's history) and the first new one.
+template <typename T, bool TT, int CHAINS>
+__global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT && CHAINS == kCorrPartChains ? 2 : 1)
+    corr_kernel(const T* __restrict__ ser, int chains, int first, int span, int ns, long long n0, int M, int L, T* __restrict__ hist,
+                T* lev, size_t lev_half, double* __restrict__ acc64, double* __restrict__ acc64tt) {
+    __shared__ alignas(16) T red[CHAINS * 96];
+    const int lane = threadIdx.x & 31, q = lane % 6;
+    const int c = (threadIdx.x >> 5) * kCorrChainsPerWarp + lane / 6;  // chain of this CTA
+    const bool mine = lane < 30 && c < chains;
+    const int m = blockIdx.x * span + first + c;
+    const bool live = mine && m < M;
+    const int src = min(lane / 6 * 6 + q % 3, 31);
     const int mm = live ? m : 0;
-    const int src_lane = min(cc * 6 + q % 3, 31);
     const size_t stride = (size_t)M * 6;
-    auto cl_of = [&](int l) { return (int)(((n0 + ns) >> l) - (n0 >> l)); };
+    auto count = [&](int l) { return l < L ? (int)(((n0 + ns) >> l) - (n0 >> l)) : 0; };
 
-    const T* yin = ser;  // level-l samples of this launch
-    int cl = ns;
-    for (int l = 0; l < L && cl > 0; ++l) {
-        const int k0 = l == 0 ? 0 : kP / 2;
-        T* h = hist + (((size_t)mm * L + l) * 6 + q) * 16;
-        T r[16], acc[16], acc2[16];
+    const T* yin = ser;  // samples of level l of this launch
+    for (int l = 0; l < L && count(l) > 0; l += 2) {
+        const int nA = count(l), nB = count(l + 1);
+        const bool odd_a = (n0 >> l) & 1, odd_b = (n0 >> (l + 1)) & 1;
+        T* const hA = hist + (((size_t)mm * L + l) * 6 + q) * 16;
+        T* const hB = hA + 6 * 16;
+        CorrPass<T> s;
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            r[i] = live ? h[i] : T(0);
-            acc[i] = T(0);
-            acc2[i] = T(0);
-        }
-        // level-(l+1) sample J is the mean of level-l samples off + 2J and
-        // off + 2J + 1 of this launch; sample -1 is the newest before it
-        const int cn = l + 1 < L ? cl_of(l + 1) : 0;
-        const int off = (int)(2 * (n0 >> (l + 1)) - (n0 >> l));  // -1 or 0
-        T* const yout = lev + (size_t)(l & 1) * lev_half;
-        T* const orow = yout + (size_t)mm * 6 + q;
-        T prev = r[15];
-        auto emit = [&](int a, T y) {
-            const int J = (a - off - 1) >> 1;
-            if (((a - off - 1) & 1) == 0 && J < cn && live) orow[(size_t)J * stride] = T(0.5) * (prev + y);
-            prev = y;
-        };
+        for (int i = 0; i < 16; ++i) s.accA[i] = s.accB[i] = s.ttA[i] = s.ttB[i] = s.rB[i] = T(0);
+        corr_hist_load(hA, s.rA);
+        s.py = s.rA[15];
+        if (nB > 0) corr_hist_load(hB, s.rB);
+        s.pz = s.rB[15];
+        T* const yout = lev + (size_t)((l >> 1) & 1) * lev_half;
+        T* const out = yout + (size_t)mm * 6 + q;
         const T* yrow = yin + (size_t)mm * 6 + q;
-        int nr = 0;
-        if (l == 0)
-            corr_ring_products<T, 0, TT>(r, acc, acc2, [&](int j) { return yrow[(size_t)j * stride]; }, emit, cl,
-                                         src_lane, nr);
-        else
-            corr_ring_products<T, kP / 2, TT>(r, acc, acc2, [&](int j) { return yrow[(size_t)j * stride]; }, emit,
-                                              cl, src_lane, nr);
-        corr_fold_slice(acc, k0, live, fslot, q, acc64 + ((size_t)blockIdx.x * L + l) * 96, red);
-        if constexpr (TT) corr_fold_slice_tt(acc2, k0, live, fslot, q, acc64tt + ((size_t)blockIdx.x * L + l) * 48, red);
-        if (live) {
-            T nh[16];
-            corr_ring_newest(r, nr, nh);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) h[i] = nh[i];
+        const bool emit = live && count(l + 2) > 0;
+        if (l == 0) {
+            if (odd_a)
+                corr_levels<T, 0, true, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+            else
+                corr_levels<T, 0, false, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+        } else {
+            if (odd_a)
+                corr_levels<T, kP / 2, true, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+            else
+                corr_levels<T, kP / 2, false, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
         }
-        yin = yout;
-        cl = cn;
+        double* const oA = acc64 + ((size_t)blockIdx.x * L + l) * 96;
+        const int col = (q % 3) * kCells + (q / 3) * kP;
+        corr_fold<T, 96>(s.accA, l == 0 ? 0 : kP / 2, live, mine, c, col, chains, oA, red);
+        if (nB > 0) corr_fold<T, 96>(s.accB, kP / 2, live, mine, c, col, chains, oA + 96, red);
+        if constexpr (TT) {
+            double* const oT = acc64tt + ((size_t)blockIdx.x * L + l) * 48;
+            corr_fold<T, 48>(s.ttA, l == 0 ? 0 : kP / 2, live, mine && q >= 3, c, (q - 3) * kP, chains, oT, red);
+            if (nB > 0) corr_fold<T, 48>(s.ttB, kP / 2, live, mine && q >= 3, c, (q - 3) * kP, chains, oT + 48, red);
+        }
+        if (live) {
+            corr_hist_store(hA, s.rA, nA);
+            if (nB > 0) corr_hist_store(hB, s.rB, nB);
+        }
+        yin = yout;  // each thread reads back the samples it stored
     }
 }
 
-// Correlator group sums from the slice sums: out[g][l][lag][ch][d] (the layout
-// of ss_corr_sums) = sum over the slices of group g, in slice order, of
-// acc64[s][l][d * 32 + ch * 16 + lag].  One thread per (g, l, cell).
-__global__ void corr_group_kernel(const double* __restrict__ acc64, int slices, int groups, int L,
+// Correlator group sums from the part sums, in order.  acc64 [slices * parts][L]
+// [W]: W = 96 (component * 32 + channel * 16 + lag) or 48 (channel TT: component *
+// 16 + lag); out[g][l][lag][channel][component], the layout of ss_corr_sums and
+// ss_corr_sums_tt.  Group g has the slices s with floor(s * groups / slices) = g.
+// One thread per (g, l, cell).
+template <int W>
+__global__ void corr_group_kernel(const double* __restrict__ acc64, int slices, int parts, int groups, int L,
                                   double* __restrict__ out) {
+    constexpr int CH = W / 48;
     const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= groups * L * 96) return;
-    const int g = id / (L * 96), l = (id / 96) % L, i = id % 96;
-    const int d = i / 32, ch = (i % 32) / 16, lag = i % 16;
-    // slices of group g: s with floor(s * groups / slices) == g
+    if (id >= groups * L * W) return;
+    const int g = id / (L * W), l = (id / W) % L, i = id % W;
+    const int d = i / (CH * kP), ch = (i / kP) % CH, lag = i % kP;
     const int s0 = (int)(((long long)g * slices + groups - 1) / groups);
     const int s1 = (int)(((long long)(g + 1) * slices + groups - 1) / groups);
     double sum = 0.0;
-    for (int sl = s0; sl < s1; ++sl) sum += acc64[((size_t)sl * L + l) * 96 + i];
-    out[((((size_t)g * L + l) * 16 + lag) * 2 + ch) * 3 + d] = sum;
+    for (int sl = s0 * parts; sl < s1 * parts; ++sl) sum += acc64[((size_t)sl * L + l) * W + i];
+    out[((((size_t)g * L + l) * 16 + lag) * CH + ch) * 3 + d] = sum;
 }
 
 }  // namespace ssk

@@ -22,6 +22,8 @@
 
 #include <type_traits>
 
+#include "ss_math64.cuh"
+
 namespace ssk {
 
 constexpr int kP = 16;      // multiple-tau points per level
@@ -174,6 +176,15 @@ __device__ __forceinline__ void box_muller(uint32_t wa, uint32_t wb, T& n_cos, T
     n_sin = r * s;
 }
 
+// The pair of the step and creation draws: in FP64 by the tables of ss_math64.cuh.
+template <typename T>
+__device__ __forceinline__ void draw_pair(uint32_t wa, uint32_t wb, T& n_cos, T& n_sin) {
+    if constexpr (sizeof(T) == 8)
+        box_muller_lattice(wa, wb, n_cos, n_sin);
+    else
+        box_muller<T>(wa, wb, n_cos, n_sin);
+}
+
 // 24-bit uniform in [0, 1) from the low bytes of words x, y, z
 __device__ __forceinline__ uint32_t lo24_bits(uint4 w) {
     return (w.x & 0xFFu) | ((w.y & 0xFFu) << 8) | ((w.z & 0xFFu) << 16);
@@ -232,6 +243,7 @@ struct StepConst {
     T two_pref;           // 2 dt kT / zeta_s
     T c2;                 // 2 chop log2(e): base-2 exponent per change of squared length
     T hmob, hdt;          // mob / 2, dt / 2: the stochastic Heun corrector
+    float c2_f, two_pref_f;  // c2, two_pref in FP32: the hop filter of FP64 runs
     uint32_t rk0[10], rk1[10];  // Philox round keys (key + r * Weyl increment)
 };
 
@@ -241,7 +253,11 @@ struct ChunkArgs {
     int32_t* S;         // [M][W]
     int32_t* Z;         // [M]
     double* logs;       // [max_logs][groups][14]
-    unsigned long long* counters;  // [8]: events 0..4, 6 non-finite states, 7 broken invariants
+    // [cnt_mask + 1][8]: events 0..4, 6 non-finite states, 7 broken invariants.  A CTA
+    // adds to copy blockIdx.x & cnt_mask: one copy for all would serialise the
+    // additions of a launch of few steps.
+    unsigned long long* counters;
+    int cnt_mask;
     int32_t* status;
     const double* kap;          // [n_kap][9]
     const long long* kap_from;  // [n_kap]
@@ -295,10 +311,15 @@ struct __align__(16) Pos {
 // CTA (against CTAs of four warps: 1.04-1.24x at N = 128 x 4096 chains and
 // N = 60 x 16384, 1.005x at N = 32 x 65536).
 constexpr int kChunkThreads = 32;
+constexpr int kCounterCopies = 64;  // power of two
 // Resident warps per SM the kernels are compiled for.  Two beads per lane fit 96
 // registers; three or more need 128 (N = 40, 65536 chains: 26.4 us per step at 16
-// warps, 28.8 at 20 with the spills of 96 registers).
-constexpr int chunk_warps_per_sm(int B) { return B == 1 ? 24 : (B == 2 ? 20 : 16); }
+// warps, 28.8 at 20 with the spills of 96 registers).  FP64 work is bound by the
+// FP64 pipe long before twelve warps.
+template <typename T>
+constexpr int chunk_warps_per_sm(int B) {
+    return sizeof(T) == 8 ? 12 : (B == 1 ? 24 : (B == 2 ? 20 : 16));
+}
 
 // Columns of a chain's row in device memory (R, A [3][NP], S, tape [NP]): a
 // property of the chain length alone, so layouts of fewer lanes x beads than
@@ -443,6 +464,48 @@ __device__ __forceinline__ float2 hop_prob_x2(const StepConst<float>& c, float2 
     return make_float2(fminf(w.x, 0.5f), fminf(w.y, 0.5f));
 }
 
+// An FP64 number in FP32, truncated, by integer operations; `odd` is set if it is
+// not a normal number there (zero among them).
+__device__ __forceinline__ float trunc_f32(double x, bool& odd) {
+    const unsigned hi = (unsigned)__double2hiint(x), fs = __funnelshift_l((unsigned)__double2loint(x), hi, 3);
+    odd |= (hi & 0x7fffffffu) - (897u << 20) >= (253u << 20);
+    return __uint_as_float(((fs ^ 0x40000000u) & 0x7fffffffu) | (hi & 0x80000000u));
+}
+// Hop decision of an FP64 slot in FP32 where that is certain: spring vectors to
+// the bead, the one above and the one below, the 24-bit uniform k.  With vectors
+// truncated to 23 bits a squared length is off by less than 4.2e-7 of itself, the
+// exponent by less than 6e-7 c2 (sum of two squared lengths), a probability by
+// less than 1.1e-7 two_pref times that plus 6e-7 two_pref; the margin is ten times
+// as wide.  Returns false if the uniform lies within it (about 1e-5 of all hops):
+// the FP64 probabilities then decide.  These are 70 FP64 instructions (two
+// exponentials, two divisions) of 64 cycles each.
+__device__ __forceinline__ bool hop_filter(const StepConst<double>& c, const double (&r0)[3], const double (&rp)[3],
+                                           const double (&rm)[3], bool has_up, bool has_dn, uint32_t k, bool& up,
+                                           bool& dn) {
+    bool odd = false;
+    float d[3] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const float x0 = trunc_f32(r0[i], odd), xp = trunc_f32(rp[i], odd), xm = trunc_f32(rm[i], odd);
+        d[0] = fmaf(x0, x0, d[0]);
+        d[1] = fmaf(xp, xp, d[1]);
+        d[2] = fmaf(xm, xm, d[2]);
+    }
+    float p[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        float e, r;
+        asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fminf(c.c2_f * (d[1 + i] - d[0]), 115.41560327111707f)));
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
+        p[i] = fminf(c.two_pref_f * r, 0.5f);
+    }
+    const float margin = c.two_pref_f * fmaf(c.c2_f * 1e-6f, d[0] + d[1] + d[2], 4e-6f);
+    const float u = (float)k * (1.0f / 16777216.0f), pp = has_up ? p[0] : 0.0f, ps = pp + (has_dn ? p[1] : 0.0f);
+    up = u < pp;
+    dn = !up && u < ps;
+    return !odd && fabsf(u - pp) > margin && fabsf(u - ps) > 2.0f * margin;
+}
+
 // ---------------------------------------------------------- chunk kernel ----
 // W lanes per chain, B beads per lane: bead i and slot i of a chain live on
 // lane i % W as its sub-slot i / W (NL = W*B >= N beads; slots only up to
@@ -527,6 +590,15 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     constexpr int SB = slot_sub(W, B);      // slot sub-slots
     constexpr int G8 = W / 8;               // lanes per value group after seg_reduce6
     constexpr int BP = std::is_same<T, float>::value ? B / 2 * 2 : 0;  // beads in packed FP32x2 pairs
+    // the uniform of a slot: itself in FP32, its 24 bits in FP64 (compared as integers)
+    constexpr bool INT_U = sizeof(T) == 8;
+    using U = typename std::conditional<INT_U, uint32_t, T>::type;
+    auto u_value = [](U u) -> T {
+        if constexpr (INT_U)
+            return T(u) * T(1.0 / 16777216.0);
+        else
+            return u;
+    };
     // per-bead slot masks: 32 bits cover every slot when NL <= 32
     using Mask = typename std::conditional<(NL <= 32), unsigned, unsigned long long>::type;
     const int lane = threadIdx.x & 31;
@@ -628,7 +700,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // slots, -inf elsewhere) and its stiffness in the stress (0 on empty slots); an
     // attempt dropped at the cap, counted on lane 0; and
     // the largest Z of this warp's chains (sub-slots at or above it hold no spring).
-    T thr_c[SB];
+    U thr_c[SB];
     int z_w = 0;
     bool c_drop = false;
     auto attempts_end = [&]() { return Z < a.zmax ? ((a.create_mode == 0) ? a.zmax : Z + 1) : Z; };
@@ -637,10 +709,15 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         z_w = (int)__reduce_max_sync(kFull, (unsigned)Z);
         const int c_last = attempts_end();
         const T pc2 = T(2) * c.pc[c_last - Z];
+        U thr;  // u < 2 p_c as a bound on U
+        if constexpr (INT_U)
+            thr = (U)__double2uint_ru(pc2 * 16777216.0);
+        else
+            thr = pc2;
 #pragma unroll
         for (int b = 0; b < SB; ++b) {
             const int i = ll + b * W;
-            thr_c[b] = (i >= Z && i < c_last) ? pc2 : T(0);
+            thr_c[b] = (i >= Z && i < c_last) ? thr : U(0);
         }
     };
     set_create();
@@ -799,7 +876,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // Random numbers of step tt: block (i, tt, STEP, chain) per bead/slot i.
     // They do not depend on the state, so each step draws the next step's
     // at its end, where their integer work interleaves with the stress.
-    auto draw = [&](const uint32_t tt, T (&nrm)[B][4], T (&u)[B]) {
+    auto draw = [&](const uint32_t tt, T (&nrm)[B][4], U (&u)[B]) {
         const unsigned long long p_shared = philox_step_shared(tt, kPurposeStep, c.rk0);
 #pragma unroll
         for (int b = 0; b < BP; b += 2) {
@@ -819,10 +896,13 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             if constexpr (std::is_same<T, float>::value) {  // the bead's two Box-Muller pairs packed
                 box_muller_x2(w.x, w.y, w.z, w.w, nrm[b][0], nrm[b][1], nrm[b][2], nrm[b][3]);
             } else {
-                box_muller<T>(w.x, w.y, nrm[b][0], nrm[b][1]);
-                box_muller<T>(w.z, w.w, nrm[b][2], nrm[b][3]);
+                draw_pair<T>(w.x, w.y, nrm[b][0], nrm[b][1]);
+                draw_pair<T>(w.z, w.w, nrm[b][2], nrm[b][3]);
             }
-            u[b] = uniform_lo24<T>(w);
+            if constexpr (INT_U)
+                u[b] = lo24_bits(w);
+            else
+                u[b] = uniform_lo24<T>(w);
         }
     };
     // decisions of a replayed step, loaded one step ahead
@@ -855,7 +935,8 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             }
         }
 
-        T nrm[B][4], u[B];
+        T nrm[B][4];
+        U u[B];
         draw(t, nrm, u);
         // ---- substep 1: forces at time t, Euler-Maruyama, anchor advection.
         // Forces on positions Ro (this lane's beads; the other beads from the
@@ -1118,20 +1199,29 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                     const T r0[3] = {q0.x - A[b][0], q0.y - A[b][1], q0.z - A[b][2]};
                     const T rp[3] = {qp.x - A[b][0], qp.y - A[b][1], qp.z - A[b][2]};
                     const T rm[3] = {qm.x - A[b][0], qm.y - A[b][1], qm.z - A[b][2]};
-                    const T d0 = r0[0] * r0[0] + r0[1] * r0[1] + r0[2] * r0[2];
-                    const T dp = fma(rp[2], rp[2], fma(rp[1], rp[1], rp[0] * rp[0]));
-                    const T dm = fma(rm[2], rm[2], fma(rm[1], rm[1], rm[0] * rm[0]));
-                    T pp, pm;
-                    if constexpr (std::is_same<T, float>::value) {
-                        const float2 ppm = hop_prob_x2(c, make_float2(dp, dm), d0);
-                        pp = (si < N - 1) ? ppm.x : T(0);
-                        pm = (si > 0) ? ppm.y : T(0);
+                    if constexpr (sizeof(T) == 8) {
+                        const bool sure = hop_filter(c, r0, rp, rm, si < N - 1, si > 0, u[b], up, dn);
+                        if (__any_sync(kFull, occ && !sure)) {
+                            const T d0 = r0[0] * r0[0] + r0[1] * r0[1] + r0[2] * r0[2];
+                            const T dp = rp[0] * rp[0] + rp[1] * rp[1] + rp[2] * rp[2];
+                            const T dm = rm[0] * rm[0] + rm[1] * rm[1] + rm[2] * rm[2];
+                            const T pp = (si < N - 1) ? hop_prob<T>(c, dp, d0) : T(0);
+                            const T pm = (si > 0) ? hop_prob<T>(c, dm, d0) : T(0);
+                            up = u_value(u[b]) < pp;
+                            dn = !up && u_value(u[b]) < pp + pm;
+                        }
+                        up = occ && up;
+                        dn = occ && dn;
                     } else {
-                        pp = (si < N - 1) ? hop_prob<T>(c, dp, d0) : T(0);
-                        pm = (si > 0) ? hop_prob<T>(c, dm, d0) : T(0);
+                        const T d0 = r0[0] * r0[0] + r0[1] * r0[1] + r0[2] * r0[2];
+                        const T dp = fma(rp[2], rp[2], fma(rp[1], rp[1], rp[0] * rp[0]));
+                        const T dm = fma(rm[2], rm[2], fma(rm[1], rm[1], rm[0] * rm[0]));
+                        const float2 ppm = hop_prob_x2(c, make_float2(dp, dm), d0);
+                        const T pp = (si < N - 1) ? ppm.x : T(0);
+                        const T pm = (si > 0) ? ppm.y : T(0);
+                        up = occ && (u[b] < pp);
+                        dn = occ && !up && (u[b] < pp + pm);
                     }
-                    up = occ && (u[b] < pp);
-                    dn = occ && !up && (u[b] < pp + pm);
                     if constexpr (WIN == kWinRecord) tb[b] = (up ? kTapeUp : 0) | (dn ? kTapeDown : 0);
                     S[b] = up ? si + 1 : (dn ? si - 1 : si);
 #pragma unroll
@@ -1174,7 +1264,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                     end_new[b] = !att ? -1 : ((tb[b] & kTapeNew0) ? 0 : ((tb[b] & kTapeNewN) ? N - 1 : -1));
                     gone[b] = i < Zc && (tb[b] & kTapeKillOld);
                 } else {
-                    end_new[b] = !att ? -1 : (u[b] < pc ? 0 : (u[b] < pc2 ? N - 1 : -1));
+                    end_new[b] = !att ? -1 : (u_value(u[b]) < pc ? 0 : (u_value(u[b]) < pc2 ? N - 1 : -1));
                     gone[b] = i < Zc && hit && (S[b] == 0 || S[b] == N - 1);
                 }
                 const bool made = end_new[b] >= 0;
@@ -1234,8 +1324,8 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                         const uint4 wc = philox4x32_10_rk((uint32_t)(ll + b * W), t, kPurposeCreate, chain_id, c.rk0,
                                                           c.rk1);
                         T n3[4];
-                        box_muller<T>(wc.x, wc.y, n3[0], n3[1]);
-                        box_muller<T>(wc.z, wc.w, n3[2], n3[3]);
+                        draw_pair<T>(wc.x, wc.y, n3[0], n3[1]);
+                        draw_pair<T>(wc.z, wc.w, n3[2], n3[3]);
                         SlotRec<T> r;
                         r.x = pe.x + c.sa * n3[0];
                         r.y = pe.y + c.sa * n3[1];
@@ -1454,13 +1544,14 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                 Aw[((size_t)mm * 3 + d) * NP + i] = occ ? A[b < SB ? b : 0][d] : T(0);
         }
     }
+    unsigned long long* const counters = a.counters + (blockIdx.x & a.cnt_mask) * 8;
     if (__any_sync(kFull, bad) && lane == 0) {
         atomicOr(a.status, 1);
-        atomicAdd(a.counters + 6, 1ull);
+        atomicAdd(counters + 6, 1ull);
     }
     if (__any_sync(kFull, broken) && lane == 0) {
         atomicOr(a.status, 2);
-        atomicAdd(a.counters + 7, 1ull);
+        atomicAdd(counters + 7, 1ull);
     }
 
     // ---- event counters (padding segments beyond the element's chains count nothing)
@@ -1472,7 +1563,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             unsigned x = v[k];
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kFull, x, off);
-            if (lane == 0 && x) atomicAdd(a.counters + k, (unsigned long long)x);
+            if (lane == 0 && x) atomicAdd(counters + k, (unsigned long long)x);
         }
     }
 
@@ -1499,7 +1590,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 // integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
 // be written (without one, its registers are free).
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm(B))
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
     run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, blockIdx.x * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
                                          a.nlog_chunk);
@@ -1518,7 +1609,7 @@ struct RunInfo {
 };
 
 template <typename T, int W, int B>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm(B))
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B))
     batched_kernel(const ChunkArgs* __restrict__ elems, const int2* __restrict__ items, const RunInfo info,
                    const StepConst<T> c) {
     static_assert(sizeof(ChunkArgs) % 8 == 0, "copied in 8-byte words");
