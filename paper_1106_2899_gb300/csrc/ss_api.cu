@@ -120,6 +120,8 @@ struct ss_ctx {
     bool opt_snap = false, opt_series = false, opt_corr_off = false;
     long long opt_snap_t0 = 0;
     cudaEvent_t xev = nullptr;  // orders the context's stream against a caller's stream
+    std::vector<cudaStream_t> side;  // streams beside the context's, for several elements (made on first use)
+    std::vector<cudaEvent_t> side_ev;
     std::string err;
 };
 
@@ -327,7 +329,7 @@ bool flow_in_window(const Elem& e, long long t0, int nsteps) {
 }
 
 template <typename T>
-int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
+int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps, cudaStream_t st) {
     NvtxRange range("chain kernel + correlator launch");
     const ss_params& p = c->P;
     ssk::ChunkArgs a{};
@@ -407,12 +409,12 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
     if (c->timing) {
         SS_CUDA(c, cudaEventCreate(&ev0));
         SS_CUDA(c, cudaEventCreate(&ev1));
-        SS_CUDA(c, cudaEventRecord(ev0, c->stream));
+        SS_CUDA(c, cudaEventRecord(ev0, st));
     }
     void* args[] = {(void*)&a, (void*)&sc};
-    SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, c->stream));
+    SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, st));
     if (c->timing) {
-        SS_CUDA(c, cudaEventRecord(ev1, c->stream));
+        SS_CUDA(c, cudaEventRecord(ev1, st));
         c->events.emplace_back(ev0, ev1);
     }
     c->launches++;
@@ -420,7 +422,7 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps) {
         const T* ser = static_cast<const T*>(a.series) + (size_t)a.series_row0 * e.M * 6;
         const int nl = corr_launches<T>(ser, ssk::corr_chains(e.M), nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
                                         e.acc64tt, static_cast<T*>(e.lev), (size_t)(e.ser_cap / 4 + 1) * e.M * 6,
-                                        c->stream);
+                                        st);
         if (nl < 0) return fail(c, SS_ECUDA, "correlator kernel launch failed");
         c->launches += nl;
     }
@@ -1056,7 +1058,7 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
         c->opt_snap = true;
         c->opt_corr_off = true;
         c->opt_snap_t0 = w.t_start + (long long)seg * w.ce;
-        rc = launch_chunk<T>(c, e, c->opt_snap_t0, seg_len(c, seg));
+        rc = launch_chunk<T>(c, e, c->opt_snap_t0, seg_len(c, seg), c->stream);
         c->opt_tape_mode = 0;
         c->opt_snap = false;
         c->opt_corr_off = false;
@@ -1089,6 +1091,35 @@ int order_streams(ss_ctx* c, cudaStream_t first, cudaStream_t later) {
     if (!c->xev) SS_CUDA(c, cudaEventCreateWithFlags(&c->xev, cudaEventDisableTiming));
     SS_CUDA(c, cudaEventRecord(c->xev, first));
     SS_CUDA(c, cudaStreamWaitEvent(later, c->xev, 0));
+    return SS_OK;
+}
+
+constexpr int kSideStreams = 7;    // beside the context's own
+constexpr int kSideMinSteps = 32;  // steps of a call from which several elements run side by side
+
+// Work enqueued on the first lanes - 1 side streams from now on runs after what is
+// enqueued on the context's stream.
+int fork_streams(ss_ctx* c, int lanes) {
+    if (lanes <= 1) return SS_OK;
+    while ((int)c->side.size() < lanes - 1) {
+        cudaStream_t s = nullptr;
+        cudaEvent_t ev = nullptr;
+        SS_CUDA(c, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        c->side_ev.push_back(ev);
+        SS_CUDA(c, cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking));
+        c->side.push_back(s);
+    }
+    if (!c->xev) SS_CUDA(c, cudaEventCreateWithFlags(&c->xev, cudaEventDisableTiming));
+    SS_CUDA(c, cudaEventRecord(c->xev, c->stream));
+    for (int k = 0; k < lanes - 1; ++k) SS_CUDA(c, cudaStreamWaitEvent(c->side[k], c->xev, 0));
+    return SS_OK;
+}
+// And the context's stream goes on after what is enqueued on them.
+int join_streams(ss_ctx* c, int lanes) {
+    for (int k = 0; k < lanes - 1 && k < (int)c->side.size(); ++k) {
+        SS_CUDA(c, cudaEventRecord(c->side_ev[k], c->side[k]));
+        SS_CUDA(c, cudaStreamWaitEvent(c->stream, c->side_ev[k], 0));
+    }
     return SS_OK;
 }
 }  // namespace
@@ -1288,19 +1319,29 @@ int ss_run(ss_ctx* c, int64_t n_steps) {
         if (p.integrator != SS_EULER) return fail(c, SS_EINVAL, "batched mode runs the Euler-Maruyama integrator");
         return c->prec == SS_FP64 ? batched_run<double>(c, n_steps) : batched_run<float>(c, n_steps);
     }
+    // Several elements run side by side: one after another, each would leave the
+    // SMs idle behind its last wave of CTAs (six ensembles of 4096 x 40 fill 0.84 of
+    // a wave each).  An element stays on one stream, so its launches keep their
+    // order.  Calls of a few steps are launch-bound and stay on one stream, as do
+    // runs whose launches are timed.
+    const int n_el = (int)c->el.size();
+    const int lanes = n_el > 1 && n_steps >= kSideMinSteps && !c->timing ? std::min(n_el, kSideStreams + 1) : 1;
+    int rc = fork_streams(c, lanes);
     long long left = n_steps;
-    while (left > 0) {
+    while (rc == SS_OK && left > 0) {
         const int ns = (int)std::min<long long>(left, p.chunk_steps);
-        for (Elem& e : c->el) {
-            int rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, ns)
-                                        : launch_chunk<float>(c, e, c->step, ns);
-            if (rc != SS_OK) return rc;
+        for (int i = 0; rc == SS_OK && i < n_el; ++i) {
+            const cudaStream_t st = i % lanes == 0 ? c->stream : c->side[i % lanes - 1];
+            rc = c->prec == SS_FP64 ? launch_chunk<double>(c, c->el[i], c->step, ns, st)
+                                    : launch_chunk<float>(c, c->el[i], c->step, ns, st);
         }
+        if (rc != SS_OK) break;
         c->step += ns;
         if (c->levels > 0) c->nsamp += ns;
         left -= ns;
     }
-    return SS_OK;
+    const int rj = join_streams(c, lanes);
+    return rc != SS_OK ? rc : rj;
 }
 
 int ss_stress(ss_ctx* c, int elem, double* t, double* mean, double* sem, int cap, int* n_out) {
@@ -1413,6 +1454,8 @@ int ss_destroy(ss_ctx* c) {
     if (c->status) cudaFree(c->status);
     if (c->stage) cudaFree(c->stage);
     if (c->xev) cudaEventDestroy(c->xev);
+    for (cudaStream_t s : c->side) cudaStreamDestroy(s);
+    for (cudaEvent_t ev : c->side_ev) cudaEventDestroy(ev);
     delete c;
     return SS_OK;
 }
@@ -1720,7 +1763,8 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
         c->opt_tape_mode = replay ? 2 : 1;
         c->opt_series = true;
         const int len = seg_len(c, seg);
-        rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, len) : launch_chunk<float>(c, e, c->step, len);
+        rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, len, c->stream)
+                                : launch_chunk<float>(c, e, c->step, len, c->stream);
         c->opt_tape_mode = 0;
         c->opt_series = false;
         if (rc != SS_OK) return rc;
