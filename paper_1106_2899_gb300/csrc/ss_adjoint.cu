@@ -8,10 +8,13 @@ namespace {
 template <typename T>
 const void* adjoint_fn(int W, int B) {
     switch (W * 16 + B) {
+        case 8 * 16 + 1: return (const void*)adjoint_kernel<T, 8, 1>;
+        case 8 * 16 + 3: return (const void*)adjoint_kernel<T, 8, 3>;
         case 16 * 16 + 1: return (const void*)adjoint_kernel<T, 16, 1>;
         case 16 * 16 + 2: return (const void*)adjoint_kernel<T, 16, 2>;
         case 16 * 16 + 3: return (const void*)adjoint_kernel<T, 16, 3>;
         case 16 * 16 + 4: return (const void*)adjoint_kernel<T, 16, 4>;
+        case 32 * 16 + 3: return (const void*)adjoint_kernel<T, 32, 3>;
         case 32 * 16 + 4: return (const void*)adjoint_kernel<T, 32, 4>;
         default: return nullptr;
     }

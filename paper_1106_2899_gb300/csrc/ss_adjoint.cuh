@@ -55,44 +55,94 @@ __global__ void adj_level_mean_kernel(T* __restrict__ X, T* __restrict__ Y, long
     Y[off * P + i] = T(0.5) * (Y[a] + Y[a + P]);
 }
 
-// cx_l(j), cy_l(j) for one level
-template <typename T>
+// cx_l(j), cy_l(j) of one level: lags K0..15 with weights w [16] and inv = 2^-l.
+// A thread takes kAdjBlock consecutive blocks j of one chain component and keeps
+// the window of block means it needs in registers: 2 + 30 / kAdjBlock loads per
+// block instead of 32.  (With one block per thread and the weights converted from
+// FP64 there, the conversions and a division bound level 0: 1.99 ms for 2048 steps
+// of 8192 chains.)
+constexpr int kAdjBlock = 16;
+template <typename T, int K0>
 __global__ void adj_block_sums_kernel(const T* __restrict__ X, const T* __restrict__ Y, T* __restrict__ CX,
-                                      T* __restrict__ CY, long long off, long long nl, long long P, int l,
-                                      const double* __restrict__ wgt) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= nl * P) return;
-    const long long j = i / P, p = i % P;
-    const T inv = T(1.0 / (double)(1ll << l));
-    T ax = T(0), ay = T(0);
-    for (int k = (l == 0 ? 0 : kP / 2); k < kP; ++k) {
-        const T w = T(wgt[l * kP + k]);
-        if (w == T(0)) continue;
-        if (j - k >= 0) ax += w * Y[(off + j - k) * P + p];
-        if (j + k < nl) ay += w * X[(off + j + k) * P + p];
+                                      T* __restrict__ CY, long long nl, long long P, T inv, const T* __restrict__ w) {
+    const unsigned nbp = (unsigned)((P + blockDim.x - 1) / blockDim.x), jb = blockIdx.x / nbp;
+    const long long p = (long long)(blockIdx.x - jb * nbp) * blockDim.x + threadIdx.x;
+    if (p >= P) return;
+    T wk[16];
+#pragma unroll
+    for (int k = K0; k < 16; ++k) wk[k] = w[k];
+    const long long j0 = (long long)jb * kAdjBlock;
+    // cx: earlier means Y(j - k); cy: later means X(j + k)
+    T v[kAdjBlock + 15];
+#pragma unroll
+    for (int i = 0; i < kAdjBlock + 15 - K0; ++i) {
+        const long long j = j0 - 15 + i;
+        v[i] = j >= 0 && j < nl ? Y[j * P + p] : T(0);
     }
-    CX[off * P + i] = ax * inv;
-    CY[off * P + i] = ay * inv;
+#pragma unroll
+    for (int i = 0; i < kAdjBlock; ++i) {
+        T a = T(0);
+#pragma unroll
+        for (int k = K0; k < 16; ++k)
+            if (wk[k] != T(0) && j0 + i - k >= 0) a += wk[k] * v[15 + i - k];
+        if (j0 + i < nl) CX[(j0 + i) * P + p] = a * inv;
+    }
+#pragma unroll
+    for (int i = K0; i < kAdjBlock + 15; ++i) {
+        const long long j = j0 + i;
+        v[i] = j < nl ? X[j * P + p] : T(0);
+    }
+#pragma unroll
+    for (int i = 0; i < kAdjBlock; ++i) {
+        T a = T(0);
+#pragma unroll
+        for (int k = K0; k < 16; ++k)
+            if (wk[k] != T(0) && j0 + i + k < nl) a += wk[k] * v[i + k];
+        if (j0 + i < nl) CY[(j0 + i) * P + p] = a * inv;
+    }
 }
 
-// dL/dx(t), dL/dy(t): sum over the levels whose block of t is complete
+// dL/dx(t), dL/dy(t): sum over the levels whose block of t is complete.  A thread
+// takes kAdjBlock consecutive samples of one chain component (t0 a multiple of
+// kAdjBlock), which share the blocks of the upper levels: 1 + 5 / 8 loads per
+// sample and array instead of one per level.
 template <typename T>
 __global__ void adj_sample_sums_kernel(const T* __restrict__ CX, const T* __restrict__ CY, long long n, long long P,
                                        int L, T* __restrict__ xbar, T* __restrict__ ybar) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n * P) return;
-    const long long t = i / P, p = i % P;
-    T xb = T(0), yb = T(0);
+    const unsigned nbp = (unsigned)((P + blockDim.x - 1) / blockDim.x), tb = blockIdx.x / nbp;
+    const long long p = (long long)(blockIdx.x - tb * nbp) * blockDim.x + threadIdx.x;
+    if (p >= P) return;
+    const long long t0 = (long long)tb * kAdjBlock;
+    T xb[kAdjBlock], yb[kAdjBlock];
+#pragma unroll
+    for (int i = 0; i < kAdjBlock; ++i) xb[i] = yb[i] = T(0);
     long long off = 0;
     for (int l = 0; l < L; ++l) {
-        const long long nl = n >> l, j = t >> l;
-        if (j >= nl) break;
-        xb += CX[(off + j) * P + p];
-        yb += CY[(off + j) * P + p];
+        const long long nl = n >> l;
+        if ((t0 >> l) >= nl) break;
+        const int mask = l < 4 ? (1 << l) - 1 : kAdjBlock - 1;
+        T cx = T(0), cy = T(0);
+#pragma unroll
+        for (int i = 0; i < kAdjBlock; ++i) {
+            const long long j = (t0 + i) >> l;
+            if ((i & mask) == 0) {
+                cx = j < nl ? CX[(off + j) * P + p] : T(0);
+                cy = j < nl ? CY[(off + j) * P + p] : T(0);
+            }
+            if (j < nl) {
+                xb[i] += cx;
+                yb[i] += cy;
+            }
+        }
         off += nl;
     }
-    xbar[i] = xb;  // [t][M][3]
-    ybar[i] = yb;
+#pragma unroll
+    for (int i = 0; i < kAdjBlock; ++i) {
+        if (t0 + i < n) {
+            xbar[(t0 + i) * P + p] = xb[i];  // [t][M][3]
+            ybar[(t0 + i) * P + p] = yb[i];
+        }
+    }
 }
 
 // ------------------------------------------------------- reverse sweep -----
@@ -114,11 +164,15 @@ struct AdjArgs {
 };
 
 template <typename T, int W, int B>
-__global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
+__global__ void __launch_bounds__(128, B == 1 ? 6 : 4)
     adjoint_kernel(const AdjArgs a, const StepConst<T> c) {
     constexpr int SEGS = 32 / W;
-    constexpr int NP = W * B;
-    using Mask = unsigned long long;
+    constexpr int NL = W * B;           // beads of a chain's lanes
+    constexpr int NP = row_stride(NL);  // columns of a chain's rows in device memory
+    // with eight lanes, a lane's even and odd sub-slots are two lanes of a 16-lane
+    // segment, whose FP32 gradient sums are kept apart
+    constexpr int VL = W == 8 ? 2 : 1;
+    using Mask = typename std::conditional<(NL <= 32), unsigned, unsigned long long>::type;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int seg = lane / W, ll = lane % W;
     const int cpc = (blockDim.x >> 5) * SEGS;
@@ -132,14 +186,14 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
 
     extern __shared__ __align__(16) unsigned char smem[];
     // per chain: a position table (Pos), a vector table (Pos), a slot table (SlotRec), slot masks
-    Pos<T>* pos = reinterpret_cast<Pos<T>*>(smem) + (warp * SEGS + seg) * NP;
-    Pos<T>* vec = reinterpret_cast<Pos<T>*>(smem) + (blockDim.x / 32) * 32 * B + (warp * SEGS + seg) * NP;
+    Pos<T>* pos = reinterpret_cast<Pos<T>*>(smem) + (warp * SEGS + seg) * NL;
+    Pos<T>* vec = reinterpret_cast<Pos<T>*>(smem) + (blockDim.x / 32) * 32 * B + (warp * SEGS + seg) * NL;
     SlotRec<T>* tab = reinterpret_cast<SlotRec<T>*>(reinterpret_cast<Pos<T>*>(smem) + 2 * (blockDim.x / 32) * 32 * B) +
-                      (warp * SEGS + seg) * NP;
+                      (warp * SEGS + seg) * NL;
     Mask* msk = reinterpret_cast<Mask*>(reinterpret_cast<SlotRec<T>*>(reinterpret_cast<Pos<T>*>(smem) +
                                                                       2 * (blockDim.x / 32) * 32 * B) +
                                         (blockDim.x / 32) * 32 * B) +
-                (warp * SEGS + seg) * NP;
+                (warp * SEGS + seg) * NL;
 
     const T* sR = static_cast<const T*>(a.snapR);
     const T* sA = static_cast<const T*>(a.snapA);
@@ -155,7 +209,9 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
         }
     // gradient sums: per-step parts in T, folded into FP64 every 32 steps
     double gkb = 0.0, gks = 0.0, gz = 0.0;
-    T tkb = T(0), tks = T(0), tz = T(0);
+    T tkb[VL], tks[VL], tz[VL];
+#pragma unroll
+    for (int v = 0; v < VL; ++v) tkb[v] = tks[v] = tz[v] = T(0);
     const T mu = c.mob, kb = c.k_b, ks = c.k_s;
     const double zeta = (double)c.dt / (double)c.mob;
     const double inv_zeta = 1.0 / zeta;
@@ -164,12 +220,12 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
     // per-bead slot masks of a state (springs grouped by bead, in slot order)
     auto build_masks = [&](const int (&Sx)[B], int Zx) {
 #pragma unroll
-        for (int b = 0; b < B; ++b) msk[ll + b * W] = 0ull;
+        for (int b = 0; b < B; ++b) msk[ll + b * W] = Mask(0);
         __syncwarp();
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             const int i = ll + b * W;
-            if (i < Zx) atomicOr(&msk[Sx[b]], 1ull << i);
+            if (i < Zx) atomicOr(&msk[Sx[b]], Mask(1) << i);
         }
         __syncwarp();
     };
@@ -177,30 +233,54 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
     PhiloxPre ppre[B];
 #pragma unroll
     for (int b = 0; b < B; ++b) ppre[b] = philox_pre((uint32_t)(ll + b * W), kPurposeStep, chain_id, c.rk0, c.rk1);
-    for (int t = a.ns - 1; t >= 0; --t) {
-        // ------------------------------------------ state after the step
-        T Ra[B][3], Aa[B][3];
-        int Sa[B];
-        const int Za = a.snapZ[(size_t)(t + 1) * a.M + mm];
+    // The state after a step is the state before the next one, kept from there; the
+    // state before a step, its decisions and the next stress adjoints are loaded at
+    // the top of the step and first needed after the stress part.
+    T Ra[B][3], Aa[B][3], xs[3], ys[3];
+    int Sa[B], Za;
+    auto load_state = [&](int t, T (&R)[B][3], T (&A)[B][3], int (&S)[B]) -> int {
+        const size_t row = (size_t)t * a.M + mm;
 #pragma unroll
         for (int b = 0; b < B; ++b) {
             const int i = ll + b * W;
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                Ra[b][d] = sR[(((size_t)(t + 1) * a.M + mm) * 3 + d) * NP + i];
-                Aa[b][d] = sA[(((size_t)(t + 1) * a.M + mm) * 3 + d) * NP + i];
+                R[b][d] = sR[(row * 3 + d) * NP + i];
+                A[b][d] = sA[(row * 3 + d) * NP + i];
             }
-            Sa[b] = a.snapS[((size_t)(t + 1) * a.M + mm) * NP + i];
+            S[b] = a.snapS[row * NP + i];
         }
+        return a.snapZ[row];
+    };
+    auto load_bars = [&](int t, T (&x)[3], T (&y)[3]) {
+        const size_t row = ((size_t)t * a.M + mm) * 3;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            x[d] = live ? static_cast<const T*>(a.xbar)[row + d] : T(0);
+            y[d] = live ? static_cast<const T*>(a.ybar)[row + d] : T(0);
+        }
+    };
+    if (a.ns > 0) {
+        Za = load_state(a.ns, Ra, Aa, Sa);
+        load_bars(a.ns - 1, xs, ys);
+    }
+    for (int t = a.ns - 1; t >= 0; --t) {
+        // ------------------------------------------ state before the step
+        T R0[B][3], A0[B][3];
+        int S0[B];
+        const int Z0 = load_state(t, R0, A0, S0);
+        uint8_t tb[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) tb[b] = live ? a.tape[((size_t)t * a.M + mm) * NP + ll + b * W] : (uint8_t)0;
+        T xn[3], yn[3];
+        load_bars(t > 0 ? t - 1 : 0, xn, yn);
         // ---- (1) the stress sample after the step: dL/dx, dL/dy
         {
-            const T* xb = static_cast<const T*>(a.xbar) + ((size_t)t * a.M + mm) * 3;
-            const T* yb = static_cast<const T*>(a.ybar) + ((size_t)t * a.M + mm) * 3;
             T g[3], h[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                h[d] = live ? yb[d] : T(0);
-                g[d] = (live ? xb[d] : T(0)) + h[d];  // sigma enters x and y
+                h[d] = ys[d];
+                g[d] = xs[d] + h[d];  // sigma enters x and y
             }
             __syncwarp();
 #pragma unroll
@@ -226,7 +306,7 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 v.z = kb * (g[1] * q[0] + g[2] * q[1]);
                 v.w = T(0);
                 vec[i] = v;
-                tkb += g[0] * q[0] * q[1] + g[1] * q[0] * q[2] + g[2] * q[1] * q[2];
+                tkb[b % VL] += g[0] * q[0] * q[1] + g[1] * q[0] * q[2] + g[2] * q[1] * q[2];
             }
             __syncwarp();
 #pragma unroll
@@ -265,15 +345,15 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 r.z = wz;
                 r.s = 0;
                 tab[i] = r;
-                tks += h[0] * dd[0] * dd[1] + h[1] * dd[0] * dd[2] + h[2] * dd[1] * dd[2];
+                tks[b % VL] += h[0] * dd[0] * dd[1] + h[1] * dd[0] * dd[2] + h[2] * dd[1] * dd[2];
             }
             __syncwarp();
 #pragma unroll
             for (int b = 0; b < B; ++b) {
                 Mask mb = msk[ll + b * W];
                 while (mb) {
-                    const SlotRec<T> r = tab[__ffsll((long long)mb) - 1];
-                    mb &= mb - 1ull;
+                    const SlotRec<T> r = tab[mask_ffs(mb) - 1];
+                    mb &= mb - Mask(1);
                     Rb[b][0] += r.x;
                     Rb[b][1] += r.y;
                     Rb[b][2] += r.z;
@@ -282,23 +362,6 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
             __syncwarp();
         }
 
-        // ------------------------------------------ state before the step
-        T R0[B][3], A0[B][3];
-        int S0[B];
-        const int Z0 = a.snapZ[(size_t)t * a.M + mm];
-#pragma unroll
-        for (int b = 0; b < B; ++b) {
-            const int i = ll + b * W;
-#pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                R0[b][d] = sR[(((size_t)t * a.M + mm) * 3 + d) * NP + i];
-                A0[b][d] = sA[(((size_t)t * a.M + mm) * 3 + d) * NP + i];
-            }
-            S0[b] = a.snapS[((size_t)t * a.M + mm) * NP + i];
-        }
-        uint8_t tb[B];
-#pragma unroll
-        for (int b = 0; b < B; ++b) tb[b] = live ? a.tape[((size_t)t * a.M + mm) * NP + ll + b * W] : (uint8_t)0;
         const uint32_t tt = (uint32_t)(a.t0 + t);
 
         // ---- (2) re-indexing and creation: adjoints of the springs after the
@@ -393,7 +456,7 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 for (int b = 0; b < B; ++b) {
                     const int i = ll + b * W;
                     if (i == 0 || i == N - 1) {
-                        for (int j = 0; j < NP; ++j) {
+                        for (int j = 0; j < NL; ++j) {
                             const SlotRec<T> r = tab[j];
                             if (r.s == i) {
                                 Rb[b][0] += r.x;
@@ -444,11 +507,11 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 const T xl[3] = {pl.x, pl.y, pl.z}, xr[3] = {pr.x, pr.y, pr.z};
                 // springs on this bead
                 Mask mb = msk[i];
-                const T nsp = T(__popcll(mb));
+                const T nsp = T(mask_popc(mb));
                 T asum[3] = {T(0), T(0), T(0)};
                 while (mb) {
-                    const SlotRec<T> r = tab[__ffsll((long long)mb) - 1];
-                    mb &= mb - 1ull;
+                    const SlotRec<T> r = tab[mask_ffs(mb) - 1];
+                    mb &= mb - Mask(1);
                     asum[0] += r.x;
                     asum[1] += r.y;
                     asum[2] += r.z;
@@ -475,8 +538,8 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                     if (bead) {
                         // d/dk_b of mu F_b is mu F_b / k_b; d/dzeta of the update is
                         // -(mu F + amp w / 2) / zeta
-                        tkb += mu * rb[d] * fbk;
-                        tz += rb[d] * (mu * (fb + fs) + half_amp * nrm[d]);
+                        tkb[b % VL] += mu * rb[d] * fbk;
+                        tz[b % VL] += rb[d] * (mu * (fb + fs) + half_amp * nrm[d]);
                     }
                 }
             }
@@ -490,7 +553,7 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                     Ab[b][0] += mu * ks * vs.x;
                     Ab[b][1] += mu * ks * vs.y;
                     Ab[b][2] += mu * ks * vs.z;
-                    tks += mu * (vs.x * (A0[b][0] - ps.x) + vs.y * (A0[b][1] - ps.y) + vs.z * (A0[b][2] - ps.z));
+                    tks[b % VL] += mu * (vs.x * (A0[b][0] - ps.x) + vs.y * (A0[b][1] - ps.y) + vs.z * (A0[b][2] - ps.z));
                 } else {
                     Ab[b][0] = Ab[b][1] = Ab[b][2] = T(0);
                 }
@@ -501,11 +564,29 @@ __global__ void __launch_bounds__(128, B == 1 ? 6 : 5)
                 for (int d = 0; d < 3; ++d) Rb[b][d] = Rn[b][d];
             __syncwarp();
         }
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                Ra[b][d] = R0[b][d];
+                Aa[b][d] = A0[b][d];
+            }
+            Sa[b] = S0[b];
+        }
+        Za = Z0;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            xs[d] = xn[d];
+            ys[d] = yn[d];
+        }
         if ((t & 31) == 0) {
-            gkb += (double)tkb;
-            gks += (double)tks;
-            gz -= (double)tz * inv_zeta;
-            tkb = tks = tz = T(0);
+#pragma unroll
+            for (int v = 0; v < VL; ++v) {
+                gkb += (double)tkb[v];
+                gks += (double)tks[v];
+                gz -= (double)tz[v] * inv_zeta;
+                tkb[v] = tks[v] = tz[v] = T(0);
+            }
         }
     }
     // ---- carry the adjoints to the previous segment, add this chain's gradient

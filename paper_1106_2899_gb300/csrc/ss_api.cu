@@ -97,6 +97,7 @@ struct ss_ctx {
         long long n = 0, t_start = 0;
         int ce = 0, nseg = 0;
         bool have_tape = false, forward_done = false;
+        bool complete = false;  // every buffer below is allocated
         uint8_t* tape = nullptr;
         void* series = nullptr;
         void* ckR = nullptr;  // [nseg+1] states
@@ -291,7 +292,10 @@ int corr_launches_t(const T* ser, int chains, int ns, int M, int L, long long n0
     const int part = std::min(chains, whole ? ssk::kSliceChains : ssk::kCorrPartChains);
     const dim3 grid((M + chains - 1) / chains), block(ssk::corr_threads(part));
     for (int first = 0; first < chains && first < M; first += part) {
-        if (whole && part > ssk::kCorrPartChains) {
+        if (ns == 1 && part <= ssk::kCorrPartChains) {
+            ssk::corr_step_kernel<T, TT>
+                <<<grid, block, 0, st>>>(ser, part, first, chains, n0, M, L, hist, acc64, acc64tt);
+        } else if (whole && part > ssk::kCorrPartChains) {
             if constexpr (whole)
                 ssk::corr_kernel<T, TT, ssk::kSliceChains>
                     <<<grid, block, 0, st>>>(ser, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
@@ -980,7 +984,10 @@ int launch_adjoint(ss_ctx* c, Elem& e, int seg) {
     a.destroy_new = c->P.destroy_new;
     a.create_mode = c->P.create_mode;
     a.zmax = e.zmax;
-    const int W = e.NP <= 64 ? 16 : 32, B = e.NP / W;  // snapshots and tape have the same columns in every layout
+    // (snapshots and tape have the same columns in every layout; 8 x 2 would round
+    // the sums of a gradient otherwise than 16 x 1)
+    const bool two = e.W == 8 && e.B == 2;
+    const int W = two ? 16 : e.W, B = two ? 1 : e.B;
     const int smem = kWarpsPerCta * 32 * B * (int)(2 * sizeof(ssk::Pos<T>) + sizeof(ssk::SlotRec<T>) + 8);
     const void* kern = sizeof(T) == 8 ? ssk::adjoint_fn_f64(W, B) : ssk::adjoint_fn_f32(W, B);
     if (!kern) return fail(c, SS_EINVAL, "no adjoint kernel for this layout");
@@ -1001,14 +1008,14 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
     const int L = c->levels;
     const double kT = c->P.kT;
     // weights of the later x origin products of each (level, lag) slot, TOTAL channel
-    std::vector<double> wg((size_t)L * 16, 0.0);
+    std::vector<T> wg((size_t)L * 16, T(0));
     for (int l = 0; l < L; ++l)
         for (int k = (l == 0 ? 0 : 8); k < 16; ++k) {
             const long long cnt = std::max(0ll, (w.n >> l) - k);
             if (cnt > 0 && dL_dG[l * 16 + k] != 0.0)
-                wg[(size_t)l * 16 + k] = dL_dG[l * 16 + k] / (3.0 * e.M * e.N * kT * kT * (double)cnt);
+                wg[(size_t)l * 16 + k] = T(dL_dG[l * 16 + k] / (3.0 * e.M * e.N * kT * kT * (double)cnt));
         }
-    SS_CUDA(c, cudaMemcpyAsync(w.wgt, wg.data(), sizeof(double) * wg.size(), cudaMemcpyHostToDevice, c->stream));
+    SS_CUDA(c, cudaMemcpyAsync(w.wgt, wg.data(), sizeof(T) * wg.size(), cudaMemcpyHostToDevice, c->stream));
     {
         // correlator adjoint: block means per level, per-block lag sums, per-sample sums
         const long long P = 3ll * e.M, n = w.n, cap = 2 * (n + 1) * P;
@@ -1016,6 +1023,7 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
         T* Y = X + cap;
         T* CX = Y + cap;
         T* CY = CX + cap;
+        const T* wt = reinterpret_cast<const T*>(w.wgt);
         const int thr = 256;
         auto blocks = [&](long long items) { return (unsigned)((items + thr - 1) / thr); };
         ssk::adj_level0_kernel<T><<<blocks(n * P), thr, 0, c->stream>>>(static_cast<const T*>(w.series), n, e.M, X, Y);
@@ -1030,12 +1038,20 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
                 SS_CUDA(c, cudaGetLastError());
                 c->launches++;
             }
-            ssk::adj_block_sums_kernel<T><<<blocks(nl * P), thr, 0, c->stream>>>(X, Y, CX, CY, off, nl, P, l, w.wgt);
+            const unsigned grid = blocks(P) * (unsigned)((nl + ssk::kAdjBlock - 1) / ssk::kAdjBlock);
+            if (l == 0)
+                ssk::adj_block_sums_kernel<T, 0><<<grid, thr, 0, c->stream>>>(X + off * P, Y + off * P, CX + off * P,
+                                                                              CY + off * P, nl, P, T(1), wt);
+            else
+                ssk::adj_block_sums_kernel<T, ssk::kP / 2><<<grid, thr, 0, c->stream>>>(
+                    X + off * P, Y + off * P, CX + off * P, CY + off * P, nl, P, T(1.0 / (double)(1ll << l)),
+                    wt + l * 16);
             SS_CUDA(c, cudaGetLastError());
             c->launches++;
             off += nl;
         }
-        ssk::adj_sample_sums_kernel<T><<<blocks(n * P), thr, 0, c->stream>>>(CX, CY, n, P, L,
+        ssk::adj_sample_sums_kernel<T><<<blocks(P) * (unsigned)((n + ssk::kAdjBlock - 1) / ssk::kAdjBlock), thr, 0,
+                                         c->stream>>>(CX, CY, n, P, L,
                                                                              static_cast<T*>(w.xbar),
                                                                              static_cast<T*>(w.ybar));
         SS_CUDA(c, cudaGetLastError());
@@ -1726,7 +1742,11 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
     }
     const size_t ts = tsize(c);
     const size_t stR = (size_t)e.M * 3 * e.NP * ts, stS = (size_t)e.M * e.NP * sizeof(int32_t);
-    if (!replay) {
+    // the buffers of a window of the same shape are kept (a fit evaluates one window
+    // again and again; allocating them took 5 ms of a 2048-step window of 8192 chains)
+    if (!replay && w.complete && w.n == n_steps && w.ce == checkpoint_every) {
+        w.have_tape = w.forward_done = false;
+    } else if (!replay) {
         free_window(c);
         w.n = n_steps;
         w.ce = checkpoint_every;
@@ -1748,6 +1768,7 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
         SS_CUDA(c, cudaMalloc(&w.Ab, stR));
         SS_CUDA(c, cudaMalloc(&w.grad, (size_t)e.M * 3 * sizeof(double)));
         SS_CUDA(c, cudaMalloc(&w.wgt, (size_t)c->levels * 16 * sizeof(double)));
+        w.complete = true;
     }
     // a replayed window draws the noise of the recorded one: same step indices
     if (replay) c->step = w.t_start;
@@ -1837,20 +1858,11 @@ __global__ void noalloc_reduce_kernel(const double* acc64, int slices, int L, do
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The velocity gradient of a call, by value: the launch copies it into the
-// scratch array, so nothing on the device reads caller or stack memory later.
-struct KappaVal {
-    double k[9];
-};
-__global__ void noalloc_put_kappa_kernel(const KappaVal kv, double* __restrict__ dst) {
-    if (threadIdx.x < 9) dst[threadIdx.x] = kv.k[threadIdx.x];
-}
-
 template <typename T>
 int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, int zmax, uint32_t chain_base, int64_t t0,
                      int64_t n_steps, void* R, void* A, int32_t* S, int32_t* Z, unsigned char* scr,
-                     size_t off_hist, size_t off_ser, size_t off_lev, int ser_cap, size_t off_acc64, size_t off_kap,
-                     size_t off_kfrom, size_t off_cnt, size_t off_status, bool flow, cudaStream_t st) {
+                     size_t off_hist, size_t off_ser, size_t off_lev, int ser_cap, size_t off_acc64, size_t off_cnt,
+                     int32_t* status, const double* kappa, cudaStream_t st) {
     ssk::ChunkArgs a{};
     a.R = R;
     a.A = A;
@@ -1858,10 +1870,10 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
     a.Z = Z;
     a.logs = nullptr;
     a.counters = reinterpret_cast<unsigned long long*>(scr + off_cnt);
-    a.status = reinterpret_cast<int32_t*>(scr + off_status);
-    a.kap = reinterpret_cast<const double*>(scr + off_kap);
-    a.kap_from = reinterpret_cast<const long long*>(scr + off_kfrom);
-    a.n_kap = 1;
+    a.status = status;
+    // the velocity gradient goes by value, in the kernel's arguments
+    if (kappa) std::memcpy(a.kap0, kappa, sizeof(a.kap0));
+    const bool flow = std::any_of(a.kap0, a.kap0 + 9, [](double k) { return k != 0.0; });
     a.M = M;
     a.N = N;
     a.zmax = zmax;
@@ -2005,17 +2017,15 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
     int rc = noalloc_scratch(&scr);
     if (rc != SS_OK) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    // what must start at zero: history, sums, counters, status (not the series)
-    if (cudaMemsetAsync(scr, 0, off_ser, st) != cudaSuccess) return SS_ECUDA;
-    KappaVal kv{};
-    if (kappa) std::memcpy(kv.k, kappa, sizeof(kv.k));
-    const bool flow = std::any_of(kv.k, kv.k + 9, [](double k) { return k != 0.0; });
-    noalloc_put_kappa_kernel<<<1, 32, 0, st>>>(kv, reinterpret_cast<double*>(scr + off_kap));
-    if (cudaGetLastError() != cudaSuccess) return SS_ECUDA;
+    // what must start at zero: history and sums of the correlator, the status word
+    // (the event counters are not read)
+    if (corr && cudaMemsetAsync(scr, 0, off_kap, st) != cudaSuccess) return SS_ECUDA;
+    if (status_out && cudaMemsetAsync(status_out, 0, sizeof(int32_t), st) != cudaSuccess) return SS_ECUDA;
+    int32_t* status = status_out ? status_out : reinterpret_cast<int32_t*>(scr + off_status);
     const int zm = c.el[0].zmax;
 #define SS_NOALLOC_ARGS                                                                                          \
     &c, e.W, e.B, c.P, n_chains, n_beads, zm, chain_base, t0, n_steps, R, A, S, Z, scr, off_hist, off_ser, off_lev,       \
-        ser_cap, off_acc64, off_kap, off_kfrom, off_cnt, off_status, flow, st
+        ser_cap, off_acc64, off_cnt, status, kappa, st
     rc = precision == SS_FP64 ? noalloc_launches<double>(SS_NOALLOC_ARGS) : noalloc_launches<float>(SS_NOALLOC_ARGS);
 #undef SS_NOALLOC_ARGS
     if (rc != SS_OK) return rc;
@@ -2025,8 +2035,5 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
                                                                 slices, c.levels, corr_out);
         if (cudaGetLastError() != cudaSuccess) return SS_ECUDA;
     }
-    if (status_out &&
-        cudaMemcpyAsync(status_out, scr + off_status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) != cudaSuccess)
-        return SS_ECUDA;
     return SS_OK;
 }

@@ -257,6 +257,54 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
     }
 }
 
+// The same for a launch of one step (programs that do something of their own
+// between steps): sample n0 enters level 0 and, while the level's sample completes
+// a pair, the levels above.  No sums live across samples, so 28 warps fit an SM
+// instead of 14 and nothing but the histories moves.
+template <typename T, bool TT>
+__global__ void __launch_bounds__(corr_threads(kCorrPartChains), sizeof(T) == 4 ? 4 : 2)
+    corr_step_kernel(const T* __restrict__ ser, int chains, int first, int span, long long n0, int M, int L,
+                     T* __restrict__ hist, double* __restrict__ acc64, double* __restrict__ acc64tt) {
+    __shared__ alignas(16) T red[kCorrPartChains * 96];
+    const int lane = threadIdx.x & 31, q = lane % 6;
+    const int c = (threadIdx.x >> 5) * kCorrChainsPerWarp + lane / 6;  // chain of this CTA
+    const bool mine = lane < 30 && c < chains;
+    const int m = blockIdx.x * span + first + c;
+    const bool live = mine && m < M;
+    const int src = min(lane / 6 * 6 + q % 3, 31);
+    const int mm = live ? m : 0;
+    T y = ser[(size_t)mm * 6 + q];
+    for (int l = 0; l < L; ++l) {
+        const int k0 = l == 0 ? 0 : kP / 2;
+        T* const h = hist + (((size_t)mm * L + l) * 6 + q) * 16;
+        alignas(16) T r[16];
+        corr_hist_load(h, r);
+        const T x = __shfl_sync(kFull, y, src);
+        const bool up = (n0 >> l) & 1;  // completes a pair
+        const T mean = T(0.5) * (r[15] + y);
+        T acc[16];
+        acc[0] = x * y;
+#pragma unroll
+        for (int k = 1; k < 16; ++k) acc[k] = x * r[16 - k];
+        const size_t part = (size_t)blockIdx.x * L + l;
+        corr_fold<T, 96>(acc, k0, live, mine, c, (q % 3) * kCells + (q / 3) * kP, chains, acc64 + part * 96, red);
+        if constexpr (TT) {
+            acc[0] = y * y;
+#pragma unroll
+            for (int k = 1; k < 16; ++k) acc[k] = y * r[16 - k];
+            corr_fold<T, 48>(acc, k0, live, mine && q >= 3, c, (q - 3) * kP, chains, acc64tt + part * 48, red);
+        }
+        if (live) {
+#pragma unroll
+            for (int i = 0; i < 15; ++i) r[i] = r[i + 1];
+            r[15] = y;
+            corr_hist_store(h, r, 0);
+        }
+        if (!up) break;
+        y = mean;
+    }
+}
+
 // Correlator group sums from the part sums, in order.  acc64 [slices * parts][L]
 // [W]: W = 96 (component * 32 + channel * 16 + lag) or 48 (channel TT: component *
 // 16 + lag); out[g][l][lag][channel][component], the layout of ss_corr_sums and

@@ -261,7 +261,8 @@ struct ChunkArgs {
     int32_t* status;
     const double* kap;          // [n_kap][9]
     const long long* kap_from;  // [n_kap]
-    int n_kap;
+    int n_kap;                  // 0: the constant gradient kap0
+    double kap0[9];
     int M, N, zmax, create_mode, destroy_new;
     int log_every, recenter_every;
     long long log_m0;           // logs are taken at steps m*log_every with m > log_m0
@@ -563,7 +564,8 @@ __device__ __forceinline__ KappaState kappa_at(Args& a, int ki, long long t0, in
     const double* const k = a.kap;
     const long long* const from = a.kap_from;
     while (ki + 1 < n && t0 + s >= __ldg(from + ki + 1)) ++ki;
-    const T v = lane < 9 ? T(__ldg(k + ki * 9 + lane)) : T(0);
+    T v = T(0);
+    if (lane < 9) v = n > 0 ? T(__ldg(k + ki * 9 + lane)) : T(a.kap0[lane]);
     if (lane < 9) reinterpret_cast<T*>(kap + lane / 3)[lane % 3] = v;
     KappaState r;
     r.ki = ki;
@@ -1560,9 +1562,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         if (!live) v[0] = v[1] = v[2] = v[3] = v[4] = 0u;
 #pragma unroll
         for (int k = 0; k < 5; ++k) {
-            unsigned x = v[k];
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(kFull, x, off);
+            const unsigned x = __reduce_add_sync(kFull, v[k]);
             if (lane == 0 && x) atomicAdd(counters + k, (unsigned long long)x);
         }
     }
