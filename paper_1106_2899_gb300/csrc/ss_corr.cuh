@@ -138,25 +138,49 @@ struct CorrPass {
     T py, pz;
 };
 
-// Up to 32 samples of level l from sample j0 on (all 32 unless TAIL): products of
-// lags K0..15, and of lags 8..15 of the pair means.  ODD: the first sample of the
+// Samples on their way: groups of eight are copied to shared memory three groups
+// ahead of their use (FP32), each lane its own row, by asynchronous 4-byte copies.
+// A warp then has 24 rows in flight instead of the eight its registers can hold:
+// the loads' latency bound the kernel.
+constexpr int kCorrStage = 32;  // samples of a row in shared memory
+__device__ __forceinline__ void corr_copy_group(float* st, const float* yrow, size_t stride, int j, int n) {
+#pragma unroll
+    for (int v = 0; v < 8; ++v) {
+        if (j + v < n) {
+            const unsigned dst = (unsigned)__cvta_generic_to_shared(st + ((j + v) & (kCorrStage - 1)) * 32);
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(yrow + (size_t)(j + v) * stride)
+                         : "memory");
+        }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// Up to 32 samples of level l from sample j0 on (all 32 unless TAIL) of n: products
+// of lags K0..15, and of lags 8..15 of the pair means.  ODD: the first sample of the
 // launch completes a pair with the newest one before it.
-template <typename T, int K0, bool ODD, bool TT, bool TAIL>
-__device__ __forceinline__ void corr_block(CorrPass<T>& s, const T* yrow, int src, size_t stride, int j0, int n,
+template <typename T, int K0, bool ODD, bool TT, bool TAIL, bool STAGE>
+__device__ __forceinline__ void corr_block(CorrPass<T>& s, const T* yrow, T* st, int src, size_t stride, int j0, int n,
                                            bool has_b, bool odd_b, T* out, bool emit) {
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-        asm volatile("" ::: "memory");  // one group of loads at a time: all 32 at once would spill
         T yv[8];
+        if constexpr (STAGE) {
+            if (!TAIL || j0 + h * 8 < n) {
+                corr_copy_group(st, yrow, stride, j0 + h * 8 + 24, n);
+                asm volatile("cp.async.wait_group 3;" ::: "memory");
+            }
 #pragma unroll
-        for (int v = 0; v < 8; ++v) {  // independent loads first
-            const int u = h * 8 + v;
-            if (!TAIL || u < n) yv[v] = yrow[(size_t)(j0 + u) * stride];
+            for (int v = 0; v < 8; ++v) yv[v] = st[(h * 8 + v) * 32];
+        } else {
+            asm volatile("" ::: "memory");  // one group of loads at a time: all 32 at once would spill
+#pragma unroll
+            for (int v = 0; v < 8; ++v)  // independent loads first
+                if (!TAIL || j0 + h * 8 + v < n) yv[v] = yrow[(size_t)(j0 + h * 8 + v) * stride];
         }
 #pragma unroll
         for (int v = 0; v < 8; ++v) {
             const int u = h * 8 + v;
-            if (!TAIL || u < n) {
+            if (!TAIL || j0 + u < n) {
                 const T y = yv[v], x = __shfl_sync(kFull, y, src);
                 s.rA[u & 15] = y;
 #pragma unroll
@@ -184,13 +208,18 @@ __device__ __forceinline__ void corr_block(CorrPass<T>& s, const T* yrow, int sr
     }
 }
 
-template <typename T, int K0, bool ODD, bool TT>
-__device__ __forceinline__ void corr_levels(CorrPass<T>& s, const T* yrow, int src, size_t stride, int n,
+template <typename T, int K0, bool ODD, bool TT, bool STAGE>
+__device__ __forceinline__ void corr_levels(CorrPass<T>& s, const T* yrow, T* st, int src, size_t stride, int n,
                                             bool has_b, bool odd_b, T* out, bool emit) {
+    if constexpr (STAGE) {
+#pragma unroll
+        for (int g = 0; g < 3; ++g) corr_copy_group(st, yrow, stride, 8 * g, n);
+    }
     int j = 0;
     for (; j + 32 <= n; j += 32)
-        corr_block<T, K0, ODD, TT, false>(s, yrow, src, stride, j, 32, has_b, odd_b, out, emit);
-    if (j < n) corr_block<T, K0, ODD, TT, true>(s, yrow, src, stride, j, n - j, has_b, odd_b, out, emit);
+        corr_block<T, K0, ODD, TT, false, STAGE>(s, yrow, st, src, stride, j, n, has_b, odd_b, out, emit);
+    if (j < n) corr_block<T, K0, ODD, TT, true, STAGE>(s, yrow, st, src, stride, j, n, has_b, odd_b, out, emit);
+    if constexpr (STAGE) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // All levels of one launch: ns samples after n0 earlier ones.  CTA b has the
@@ -201,7 +230,9 @@ template <typename T, bool TT, int CHAINS>
 __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT && CHAINS == kCorrPartChains ? 2 : 1)
     corr_kernel(const T* __restrict__ ser, int chains, int first, int span, int ns, long long n0, int M, int L, T* __restrict__ hist,
                 T* lev, size_t lev_half, double* __restrict__ acc64, double* __restrict__ acc64tt) {
+    constexpr bool STAGE = sizeof(T) == 4 && CHAINS == kCorrPartChains;
     __shared__ alignas(16) T red[CHAINS * 96];
+    __shared__ T stage[STAGE ? corr_threads(CHAINS) * kCorrStage : 1];
     const int lane = threadIdx.x & 31, q = lane % 6;
     const int c = (threadIdx.x >> 5) * kCorrChainsPerWarp + lane / 6;  // chain of this CTA
     const bool mine = lane < 30 && c < chains;
@@ -209,6 +240,7 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
     const bool live = mine && m < M;
     const int src = min(lane / 6 * 6 + q % 3, 31);
     const int mm = live ? m : 0;
+    T* const st = stage + (STAGE ? (threadIdx.x >> 5) * kCorrStage * 32 + lane : 0);
     const size_t stride = (size_t)M * 6;
     auto count = [&](int l) { return l < L ? (int)(((n0 + ns) >> l) - (n0 >> l)) : 0; };
 
@@ -231,14 +263,14 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
         const bool emit = live && count(l + 2) > 0;
         if (l == 0) {
             if (odd_a)
-                corr_levels<T, 0, true, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+                corr_levels<T, 0, true, TT, STAGE>(s, yrow, st, src, stride, nA, nB > 0, odd_b, out, emit);
             else
-                corr_levels<T, 0, false, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+                corr_levels<T, 0, false, TT, STAGE>(s, yrow, st, src, stride, nA, nB > 0, odd_b, out, emit);
         } else {
             if (odd_a)
-                corr_levels<T, kP / 2, true, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+                corr_levels<T, kP / 2, true, TT, STAGE>(s, yrow, st, src, stride, nA, nB > 0, odd_b, out, emit);
             else
-                corr_levels<T, kP / 2, false, TT>(s, yrow, src, stride, nA, nB > 0, odd_b, out, emit);
+                corr_levels<T, kP / 2, false, TT, STAGE>(s, yrow, st, src, stride, nA, nB > 0, odd_b, out, emit);
         }
         double* const oA = acc64 + ((size_t)blockIdx.x * L + l) * 96;
         const int col = (q % 3) * kCells + (q / 3) * kP;
