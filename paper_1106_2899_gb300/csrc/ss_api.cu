@@ -44,7 +44,7 @@ struct Elem {
     void* ser = nullptr;     // [ser_cap][M][6] T: stress series of one launch
     void* lev = nullptr;     // [2][ser_cap / 4 + 1][M][6] T: correlator level samples (ping-pong)
     int ser_cap = 0;
-    double* logs = nullptr;
+    double* logs = nullptr;  // in the context's block
     double* kap_d = nullptr;
     long long* kfrom_d = nullptr;
     int n_kap_d = 0;
@@ -66,6 +66,7 @@ struct BatchedClass {
 struct ss_ctx {
     cudaStream_t stream = nullptr;
     int prec = SS_FP32;
+    int sms = 1;  // of the device
     uint64_t seed = 0;
     std::vector<Elem> el;
     ss_params P{};
@@ -78,6 +79,11 @@ struct ss_ctx {
     long long log_m0 = 0;
     unsigned long long* counters = nullptr;  // [kCounterCopies][8]
     int32_t* status = nullptr;
+    // stress logs of all elements, one block [element][max_logs][groups][14]
+    double* logs = nullptr;
+    size_t logs_n = 0;
+    std::vector<double> logs_host;  // what the last read copied back
+    bool logs_read = false;         // logs_host holds the whole block as it is now
     void* stage = nullptr;  // device staging for state uploads and correlator readout
     size_t stage_bytes = 0;
     long long launches = 0;
@@ -166,7 +172,7 @@ int stage_at_least(ss_ctx* c, size_t bytes) {
 }
 
 void free_elem(Elem& e) {
-    void* ptrs[] = {e.R, e.A, e.S, e.Z, e.hist, e.acc64, e.acc64tt, e.ser, e.lev, e.logs, e.kap_d, e.kfrom_d};
+    void* ptrs[] = {e.R, e.A, e.S, e.Z, e.hist, e.acc64, e.acc64tt, e.ser, e.lev, e.kap_d, e.kfrom_d};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     e.R = e.A = e.hist = e.ser = e.lev = nullptr;
@@ -175,6 +181,33 @@ void free_elem(Elem& e) {
     e.acc64 = e.acc64tt = e.logs = e.kap_d = nullptr;
     e.kfrom_d = nullptr;
     e.n_kap_d = 0;
+}
+
+void free_logs(ss_ctx* c) {
+    if (c->logs) cudaFree(c->logs);
+    c->logs = nullptr;
+    c->logs_n = 0;
+    c->logs_read = false;
+    for (Elem& e : c->el) e.logs = nullptr;
+}
+
+// The first n stress logs of an element on the host.  The logs of several elements
+// are usually read one after another, so a block of up to kLogBlockBytes comes over
+// in one copy and stays until the next run or reset (512 elements: 512 copies and
+// synchronisations took 7 ms).
+constexpr size_t kLogBlockBytes = 4 << 20;
+int read_logs(ss_ctx* c, const Elem& e, int n, const double** out) {
+    const bool all = c->el.size() > 1 && c->logs_n * sizeof(double) <= kLogBlockBytes;
+    const size_t first = (size_t)(e.logs - c->logs), count = (size_t)n * e.groups * 14;
+    if (!all || !c->logs_read) {
+        c->logs_host.resize(all ? c->logs_n : count);
+        SS_CUDA(c, cudaMemcpyAsync(c->logs_host.data(), all ? c->logs : e.logs, c->logs_host.size() * sizeof(double),
+                                   cudaMemcpyDeviceToHost, c->stream));
+        SS_CUDA(c, cudaStreamSynchronize(c->stream));
+        c->logs_read = all;
+    }
+    *out = c->logs_host.data() + (all ? first : 0);
+    return SS_OK;
 }
 
 // Chain layout for N beads: W lanes per chain, B beads per lane (W*B >= N).  Every
@@ -277,31 +310,33 @@ ssk::StepConst<T> step_const(const ss_ctx* c, int N) {
     return s;
 }
 
-// The correlator kernel of one launch: all levels over the launch's series
+// The correlator kernel of one launch: all levels over the launch's series of the
+// chains m0 (a multiple of kSliceChains) .. m1 - 1
 // (ns rows of [M][6]); each CTA folds its chains' sums into acc64.  n0:
 // samples before the launch; lev: two level-sample buffers of lev_half
 // elements.  Returns the number of kernels launched, or -1.
 // chains: those of one FP64 sum (a part of a slice, or a whole one).
 template <typename T, bool TT>
-int corr_launches_t(const T* ser, int chains, int ns, int M, int L, long long n0, T* hist, double* acc64,
-                    double* acc64tt, T* lev, size_t lev_half, cudaStream_t st) {
+int corr_launches_t(const T* ser, int m0, int m1, int chains, int ns, int M, int L, long long n0, T* hist,
+                    double* acc64, double* acc64tt, T* lev, size_t lev_half, cudaStream_t st) {
     // one sum per slice: the FP32 kernel takes whole slices, the FP64 one (more
     // registers) half of every slice at a time
     constexpr bool whole = sizeof(T) == 4 && !TT;
     int launched = 0;
     const int part = std::min(chains, whole ? ssk::kSliceChains : ssk::kCorrPartChains);
-    const dim3 grid((M + chains - 1) / chains), block(ssk::corr_threads(part));
-    for (int first = 0; first < chains && first < M; first += part) {
+    const int b0 = m0 / chains;
+    const dim3 grid((m1 - m0 + chains - 1) / chains), block(ssk::corr_threads(part));
+    for (int first = 0; first < chains && m0 + first < m1; first += part) {
         if (ns == 1 && part <= ssk::kCorrPartChains) {
             ssk::corr_step_kernel<T, TT>
-                <<<grid, block, 0, st>>>(ser, part, first, chains, n0, M, L, hist, acc64, acc64tt);
+                <<<grid, block, 0, st>>>(ser, b0, part, first, chains, n0, M, L, hist, acc64, acc64tt);
         } else if (whole && part > ssk::kCorrPartChains) {
             if constexpr (whole)
                 ssk::corr_kernel<T, TT, ssk::kSliceChains>
-                    <<<grid, block, 0, st>>>(ser, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
+                    <<<grid, block, 0, st>>>(ser, b0, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
         } else {
             ssk::corr_kernel<T, TT, ssk::kCorrPartChains>
-                <<<grid, block, 0, st>>>(ser, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
+                <<<grid, block, 0, st>>>(ser, b0, part, first, chains, ns, n0, M, L, hist, lev, lev_half, acc64, acc64tt);
         }
         if (cudaGetLastError() != cudaSuccess) return -1;
         ++launched;
@@ -311,10 +346,10 @@ int corr_launches_t(const T* ser, int chains, int ns, int M, int L, long long n0
 
 // acc64tt null: channel TT off
 template <typename T>
-int corr_launches(const T* ser, int chains, int ns, int M, int L, long long n0, T* hist, double* acc64,
+int corr_launches(const T* ser, int m0, int m1, int chains, int ns, int M, int L, long long n0, T* hist, double* acc64,
                   double* acc64tt, T* lev, size_t lev_half, cudaStream_t st) {
-    return acc64tt ? corr_launches_t<T, true>(ser, chains, ns, M, L, n0, hist, acc64, acc64tt, lev, lev_half, st)
-                   : corr_launches_t<T, false>(ser, chains, ns, M, L, n0, hist, acc64, nullptr, lev, lev_half, st);
+    return acc64tt ? corr_launches_t<T, true>(ser, m0, m1, chains, ns, M, L, n0, hist, acc64, acc64tt, lev, lev_half, st)
+                   : corr_launches_t<T, false>(ser, m0, m1, chains, ns, M, L, n0, hist, acc64, nullptr, lev, lev_half, st);
 }
 
 // Whether element e has a nonzero velocity gradient at any step of t0 ..
@@ -333,7 +368,7 @@ bool flow_in_window(const Elem& e, long long t0, int nsteps) {
 }
 
 template <typename T>
-int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps, cudaStream_t st) {
+int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, cudaStream_t st) {
     NvtxRange range("chain kernel + correlator launch");
     const ss_params& p = c->P;
     ssk::ChunkArgs a{};
@@ -408,7 +443,8 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps, cudaStream_t st) 
     if (plan.total > 48 * 1024)
         SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total));
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
-    const int cpc = chains_per_cta(e.W), ctas = (e.M + cpc - 1) / cpc;
+    const int cpc = chains_per_cta(e.W), ctas = (m1 - m0 + cpc - 1) / cpc;
+    a.cta0 = m0 / cpc;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     if (c->timing) {
         SS_CUDA(c, cudaEventCreate(&ev0));
@@ -424,7 +460,7 @@ int launch_chunk(ss_ctx* c, Elem& e, long long t0, int nsteps, cudaStream_t st) 
     c->launches++;
     if (corr) {
         const T* ser = static_cast<const T*>(a.series) + (size_t)a.series_row0 * e.M * 6;
-        const int nl = corr_launches<T>(ser, ssk::corr_chains(e.M), nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
+        const int nl = corr_launches<T>(ser, m0, m1, ssk::corr_chains(e.M), nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
                                         e.acc64tt, static_cast<T*>(e.lev), (size_t)(e.ser_cap / 4 + 1) * e.M * 6,
                                         st);
         if (nl < 0) return fail(c, SS_ECUDA, "correlator kernel launch failed");
@@ -496,10 +532,9 @@ int zero_observables(ss_ctx* c) {
         if (e.acc64tt)
             SS_CUDA(c, cudaMemsetAsync(e.acc64tt, 0, (size_t)e.slices * e.parts * c->levels * 48 * sizeof(double),
                                        c->stream));
-        if (e.logs && c->P.max_logs > 0)
-            SS_CUDA(c, cudaMemsetAsync(e.logs, 0, (size_t)c->P.max_logs * e.groups * 14 * sizeof(double),
-                                       c->stream));
     }
+    if (c->logs) SS_CUDA(c, cudaMemsetAsync(c->logs, 0, c->logs_n * sizeof(double), c->stream));
+    c->logs_read = false;
     c->nsamp = 0;
     c->log_m0 = c->P.log_every > 0 ? c->step / c->P.log_every : 0;
     return SS_OK;
@@ -1074,7 +1109,7 @@ int window_backward_t(ss_ctx* c, const double* dL_dG, double grad[3]) {
         c->opt_snap = true;
         c->opt_corr_off = true;
         c->opt_snap_t0 = w.t_start + (long long)seg * w.ce;
-        rc = launch_chunk<T>(c, e, c->opt_snap_t0, seg_len(c, seg), c->stream);
+        rc = launch_chunk<T>(c, e, 0, e.M, c->opt_snap_t0, seg_len(c, seg), c->stream);
         c->opt_tape_mode = 0;
         c->opt_snap = false;
         c->opt_corr_off = false;
@@ -1111,6 +1146,18 @@ int order_streams(ss_ctx* c, cudaStream_t first, cudaStream_t later) {
 }
 
 constexpr int kSideStreams = 7;    // beside the context's own
+// Parts of one element's chains that run side by side: for runs long enough to pay
+// for the launches (256 steps), of more warps than the chip holds at once.  Four
+// parts fill the last wave best (16384 x 8: 4.49 -> 4.02 ms, two parts 4.20; 4096 x
+// 80: 7.41 -> 6.74, 6.72); from eight waves on the tail is small and two parts let
+// the correlator overlap (65536 x 32: 34.7 -> 34.4 ms, four parts 34.6).
+int run_parts(const ss_ctx* c, const Elem& e, long long n_steps) {
+    const int per_sm = c->prec == SS_FP64 ? ssk::chunk_warps_per_sm<double>(e.B) : ssk::chunk_warps_per_sm<float>(e.B);
+    const long long warps = ((long long)e.M * e.W + 31) / 32, slots = (long long)per_sm * c->sms;
+    if (n_steps < 256 || warps <= slots) return 1;
+    return std::min(e.slices, warps < 8 * slots ? 4 : 2);
+}
+
 constexpr int kSideMinSteps = 32;  // steps of a call from which several elements run side by side
 
 // Work enqueued on the first lanes - 1 side streams from now on runs after what is
@@ -1175,6 +1222,12 @@ int ss_create(ss_ctx** out, const ss_element* elems, int n_elems, int precision,
         ss_destroy(c);
         return SS_ECUDA;
     }
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        ss_destroy(c);
+        return SS_ECUDA;
+    }
     cudaMemset(c->counters, 0, ssk::kCounterCopies * 8 * sizeof(unsigned long long));
     cudaMemset(c->status, 0, sizeof(int32_t));
     *out = c;
@@ -1219,6 +1272,7 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
     }
     if (c->counters) cudaStreamSynchronize(c->stream);
     for (Elem& e : c->el) free_elem(e);
+    free_logs(c);
     free_batched(c);
     free_window(c);
     c->P = p;
@@ -1251,8 +1305,16 @@ int ss_set_params(ss_ctx* c, const ss_params* pin) {
             if (p.corr_tt)
                 SS_CUDA(c, cudaMalloc(&e.acc64tt, (size_t)e.slices * e.parts * c->levels * 48 * sizeof(double)));
         }
-        if (p.max_logs > 0) SS_CUDA(c, cudaMalloc(&e.logs, (size_t)p.max_logs * e.groups * 14 * sizeof(double)));
         e.flow_dirty = true;
+    }
+    if (p.max_logs > 0) {
+        for (const Elem& e : c->el) c->logs_n += (size_t)p.max_logs * e.groups * 14;
+        SS_CUDA(c, cudaMalloc(&c->logs, c->logs_n * sizeof(double)));
+        size_t off = 0;
+        for (Elem& e : c->el) {
+            e.logs = c->logs + off;
+            off += (size_t)p.max_logs * e.groups * 14;
+        }
     }
     SS_CUDA(c, cudaMemsetAsync(c->counters, 0, ssk::kCounterCopies * 8 * sizeof(unsigned long long), c->stream));
     SS_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(int32_t), c->stream));
@@ -1319,6 +1381,7 @@ int ss_run(ss_ctx* c, int64_t n_steps) {
         const long long nlog = (c->step + n_steps) / p.log_every - c->log_m0;
         if (nlog > p.max_logs) return fail(c, SS_EINVAL, "stress log capacity (max_logs) exceeded");
     }
+    c->logs_read = false;
     for (Elem& e : c->el) {
         int rc = upload_flow(c, e);
         if (rc != SS_OK) return rc;
@@ -1335,21 +1398,38 @@ int ss_run(ss_ctx* c, int64_t n_steps) {
         if (p.integrator != SS_EULER) return fail(c, SS_EINVAL, "batched mode runs the Euler-Maruyama integrator");
         return c->prec == SS_FP64 ? batched_run<double>(c, n_steps) : batched_run<float>(c, n_steps);
     }
-    // Several elements run side by side: one after another, each would leave the
-    // SMs idle behind its last wave of CTAs (six ensembles of 4096 x 40 fill 0.84 of
-    // a wave each).  An element stays on one stream, so its launches keep their
-    // order.  Calls of a few steps are launch-bound and stay on one stream, as do
-    // runs whose launches are timed.
-    const int n_el = (int)c->el.size();
-    const int lanes = n_el > 1 && n_steps >= kSideMinSteps && !c->timing ? std::min(n_el, kSideStreams + 1) : 1;
+    // Several elements run side by side, and so do parts of a large one: one after
+    // another, launches leave the SMs idle behind their last wave of CTAs (six
+    // ensembles of 4096 x 40 fill 0.84 of a wave each, 16384 x 8 1.12), and the
+    // correlator, bound by memory, would run alone instead of beside the chain
+    // kernel.  A unit of work stays on one stream, so its launches keep their order.
+    // Calls of a few steps are launch-bound and stay on one stream, as do runs whose
+    // launches are timed.
+    struct Unit {
+        Elem* e;
+        int m0, m1;
+    };
+    std::vector<Unit> units;
+    const bool side = n_steps >= kSideMinSteps && !c->timing;
+    for (Elem& e : c->el) {
+        const int parts = side && c->el.size() == 1 ? run_parts(c, e, n_steps) : 1;
+        const int sc = ssk::kSliceChains;
+        for (int k = 0; k < parts; ++k) {
+            const int s0 = (int)((long long)e.slices * k / parts), s1 = (int)((long long)e.slices * (k + 1) / parts);
+            units.push_back({&e, s0 * sc, std::min(e.M, s1 * sc)});
+        }
+    }
+    const int n_units = (int)units.size();
+    const int lanes = side ? std::min(n_units, kSideStreams + 1) : 1;
     int rc = fork_streams(c, lanes);
     long long left = n_steps;
     while (rc == SS_OK && left > 0) {
         const int ns = (int)std::min<long long>(left, p.chunk_steps);
-        for (int i = 0; rc == SS_OK && i < n_el; ++i) {
+        for (int i = 0; rc == SS_OK && i < n_units; ++i) {
+            const Unit& u = units[i];
             const cudaStream_t st = i % lanes == 0 ? c->stream : c->side[i % lanes - 1];
-            rc = c->prec == SS_FP64 ? launch_chunk<double>(c, c->el[i], c->step, ns, st)
-                                    : launch_chunk<float>(c, c->el[i], c->step, ns, st);
+            rc = c->prec == SS_FP64 ? launch_chunk<double>(c, *u.e, u.m0, u.m1, c->step, ns, st)
+                                    : launch_chunk<float>(c, *u.e, u.m0, u.m1, c->step, ns, st);
         }
         if (rc != SS_OK) break;
         c->step += ns;
@@ -1369,9 +1449,9 @@ int ss_stress(ss_ctx* c, int elem, double* t, double* mean, double* sem, int cap
     if (n_out) *n_out = n;
     if (n == 0 || cap == 0) return SS_OK;
     const std::vector<int> gsz = group_sizes(*e);
-    std::vector<double> L((size_t)n * e->groups * 14);
-    SS_CUDA(c, cudaMemcpyAsync(L.data(), e->logs, L.size() * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    SS_CUDA(c, cudaStreamSynchronize(c->stream));
+    const double* L = nullptr;
+    const int rc = read_logs(c, *e, n, &L);
+    if (rc != SS_OK) return rc;
     for (int i = 0; i < std::min(n, cap); ++i) {
         if (t) t[i] = (double)((c->log_m0 + 1 + i) * p.log_every) * p.dt;
         for (int k = 0; k < 6; ++k) {
@@ -1464,6 +1544,7 @@ int ss_destroy(ss_ctx* c) {
         cudaEventDestroy(pr.second);
     }
     for (Elem& e : c->el) free_elem(e);
+    free_logs(c);
     free_batched(c);
     free_window(c);
     if (c->counters) cudaFree(c->counters);
@@ -1648,9 +1729,10 @@ int ss_log_sums(ss_ctx* c, int elem, int64_t* log_step, double* sums, int cap, i
     if (n_groups) *n_groups = e->groups;
     const int k = std::min(n, cap);
     if (k > 0 && sums) {
-        SS_CUDA(c, cudaMemcpyAsync(sums, e->logs, (size_t)k * e->groups * 14 * sizeof(double),
-                                   cudaMemcpyDeviceToHost, c->stream));
-        SS_CUDA(c, cudaStreamSynchronize(c->stream));
+        const double* L = nullptr;
+        const int rc = read_logs(c, *e, k, &L);
+        if (rc != SS_OK) return rc;
+        std::memcpy(sums, L, (size_t)k * e->groups * 14 * sizeof(double));
     }
     if (log_step)
         for (int i = 0; i < k; ++i) log_step[i] = (c->log_m0 + 1 + i) * p.log_every;
@@ -1770,6 +1852,7 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
         SS_CUDA(c, cudaMalloc(&w.wgt, (size_t)c->levels * 16 * sizeof(double)));
         w.complete = true;
     }
+    c->logs_read = false;
     // a replayed window draws the noise of the recorded one: same step indices
     if (replay) c->step = w.t_start;
     rc = zero_observables(c);
@@ -1784,8 +1867,8 @@ int ss_window_forward(ss_ctx* c, int64_t n_steps, int checkpoint_every, int repl
         c->opt_tape_mode = replay ? 2 : 1;
         c->opt_series = true;
         const int len = seg_len(c, seg);
-        rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, c->step, len, c->stream)
-                                : launch_chunk<float>(c, e, c->step, len, c->stream);
+        rc = c->prec == SS_FP64 ? launch_chunk<double>(c, e, 0, e.M, c->step, len, c->stream)
+                                : launch_chunk<float>(c, e, 0, e.M, c->step, len, c->stream);
         c->opt_tape_mode = 0;
         c->opt_series = false;
         if (rc != SS_OK) return rc;
@@ -1910,7 +1993,7 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
         if (cudaLaunchKernel(kern, dim3((M + cpc - 1) / cpc), dim3(kThreads), args, plan.total, st) != cudaSuccess)
             return SS_ECUDA;
         if (c->levels > 0 &&
-            corr_launches<T>(static_cast<const T*>(a.series), ssk::kSliceChains, ns, M, c->levels, done,
+            corr_launches<T>(static_cast<const T*>(a.series), 0, M, ssk::kSliceChains, ns, M, c->levels, done,
                              reinterpret_cast<T*>(scr + off_hist), reinterpret_cast<double*>(scr + off_acc64), nullptr,
                              reinterpret_cast<T*>(scr + off_lev), (size_t)(ser_cap / 2 + 1) * M * 6, st) < 0)
             return SS_ECUDA;
@@ -1986,10 +2069,8 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
     off = align256(off + (corr ? (size_t)n_chains * c.levels * 96 * ts : 0));
     const size_t off_acc64 = off;
     off = align256(off + (corr ? (size_t)slices * c.levels * 96 * sizeof(double) : 0));
-    const size_t off_kap = off;
-    off = align256(off + 9 * sizeof(double));
-    const size_t off_kfrom = off;
-    off = align256(off + sizeof(long long));
+    const size_t off_zero = off;  // history and sums start at zero
+    off = align256(off + 9 * sizeof(double)) + 256;
     const size_t off_cnt = off;
     off = align256(off + 8 * sizeof(unsigned long long));
     const size_t off_status = off;
@@ -2019,7 +2100,7 @@ extern "C" int ss_run_noalloc(const ss_params* params, int precision, uint64_t s
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     // what must start at zero: history and sums of the correlator, the status word
     // (the event counters are not read)
-    if (corr && cudaMemsetAsync(scr, 0, off_kap, st) != cudaSuccess) return SS_ECUDA;
+    if (corr && cudaMemsetAsync(scr, 0, off_zero, st) != cudaSuccess) return SS_ECUDA;
     if (status_out && cudaMemsetAsync(status_out, 0, sizeof(int32_t), st) != cudaSuccess) return SS_ECUDA;
     int32_t* status = status_out ? status_out : reinterpret_cast<int32_t*>(scr + off_status);
     const int zm = c.el[0].zmax;

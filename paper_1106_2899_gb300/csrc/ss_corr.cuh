@@ -222,13 +222,14 @@ __device__ __forceinline__ void corr_levels(CorrPass<T>& s, const T* yrow, T* st
     if constexpr (STAGE) asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// All levels of one launch: ns samples after n0 earlier ones.  CTA b has the
-// `chains` <= CHAINS chains from b * span + first on and the sums of part b.  lev: two buffers of lev_half elements for the samples the
+// All levels of one launch: ns samples after n0 earlier ones.  CTA b + b0
+// = B has the `chains` <= CHAINS chains from B * span + first on and the sums of
+// part B.  lev: two buffers of lev_half elements for the samples the
 // passes store.  A pair may join the newest sample of the previous launch (the last
 // entry of the level's history) and the first new one.
 template <typename T, bool TT, int CHAINS>
 __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT && CHAINS == kCorrPartChains ? 2 : 1)
-    corr_kernel(const T* __restrict__ ser, int chains, int first, int span, int ns, long long n0, int M, int L, T* __restrict__ hist,
+    corr_kernel(const T* __restrict__ ser, int b0, int chains, int first, int span, int ns, long long n0, int M, int L, T* __restrict__ hist,
                 T* lev, size_t lev_half, double* __restrict__ acc64, double* __restrict__ acc64tt) {
     constexpr bool STAGE = sizeof(T) == 4 && CHAINS == kCorrPartChains;
     __shared__ alignas(16) T red[CHAINS * 96];
@@ -236,7 +237,8 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
     const int lane = threadIdx.x & 31, q = lane % 6;
     const int c = (threadIdx.x >> 5) * kCorrChainsPerWarp + lane / 6;  // chain of this CTA
     const bool mine = lane < 30 && c < chains;
-    const int m = blockIdx.x * span + first + c;
+    const int block = blockIdx.x + b0;
+    const int m = block * span + first + c;
     const bool live = mine && m < M;
     const int src = min(lane / 6 * 6 + q % 3, 31);
     const int mm = live ? m : 0;
@@ -272,12 +274,12 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
             else
                 corr_levels<T, kP / 2, false, TT, STAGE>(s, yrow, st, src, stride, nA, nB > 0, odd_b, out, emit);
         }
-        double* const oA = acc64 + ((size_t)blockIdx.x * L + l) * 96;
+        double* const oA = acc64 + ((size_t)block * L + l) * 96;
         const int col = (q % 3) * kCells + (q / 3) * kP;
         corr_fold<T, 96>(s.accA, l == 0 ? 0 : kP / 2, live, mine, c, col, chains, oA, red);
         if (nB > 0) corr_fold<T, 96>(s.accB, kP / 2, live, mine, c, col, chains, oA + 96, red);
         if constexpr (TT) {
-            double* const oT = acc64tt + ((size_t)blockIdx.x * L + l) * 48;
+            double* const oT = acc64tt + ((size_t)block * L + l) * 48;
             corr_fold<T, 48>(s.ttA, l == 0 ? 0 : kP / 2, live, mine && q >= 3, c, (q - 3) * kP, chains, oT, red);
             if (nB > 0) corr_fold<T, 48>(s.ttB, kP / 2, live, mine && q >= 3, c, (q - 3) * kP, chains, oT + 48, red);
         }
@@ -295,13 +297,14 @@ __global__ void __launch_bounds__(corr_threads(CHAINS), sizeof(T) == 4 && !TT &&
 // instead of 14 and nothing but the histories moves.
 template <typename T, bool TT>
 __global__ void __launch_bounds__(corr_threads(kCorrPartChains), sizeof(T) == 4 ? 4 : 2)
-    corr_step_kernel(const T* __restrict__ ser, int chains, int first, int span, long long n0, int M, int L,
+    corr_step_kernel(const T* __restrict__ ser, int b0, int chains, int first, int span, long long n0, int M, int L,
                      T* __restrict__ hist, double* __restrict__ acc64, double* __restrict__ acc64tt) {
     __shared__ alignas(16) T red[kCorrPartChains * 96];
     const int lane = threadIdx.x & 31, q = lane % 6;
     const int c = (threadIdx.x >> 5) * kCorrChainsPerWarp + lane / 6;  // chain of this CTA
     const bool mine = lane < 30 && c < chains;
-    const int m = blockIdx.x * span + first + c;
+    const int block = blockIdx.x + b0;
+    const int m = block * span + first + c;
     const bool live = mine && m < M;
     const int src = min(lane / 6 * 6 + q % 3, 31);
     const int mm = live ? m : 0;
@@ -318,7 +321,7 @@ __global__ void __launch_bounds__(corr_threads(kCorrPartChains), sizeof(T) == 4 
         acc[0] = x * y;
 #pragma unroll
         for (int k = 1; k < 16; ++k) acc[k] = x * r[16 - k];
-        const size_t part = (size_t)blockIdx.x * L + l;
+        const size_t part = (size_t)block * L + l;
         corr_fold<T, 96>(acc, k0, live, mine, c, (q % 3) * kCells + (q / 3) * kP, chains, acc64 + part * 96, red);
         if constexpr (TT) {
             acc[0] = y * y;

@@ -264,6 +264,7 @@ struct ChunkArgs {
     int n_kap;                  // 0: the constant gradient kap0
     double kap0[9];
     int M, N, zmax, create_mode, destroy_new;
+    int cta0;                   // first CTA tile of this launch
     int log_every, recenter_every;
     long long log_m0;           // logs are taken at steps m*log_every with m > log_m0
     int max_logs, groups, slices;  // slices of kSliceChains chains
@@ -1592,7 +1593,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
 __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
-    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, blockIdx.x * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
+    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
                                          a.nlog_chunk);
 }
 
