@@ -628,8 +628,9 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // positions, with a guard entry on either side (read for a hop beyond an end,
     // whose probability is then replaced by 0)
     Pos<T>* pos = reinterpret_cast<Pos<T>*>(smem + plan.off_pos) + cslot * (NL + 2) + 1;
-    // bond vectors Q_i = R_{i+1} - R_i of the current state, one entry up:
-    // bq[i + 1] = Q_i, bq[0] = 0 (bead 0 has no left bond)
+    // bond vectors Q_i = R_{i+1} - R_i of the current state times k_b, one entry up:
+    // bq[i + 1] = k_b Q_i, bq[0] = 0 (bead 0 has no left bond); with HEUN Q_i itself,
+    // whose corrector rounds the bond force from it
     Pos<T>* bq = reinterpret_cast<Pos<T>*>(smem + plan.off_bq) + cslot * (NL + 1);
     Mask* msk = reinterpret_cast<Mask*>(smem + plan.off_msk) + cslot * NL;
     [[maybe_unused]] T* const red = reinterpret_cast<T*>(smem + plan.off_red) + warp * SEGS * red_chain(W);
@@ -867,9 +868,10 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             Q[b][1] = p1.y - R[b][1];
             Q[b][2] = p1.z - R[b][2];
             Pos<T> qq;
-            qq.x = Q[b][0];
-            qq.y = Q[b][1];
-            qq.z = Q[b][2];
+            const T f = HEUN ? T(1) : c.k_b;
+            qq.x = f * Q[b][0];
+            qq.y = f * Q[b][1];
+            qq.z = f * Q[b][2];
             qq.w = T(0);
             bq[i + 1] = qq;
         }
@@ -952,10 +954,15 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             if (bonds_from_q) {
 #pragma unroll
                 for (int b = 0; b < B; ++b) {
-                    const Pos<T> qm = bq[ll + b * W];  // Q_{i-1} (0 for bead 0)
+                    const Pos<T> qm = bq[ll + b * W];  // k_b Q_{i-1} (0 for bead 0; HEUN: Q_{i-1})
                     const T Qm[3] = {qm.x, qm.y, qm.z};
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) Fo[b][d] = c.k_b * Q[b][d] - c.k_b * Qm[d];
+                    for (int d = 0; d < 3; ++d) {
+                        if constexpr (HEUN)
+                            Fo[b][d] = c.k_b * Q[b][d] - c.k_b * Qm[d];
+                        else
+                            Fo[b][d] = fma(c.k_b, Q[b][d], -Qm[d]);
+                    }
                 }
             } else {
 #pragma unroll
