@@ -78,7 +78,7 @@ class SlipSpring:
                                              _p(k, C.c_double)), "ss_set_flow_table")
 
     def set_batched(self, enable=True):
-        """One persistent, graph-replayed launch per chunk over all elements."""
+        """One graph launch per chunk over all elements."""
         self._chk(self.lib.ss_set_batched(self.h, 1 if enable else 0), "ss_set_batched")
 
     def set_coefficients(self, k_b, k_s, zeta):

@@ -748,12 +748,25 @@ int batched_launch_direct(ss_ctx* c, int k, const ssk::ChunkArgs* d_elems, const
     return SS_OK;
 }
 
-// Candidate lane layouts of the batched kernel, the default first.
-std::vector<std::pair<int, int>> layout_candidates(int N) {
+// Candidate lane layouts of the batched kernel for `total` chains of length N, the
+// default first: by the waves of warps they take (24 warps per SM at one bead per
+// lane, 20 at two).  N = 9..16: 16 x 1 while it fits one wave (7296 chains on 152
+// SMs), 8 x 2 while that does (12160), 16 x 1 for its two and a half waves (19000),
+// then 8 x 2, which does less per chain (us per step at 4096 / 16384 / 65536 chains:
+// 16 x 1 0.99 / 2.89 / 10.4, 8 x 2 1.35 / 3.10 / 10.0).  N = 17..32: 32 x 1 for
+// ensembles of one wave (1024 chains: 1.27 us per step, 16 x 2 1.5), then 16 x 2, or
+// 8 x 3 as in layout_for.
+std::vector<std::pair<int, int>> layout_candidates(int N, long long total, long long sms) {
+    using L = std::vector<std::pair<int, int>>;
     if (N <= 8) return {{8, 1}};
-    if (N <= 16) return {{16, 1}, {8, 2}};
-    if (N <= 24) return {{16, 2}, {8, 3}, {32, 1}};
-    if (N <= 32) return {{16, 2}, {32, 1}};
+    if (N <= 16) {
+        const bool wide = total <= 48 * sms || (total > 80 * sms && total <= 125 * sms);
+        return wide ? L{{16, 1}, {8, 2}} : L{{8, 2}, {16, 1}};
+    }
+    if (N <= 32) {
+        const std::pair<int, int> two = N <= 24 && total >= 8192 ? std::pair<int, int>{8, 3} : std::pair<int, int>{16, 2};
+        return total <= 24 * sms ? L{{32, 1}, two} : L{two, {32, 1}};
+    }
     if (N <= 48) return {{16, 3}};
     if (N <= 64) return {{16, 4}};
     if (N <= 96) return {{32, 3}};
@@ -763,7 +776,7 @@ std::vector<std::pair<int, int>> layout_candidates(int N) {
 // Project-written autotuner: for each chain length, time every candidate layout
 // on a trial ensemble (equilibrium start, no flow, no logs, up to 65536 chains)
 // with the batched kernel of that layout, twice each, and keep the fastest
-// (the default layout unless another is at least 3% faster); results are
+// (the default layout unless another is at least a quarter faster); results are
 // cached per (N, precision) for the process.
 template <typename T>
 int autotune(ss_ctx* c) {
@@ -780,12 +793,12 @@ int autotune(ss_ctx* c) {
                 if (r[0] == N && r[1] == c->prec) bestW = r[2], bestB = r[3];
         }
         if (bestW < 0) {
-            auto cand = layout_candidates(N);
+            long long total = 0;
+            for (const Elem& e : c->el)
+                if (e.N == N) total += e.M;
+            auto cand = layout_candidates(N, total, c->sms);
             bestW = cand[0].first, bestB = cand[0].second;
             if (cand.size() > 1) {
-                long long total = 0;
-                for (const Elem& e : c->el)
-                    if (e.N == N) total += e.M;
                 Elem t;
                 // as many chains as the workload has, up to enough for many waves:
                 // the comparison is then one of steady throughput
@@ -853,11 +866,13 @@ int autotune(ss_ctx* c) {
                     if (rc == SS_OK) cand_ms[ci] = std::min(cand_ms[ci], ms);
                 }
                 // the default layout (the first candidate) gives way only to one
-                // at least 3% faster, so that near-equal layouts do not flip
-                // from one process to the next on timing noise
+                // at least a quarter faster: the candidates are within a few percent
+                // of one another near the lines of the default, and a choice by
+                // timing noise would change the rounding of the stress from one
+                // process to the next
                 size_t pick = 0;
                 for (size_t ci = 1; ci < cand.size(); ++ci)
-                    if (cand_ms[ci] < 0.97f * cand_ms[0] && cand_ms[ci] < cand_ms[pick]) pick = ci;
+                    if (cand_ms[ci] < 0.75f * cand_ms[0] && cand_ms[ci] < cand_ms[pick]) pick = ci;
                 bestW = cand[pick].first;
                 bestB = cand[pick].second;
                 c->log_m0 = saved_m0;
@@ -870,6 +885,15 @@ int autotune(ss_ctx* c) {
                 std::lock_guard<std::mutex> lk(mu);
                 cache.push_back({N, c->prec, bestW, bestB});
             }
+        }
+        // 16 x 2 and 8 x 3 round alike: whichever was timed, the size of this
+        // context's ensembles decides between them
+        if (N > 16 && N <= 24 && bestW != 32) {
+            long long total = 0;
+            for (const Elem& e : c->el)
+                if (e.N == N) total += e.M;
+            bestW = total >= 8192 ? 8 : 16;
+            bestB = total >= 8192 ? 3 : 2;
         }
         for (Elem& e : c->el)
             if (e.N == N) e.W = bestW, e.B = bestB;

@@ -3,12 +3,13 @@
 // for the multiple-tau correlator (a separate kernel) and ensemble stress logs.
 //
 // Layout: one chain per W-lane segment of a warp (W = 32: one chain per warp,
-// W = 16: two), B beads per lane: lane l of a segment owns beads and
+// W = 16: two, W = 8: four), B beads per lane: lane l of a segment owns beads and
 // slip-spring slots l, l + W, ..., so N <= W*B and z_max <= N (the paper's
 // one-slot-per-bead bound, Sec. 3.2); slots above 64 stay empty (z_max <= 64,
 // so a 64-bit mask covers a bead's springs).  A launch advances each chain `nsteps`
 // steps with its whole state in registers; neighbouring beads are read from a
-// per-warp shared-memory position table, stresses are reduced with shuffles.
+// per-warp shared-memory position table, stress parts wait in shared memory for a
+// few steps and are summed there (FP32) or reduced with shuffles (FP64, log steps).
 //
 // Random numbers: Philox4x32-10 (Salmon et al., SC'11), counter = (index,
 // step, purpose, chain id), key = seed.  Per step, slot/bead index l draws
@@ -319,7 +320,8 @@ constexpr int kCounterCopies = 64;  // power of two
 // warps, 28.8 at 20 with the spills of 96 registers).  FP64 work is bound by the
 // FP64 pipe long before twelve warps.
 template <typename T>
-constexpr int chunk_warps_per_sm(int B) {
+constexpr int chunk_warps_per_sm(int B, bool heun_flow = false) {
+    if (heun_flow) return sizeof(T) == 8 ? 8 : (B == 1 ? 20 : (B == 2 ? 16 : 12));  // both states live at once
     return sizeof(T) == 8 ? 12 : (B == 1 ? 24 : (B == 2 ? 20 : 16));
 }
 
@@ -1598,7 +1600,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 // integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
 // be written (without one, its registers are free).
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B))
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B, HEUN && FLOW))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
     run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
                                          a.nlog_chunk);
