@@ -1176,7 +1176,7 @@ constexpr int kSideStreams = 7;    // beside the context's own
 // 80: 7.41 -> 6.74, 6.72); from eight waves on the tail is small and two parts let
 // the correlator overlap (65536 x 32: 34.7 -> 34.4 ms, four parts 34.6).
 int run_parts(const ss_ctx* c, const Elem& e, long long n_steps) {
-    const int per_sm = c->prec == SS_FP64 ? ssk::chunk_warps_per_sm<double>(e.B) : ssk::chunk_warps_per_sm<float>(e.B);
+    const int per_sm = c->prec == SS_FP64 ? ssk::chunk_warps_per_sm<double>(e.W, e.B) : ssk::chunk_warps_per_sm<float>(e.W, e.B);
     const long long warps = ((long long)e.M * e.W + 31) / 32, slots = (long long)per_sm * c->sms;
     if (n_steps < 256 || warps <= slots) return 1;
     return std::min(e.slices, warps < 8 * slots ? 4 : 2);

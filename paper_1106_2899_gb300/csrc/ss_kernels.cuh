@@ -317,12 +317,19 @@ constexpr int kChunkThreads = 32;
 constexpr int kCounterCopies = 64;  // power of two
 // Resident warps per SM the kernels are compiled for.  Two beads per lane fit 96
 // registers; three or more need 128 (N = 40, 65536 chains: 26.4 us per step at 16
-// warps, 28.8 at 20 with the spills of 96 registers).  FP64 work is bound by the
+// warps, 28.8 at 20 with the spills of 96 registers).  Sixteen lanes of four beads
+// spill 136-188 bytes at 128 registers and none at 168 (N = 62, 9000 chains, 400
+// steps: 2.97 -> 2.67 ms; N = 56, 16000 chains: 4.62 -> 4.20) and take 254 with Heun
+// and flow (N = 50, 1000 chains: 1.53 -> 1.35 ms); Heun without flow stays at 128,
+// since at 168 the compiler contracts its sums in another order and the results
+// differ in the last bits.  FP64 work is bound by the
 // FP64 pipe long before twelve warps.
 template <typename T>
-constexpr int chunk_warps_per_sm(int B, bool heun_flow = false) {
-    if (heun_flow) return sizeof(T) == 8 ? 8 : (B == 1 ? 20 : (B == 2 ? 16 : 12));  // both states live at once
-    return sizeof(T) == 8 ? 12 : (B == 1 ? 24 : (B == 2 ? 20 : 16));
+constexpr int chunk_warps_per_sm(int W, int B, bool heun = false, bool flow = false) {
+    if (sizeof(T) == 8) return heun && flow ? 8 : 12;
+    if (W == 16 && B == 4 && !(heun && !flow)) return heun ? 8 : 12;
+    if (heun && flow) return B == 1 ? 20 : (B == 2 ? 16 : 12);  // both states live at once
+    return B == 1 ? 24 : (B == 2 ? 20 : 16);
 }
 
 // Columns of a chain's row in device memory (R, A [3][NP], S, tape [NP]): a
@@ -1600,7 +1607,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 // integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
 // be written (without one, its registers are free).
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B, HEUN && FLOW))
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B, HEUN, FLOW))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
     run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
                                          a.nlog_chunk);
@@ -1619,7 +1626,7 @@ struct RunInfo {
 };
 
 template <typename T, int W, int B>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(B))
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B))
     batched_kernel(const ChunkArgs* __restrict__ elems, const int2* __restrict__ items, const RunInfo info,
                    const StepConst<T> c) {
     static_assert(sizeof(ChunkArgs) % 8 == 0, "copied in 8-byte words");
