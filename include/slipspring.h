@@ -107,7 +107,9 @@ typedef struct {
                                reduced to 1024): the launch's stress series, 24 B per
                                chain and step in FP32, is what the correlator reads.
                                The chain states and event counts do not depend on it
-                               (random numbers are indexed by the absolute step); the
+                               (random numbers are indexed by the absolute step; under
+                               SS_HEUN a launch with a flow in any of its steps rounds
+                               the corrector otherwise than one without); the
                                correlator folds its FP32 sums of each launch into FP64,
                                so its sums depend on it at the rounding level        */
     int32_t corr_tt;        /* 1: also correlate sigma + sigma^(v) with itself (channels

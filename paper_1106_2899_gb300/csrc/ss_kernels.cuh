@@ -886,10 +886,14 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         }
     };
     bond_vectors();
+    // the first step's forces read records, masks and bond vectors that other lanes
+    // of the chain have written (the later steps' lie behind the barrier that ends a
+    // step)
+    __syncwarp();
 
     // Random numbers of step tt: block (i, tt, STEP, chain) per bead/slot i.
-    // They do not depend on the state, so each step draws the next step's
-    // at its end, where their integer work interleaves with the stress.
+    // They do not depend on the state: a step draws its own at its top, where their
+    // integer work interleaves with the forces.
     auto draw = [&](const uint32_t tt, T (&nrm)[B][4], U (&u)[B]) {
         const unsigned long long p_shared = philox_step_shared(tt, kPurposeStep, c.rk0);
 #pragma unroll
@@ -1182,8 +1186,8 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         }
         // the Heun corrector above read other lanes' positions, so they are
         // overwritten only after a barrier; in the Euler step the last reads
-        // of the position table lie behind the barriers of the slot masks and
-        // of the forces already
+        // of the position table lie behind the barrier that ended the last step
+        // (or the setup of the launch) already
         if constexpr (HEUN) __syncwarp();
         store_pos(Rn);
         __syncwarp();
