@@ -1643,7 +1643,10 @@ __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B))
         args_s[i] = reinterpret_cast<const unsigned long long*>(elems + wi.x)[i];
     __syncthreads();
     const int nlog = a.log_every > 0 ? (int)((info.t0 + info.nsteps) / a.log_every - info.t0 / a.log_every) : 0;
-    // the 8 x 2 layout sums its lanes' two beads first, as its own layout
+    // 8 x 2 adds the stress of a lane's two beads in one fused sum here and in two
+    // in chunk_kernel: the stress logs of the two paths differ by FP32 rounding there.
+    // The centre of mass, the only sum over beads that enters a state, is the same
+    // either way.
     constexpr int VL = W == 8 && B != 2 ? 2 : 1;
     run_chains<T, W, B, kWinOff, true, false, false, VL>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
                                                      info.log_m0, nlog);
