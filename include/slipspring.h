@@ -165,8 +165,9 @@ int ss_set_flow_table(ss_ctx* ctx, int n, const int32_t* elem, const int64_t* fr
  * layout; each CTA runs one (element, chain tile) work item for the whole
  * chunk, longest chains first.  Before the first batched launch an autotuner times the candidate lane
  * layouts of each chain length on a scratch ensemble and keeps the fastest (the
- * default layout unless another is at least a quarter faster; results cached per
- * process).  Batched mode keeps the stress logs, not the
+ * default layout, which follows the number of chains of that length, unless
+ * another is at least a quarter faster; results cached for the process by device,
+ * length, precision and default).  Batched mode keeps the stress logs, not the
  * correlator: ss_run fails with SS_EINVAL unless corr_levels < 0.  The
  * numbers drawn, the states and the event counts are those of the per-element
  * path bit for bit, the stress logs those up to the rounding of sums over the

@@ -66,7 +66,7 @@ struct BatchedClass {
 struct ss_ctx {
     cudaStream_t stream = nullptr;
     int prec = SS_FP32;
-    int sms = 1;  // of the device
+    int dev = 0, sms = 1;  // the device and its SMs
     uint64_t seed = 0;
     std::vector<Elem> el;
     ss_params P{};
@@ -776,27 +776,35 @@ std::vector<std::pair<int, int>> layout_candidates(int N, long long total, long 
 // Project-written autotuner: for each chain length, time every candidate layout
 // on a trial ensemble (equilibrium start, no flow, no logs, up to 65536 chains)
 // with the batched kernel of that layout, twice each, and keep the fastest
-// (the default layout unless another is at least a quarter faster); results are
-// cached per (N, precision) for the process.
+// (the default layout unless another is at least a quarter faster).  Results are
+// cached for the process by what they depend on: the device, the length, the
+// precision and the default, which follows the number of chains.  (Cached by length
+// and precision alone, a context of 65536 chains of N = 32 after one of 1000 ran
+// 32 x 1, the layout for one wave.)
 template <typename T>
 int autotune(ss_ctx* c) {
     static std::mutex mu;
-    static std::vector<std::array<int, 4>> cache;  // N, prec, W, B
+    struct Tuned {
+        int dev, N, prec;
+        std::pair<int, int> first, best;  // layouts (W, B): the default and the one kept
+    };
+    static std::vector<Tuned> cache;
     std::vector<int> lengths;
     for (const Elem& e : c->el)
         if (std::find(lengths.begin(), lengths.end(), e.N) == lengths.end()) lengths.push_back(e.N);
     for (int N : lengths) {
         int bestW = -1, bestB = -1;
+        long long total = 0;
+        for (const Elem& e : c->el)
+            if (e.N == N) total += e.M;
+        const auto cand = layout_candidates(N, total, c->sms);
         {
             std::lock_guard<std::mutex> lk(mu);
-            for (auto& r : cache)
-                if (r[0] == N && r[1] == c->prec) bestW = r[2], bestB = r[3];
+            for (const Tuned& r : cache)
+                if (r.dev == c->dev && r.N == N && r.prec == c->prec && r.first == cand[0])
+                    bestW = r.best.first, bestB = r.best.second;
         }
         if (bestW < 0) {
-            long long total = 0;
-            for (const Elem& e : c->el)
-                if (e.N == N) total += e.M;
-            auto cand = layout_candidates(N, total, c->sms);
             bestW = cand[0].first, bestB = cand[0].second;
             if (cand.size() > 1) {
                 Elem t;
@@ -883,17 +891,8 @@ int autotune(ss_ctx* c) {
                 free_elem(t);
                 if (rc != SS_OK) return rc;
                 std::lock_guard<std::mutex> lk(mu);
-                cache.push_back({N, c->prec, bestW, bestB});
+                cache.push_back({c->dev, N, c->prec, cand[0], cand[pick]});
             }
-        }
-        // 16 x 2 and 8 x 3 round alike: whichever was timed, the size of this
-        // context's ensembles decides between them
-        if (N > 16 && N <= 24 && bestW != 32) {
-            long long total = 0;
-            for (const Elem& e : c->el)
-                if (e.N == N) total += e.M;
-            bestW = total >= 8192 ? 8 : 16;
-            bestB = total >= 8192 ? 3 : 2;
         }
         for (Elem& e : c->el)
             if (e.N == N) e.W = bestW, e.B = bestB;
@@ -1246,9 +1245,8 @@ int ss_create(ss_ctx** out, const ss_element* elems, int n_elems, int precision,
         ss_destroy(c);
         return SS_ECUDA;
     }
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    if (cudaGetDevice(&c->dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->dev) != cudaSuccess) {
         ss_destroy(c);
         return SS_ECUDA;
     }
