@@ -367,6 +367,20 @@ bool flow_in_window(const Elem& e, long long t0, int nsteps) {
     return false;
 }
 
+// Stress-log steps of one chain-kernel launch at most.  Every CTA keeps 112 bytes per
+// log step of its launch in shared memory, and CTAs are single warps: a launch with
+// many log steps would leave room for few of them on an SM (N = 32: 20 without logs,
+// 17 with 16, 10 with 103, one with 1024).  Such a chunk is split into launches (us per
+// step of 65536 x 32 under shear, log_every 10 / 1: 27.2 / 685 unsplit, 19.3 / 86.1 at
+// 16 log steps, 20.5 / 86.3 at 32; 4096 x 40: 3.7 / 49.6, 2.7 / 6.8, 3.6 / 9.6).  The sums
+// of every warp enter device memory by FP64 atomics, which bound a log at every step.
+constexpr int kLaunchLogs = 16;
+// steps from t on, n at most, with no more log steps than that
+int log_bounded_steps(const ss_params& p, long long t, int n) {
+    if (p.log_every <= 0) return n;
+    return (int)std::min<long long>(n, (t / p.log_every + kLaunchLogs + 1) * p.log_every - 1 - t);
+}
+
 template <typename T>
 int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, cudaStream_t st) {
     NvtxRange range("chain kernel + correlator launch");
@@ -394,12 +408,9 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     a.max_logs = p.max_logs;
     a.groups = e.groups;
     a.slices = e.slices;
-    a.t0 = t0;
-    a.nsteps = nsteps;
     a.key0 = (uint32_t)c->seed;
     a.key1 = (uint32_t)(c->seed >> 32);
     a.chain_base = e.chain_base;
-    a.nlog_chunk = p.log_every > 0 ? (int)((t0 + nsteps) / p.log_every - t0 / p.log_every) : 0;
     // the correlator's input: this launch's stress series (a window keeps the
     // series of the whole window for its adjoint)
     const bool corr = c->levels > 0 && !c->opt_corr_off;
@@ -413,10 +424,7 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
             a.series_row0 = 0;
         }
     }
-    if (c->opt_corr_off) {  // recomputation: no observables at all
-        a.log_every = 0;
-        a.nlog_chunk = 0;
-    }
+    if (c->opt_corr_off) a.log_every = 0;  // recomputation: no observables at all
     if (c->opt_tape_mode) {
         a.tape = c->win.tape;
         a.tape_mode = c->opt_tape_mode;
@@ -437,29 +445,36 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     const int win = c->opt_tape_mode == 1 ? ssk::kWinRecord : (c->opt_tape_mode == 2 ? ssk::kWinReplay : ssk::kWinOff);
     const void* kern = chunk_fn<T>(e.W, e.B, win, flow_in_window(e, t0, nsteps), c->P.integrator == SS_HEUN, corr);
     if (!kern) return fail(c, SS_EINVAL, "no chain kernel for this layout");
-    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk);
-    // the attribute belongs to the current device: set it on every launch that
-    // needs more than the default 48 KiB (a host call per launch of many steps)
-    if (plan.total > 48 * 1024)
-        SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total));
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
     const int cpc = chains_per_cta(e.W), ctas = (m1 - m0 + cpc - 1) / cpc;
     a.cta0 = m0 / cpc;
-    cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    if (c->timing) {
-        SS_CUDA(c, cudaEventCreate(&ev0));
-        SS_CUDA(c, cudaEventCreate(&ev1));
-        SS_CUDA(c, cudaEventRecord(ev0, st));
-    }
     void* args[] = {(void*)&a, (void*)&sc};
-    SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, st));
-    if (c->timing) {
-        SS_CUDA(c, cudaEventRecord(ev1, st));
-        c->events.emplace_back(ev0, ev1);
+    const long long row0 = a.series_row0;
+    for (int done = 0; done < nsteps; done += a.nsteps) {
+        a.t0 = t0 + done;
+        a.nsteps = a.log_every > 0 ? log_bounded_steps(p, a.t0, nsteps - done) : nsteps - done;
+        a.series_row0 = row0 + done;
+        a.nlog_chunk = a.log_every > 0 ? (int)((a.t0 + a.nsteps) / a.log_every - a.t0 / a.log_every) : 0;
+        const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk);
+        // the attribute belongs to the current device: set it on every launch that
+        // needs more than the default 48 KiB (a host call per launch of many steps)
+        if (plan.total > 48 * 1024)
+            SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total));
+        cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+        if (c->timing) {
+            SS_CUDA(c, cudaEventCreate(&ev0));
+            SS_CUDA(c, cudaEventCreate(&ev1));
+            SS_CUDA(c, cudaEventRecord(ev0, st));
+        }
+        SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, st));
+        if (c->timing) {
+            SS_CUDA(c, cudaEventRecord(ev1, st));
+            c->events.emplace_back(ev0, ev1);
+        }
+        c->launches++;
     }
-    c->launches++;
     if (corr) {
-        const T* ser = static_cast<const T*>(a.series) + (size_t)a.series_row0 * e.M * 6;
+        const T* ser = static_cast<const T*>(a.series) + (size_t)row0 * e.M * 6;
         const int nl = corr_launches<T>(ser, m0, m1, ssk::corr_chains(e.M), nsteps, e.M, c->levels, c->nsamp, static_cast<T*>(e.hist), e.acc64,
                                         e.acc64tt, static_cast<T*>(e.lev), (size_t)(e.ser_cap / 4 + 1) * e.M * 6,
                                         st);
@@ -734,7 +749,7 @@ const void* batched_fn_of(int k) {
 
 template <typename T>
 int batched_smem_bytes(const ss_ctx* c, int k) {
-    const int nlog = c->P.log_every > 0 ? c->P.chunk_steps / c->P.log_every + 1 : 0;
+    const int nlog = c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
     return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog).total;
 }
 
@@ -982,7 +997,7 @@ int batched_run(ss_ctx* c, long long n_steps) {
     }
     long long left = n_steps;
     while (left > 0) {
-        const int ns = (int)std::min<long long>(left, c->P.chunk_steps);
+        const int ns = log_bounded_steps(c->P, c->step, (int)std::min<long long>(left, c->P.chunk_steps));
         int rc = batched_chunk<T>(c, c->step, ns);
         if (rc != SS_OK) return rc;
         c->step += ns;
