@@ -455,7 +455,9 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
         a.nsteps = a.log_every > 0 ? log_bounded_steps(p, a.t0, nsteps - done) : nsteps - done;
         a.series_row0 = row0 + done;
         a.nlog_chunk = a.log_every > 0 ? (int)((a.t0 + a.nsteps) / a.log_every - a.t0 / a.log_every) : 0;
-        const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk);
+        // (the window kernels have the series compiled in, also for a replay without it)
+        const ssk::SmemPlan plan =
+            ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk, corr || win != ssk::kWinOff);
         // the attribute belongs to the current device: set it on every launch that
         // needs more than the default 48 KiB (a host call per launch of many steps)
         if (plan.total > 48 * 1024)
@@ -750,7 +752,7 @@ const void* batched_fn_of(int k) {
 template <typename T>
 int batched_smem_bytes(const ss_ctx* c, int k) {
     const int nlog = c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
-    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog).total;
+    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog, false).total;
 }
 
 template <typename T>
@@ -1183,6 +1185,14 @@ int order_streams(ss_ctx* c, cudaStream_t first, cudaStream_t later) {
     return SS_OK;
 }
 
+// warps per SM of the chain kernel's launches over an element
+template <typename T>
+int resident_warps(const ss_ctx* c, const Elem& e, bool flow) {
+    const int nlog = c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
+    return std::min(ssk::chunk_warps_per_sm<T>(e.W, e.B, c->P.integrator == SS_HEUN, flow),
+                    ssk::ctas_by_smem(ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, nlog, c->levels > 0).total));
+}
+
 constexpr int kSideStreams = 7;    // beside the context's own
 // Parts of one element's chains that run side by side: for runs long enough to pay
 // for the launches (256 steps), of more warps than the chip holds at once.  Four
@@ -1190,7 +1200,8 @@ constexpr int kSideStreams = 7;    // beside the context's own
 // 80: 7.41 -> 6.74, 6.72); from eight waves on the tail is small and two parts let
 // the correlator overlap (65536 x 32: 34.7 -> 34.4 ms, four parts 34.6).
 int run_parts(const ss_ctx* c, const Elem& e, long long n_steps) {
-    const int per_sm = c->prec == SS_FP64 ? ssk::chunk_warps_per_sm<double>(e.W, e.B) : ssk::chunk_warps_per_sm<float>(e.W, e.B);
+    const bool flow = flow_in_window(e, c->step, (int)std::min<long long>(n_steps, 1 << 30));
+    const int per_sm = c->prec == SS_FP64 ? resident_warps<double>(c, e, flow) : resident_warps<float>(c, e, flow);
     const long long warps = ((long long)e.M * e.W + 31) / 32, slots = (long long)per_sm * c->sms;
     if (n_steps < 256 || warps <= slots) return 1;
     return std::min(e.slices, warps < 8 * slots ? 4 : 2);
@@ -2016,7 +2027,7 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
     const void* kern = chunk_fn<T>(W, B, ssk::kWinOff, flow, false, c->levels > 0);
     if (!kern) return SS_EINVAL;
     const int cpc = chains_per_cta(W);
-    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, W, B, 0);
+    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, W, B, 0, c->levels > 0);
     if (plan.total > 48 * 1024 &&
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total) != cudaSuccess)
         return SS_ECUDA;

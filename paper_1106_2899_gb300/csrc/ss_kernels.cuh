@@ -362,8 +362,13 @@ __host__ __device__ constexpr int red_chain(int W) {
     return n + (W == 32 ? 0 : pad);
 }
 
+// series: a stress series may be written.  Without one nothing touches the reduction
+// buffer, a third of the shared memory of a CTA: left out, the batched kernel and the
+// chain kernel without the correlator run the warps their registers are planned for
+// (16 x 2 with 11 log steps: 17 and 18 warps/SM -> 20; 512 elements, 1000 steps: 57.4 ->
+// 52.3 ms, six ensembles of 4096 x 40 under shear: 11.1 -> 10.7 ms).
 template <typename T>
-__host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_chunk) {
+__host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_chunk, bool series) {
     SmemPlan p;
     const int chains = warps * (32 / W), NL = W * B;
     p.off_rec = 0;
@@ -378,7 +383,7 @@ __host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_
     p.off_msk = (sz + 15) & ~15;
     sz = p.off_msk + chains * NL * (int)(NL <= 32 ? sizeof(unsigned) : sizeof(unsigned long long));
     p.off_red = (sz + 15) & ~15;
-    sz = p.off_red + (sizeof(T) == 4 ? chains * red_chain(W) * (int)sizeof(T) : 0);
+    sz = p.off_red + (series && sizeof(T) == 4 ? chains * red_chain(W) * (int)sizeof(T) : 0);
     p.off_kap = (sz + 15) & ~15;
     sz = p.off_kap + warps * 3 * (int)sizeof(Pos<T>);
     p.off_log = (sz + 15) & ~15;
@@ -386,6 +391,10 @@ __host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_
     p.total = (sz + 15) & ~15;
     return p;
 }
+
+// CTAs that `bytes` of shared memory each leave room for on an SM: 228 KB, 1 KB per CTA
+// for the system, granules of 128 bytes
+constexpr int ctas_by_smem(int bytes) { return 228 * 1024 / ((bytes + 1024 + 127) / 128 * 128); }
 
 // -------------------------------------------------------------- helpers -----
 // 1 + index of the lowest set bit (0 for none) of a 32- or 64-bit slot mask
@@ -628,7 +637,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     const unsigned lt = ((1u << lane) - 1u) & segmask;  // lanes of this segment below this one
 
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemPlan plan = smem_plan<T>(nwarps, W, B, nlog_);
+    const SmemPlan plan = smem_plan<T>(nwarps, W, B, nlog_, CORR);
     // spring records of this chain: [0, NL) the first spring of each bead, [NL, 2 NL)
     // the second (zeros where there is none), [2 NL, 3 NL) by slot: springs beyond
     // the second of a bead, and scratch of the re-indexing
