@@ -51,7 +51,8 @@ def test_without_a_series_registers_decide(table):
 
 
 def test_with_a_series(table):
-    # the correlator runs without logs at the register figure, but 8 x 2 (18 of 20),
-    # 8 x 3 (15 of 16), 16 x 3 (15 of 16) and 32 x 4 (13 of 16)
-    short = {k[:2]: v[1] for k, v in table.items() if k[2] == 0 and k[3] and v[1] < v[0]}
-    assert short == {(8, 2): 18, (8, 3): 15, (16, 3): 15, (32, 4): 13}
+    # without logs the register figure or, of these, nearly
+    least = {(8, 2): 18, (8, 3): 15, (16, 3): 15, (32, 4): 13}
+    for (w, b, logs, series), (regs, chunk, _) in table.items():
+        if series and logs == 0:
+            assert chunk >= least.get((w, b), regs), (w, b)
