@@ -456,7 +456,7 @@ def run_ours(args):
         "gpu_launches": int(launches),
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "lane-ops/s",
                      "frac": achieved / peak, "traffic": traffic,
-                     "kernel": "chunk_kernel<float, 16, 2, 0, 0, 0, 1>", "kernel_ms": kernel_ms,
+                     "kernel": "chunk_kernel<float, 16, 2, 0, 0, 0, 1, 0>", "kernel_ms": kernel_ms,
                      "kernel_share_of_region": kernel_ms * spc * args.steps / steps_per_launch / ms_total if ws == 1 else None,
                      "alg_ops_per_bead_step": ops_lve,
                      "alg_ops_source": "oracle counting build (tests/golden/alg_ops.txt)",

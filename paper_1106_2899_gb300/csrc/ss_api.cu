@@ -246,10 +246,40 @@ int chains_per_cta(int W) { return kWarpsPerCta * (32 / W); }
 
 // the chain kernel of this precision (windows refuse a velocity gradient)
 template <typename T>
-const void* chunk_fn(int W, int B, int win, bool flow, bool heun, bool corr) {
+const void* chunk_fn(int W, int B, int win, bool flow, bool heun, bool corr, bool alt) {
     if (sizeof(T) == 8)
-        return flow ? ssk::chunk_fn_f64_flow(W, B, win, heun, corr) : ssk::chunk_fn_f64(W, B, win, heun, corr);
-    return flow ? ssk::chunk_fn_f32_flow(W, B, win, heun, corr) : ssk::chunk_fn_f32(W, B, win, heun, corr);
+        return flow ? ssk::chunk_fn_f64_flow(W, B, win, heun, corr, alt) : ssk::chunk_fn_f64(W, B, win, heun, corr, alt);
+    return flow ? ssk::chunk_fn_f32_flow(W, B, win, heun, corr, alt) : ssk::chunk_fn_f32(W, B, win, heun, corr, alt);
+}
+// its shared memory with nlog log steps; series: a stress series may be written
+template <typename T>
+int chunk_smem(int W, int B, int nlog, bool flow, bool heun, bool series, bool alt) {
+    return ssk::smem_plan<T>(kWarpsPerCta, W, B, nlog, series ? ssk::red_steps<T>(W, B, heun, flow, alt) : 0).total;
+}
+// and its warps per SM
+template <typename T>
+int chunk_resident(int W, int B, int nlog, bool flow, bool heun, bool series, bool alt) {
+    return std::min(ssk::chunk_warps_per_sm<T>(W, B, heun, flow, alt),
+                    ssk::ctas_by_smem(chunk_smem<T>(W, B, nlog, flow, heun, series, alt)));
+}
+// Whether M chains of 49..64 beads (16 x 4) run the second form of the chain kernel.
+// Euler-Maruyama and Heun without a flow: more warps per SM do the same work per time,
+// or a little less, but may save a wave (us of 400 steps, first / second form: 4000 x 60,
+// 13.2 warps per SM, Euler-Maruyama 1516 / 1335, with shear 1592 / 1355, Heun 2104 /
+// 1740; 9000 x 62, 29.6 per SM: 2578 / 2640, 2718 / 2680, 3852 / 3490; 2500 x 52: 951 / 1079,
+// 1001 / 1145, 1376 / 1420).  Heun with flow: the first form does more per time (30000 x
+// 60: 15.1 / 17.4 ms; 3000 x 60: 1.87 / 2.53), the second is faster in one wave of its
+// own and in two where the first, of whose warps 12 fit an SM, takes two as well
+// (2300 x 60: 1.67 / 1.59; 3500 x 60: 1.97 / 2.69; 4000 x 60: 2.98 / 2.77).
+template <typename T>
+bool four_bead_alt(int M, int W, int B, int sms, int nlog, bool flow, bool heun, bool series) {
+    if (sizeof(T) == 8 || W != 16 || B != 4) return false;
+    const int warps = (M + 1) / 2;
+    const int a = sms * chunk_resident<T>(W, B, nlog, flow, heun, series, false);
+    const int b = sms * chunk_resident<T>(W, B, nlog, flow, heun, series, true);
+    if (heun && flow) return warps <= b || (warps > 12 * sms && warps <= 2 * b);
+    const auto cost = [&](int slots) { return (long long)((warps + slots - 1) / slots) * slots; };
+    return cost(b) * 23 < cost(a) * 20;
 }
 
 // z_max by default: one slot per bead (Sec. 3.2), at most SS_MAX_SLOTS
@@ -381,6 +411,10 @@ int log_bounded_steps(const ss_params& p, long long t, int n) {
     return (int)std::min<long long>(n, (t / p.log_every + kLaunchLogs + 1) * p.log_every - 1 - t);
 }
 
+int logs_per_launch(const ss_ctx* c) {
+    return c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
+}
+
 template <typename T>
 int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, cudaStream_t st) {
     NvtxRange range("chain kernel + correlator launch");
@@ -443,7 +477,12 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     // refuse a velocity gradient), a launch without a velocity gradient the one
     // without the flow terms
     const int win = c->opt_tape_mode == 1 ? ssk::kWinRecord : (c->opt_tape_mode == 2 ? ssk::kWinReplay : ssk::kWinOff);
-    const void* kern = chunk_fn<T>(e.W, e.B, win, flow_in_window(e, t0, nsteps), c->P.integrator == SS_HEUN, corr);
+    // (the window kernels have the series compiled in, also for a replay without it)
+    const bool flow = flow_in_window(e, t0, nsteps), heun = c->P.integrator == SS_HEUN;
+    const bool series = corr || win != ssk::kWinOff;
+    const bool alt =
+        win == ssk::kWinOff && four_bead_alt<T>(e.M, e.W, e.B, c->sms, logs_per_launch(c), flow, heun, series);
+    const void* kern = chunk_fn<T>(e.W, e.B, win, flow, heun, corr, alt);
     if (!kern) return fail(c, SS_EINVAL, "no chain kernel for this layout");
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
     const int cpc = chains_per_cta(e.W), ctas = (m1 - m0 + cpc - 1) / cpc;
@@ -455,20 +494,18 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
         a.nsteps = a.log_every > 0 ? log_bounded_steps(p, a.t0, nsteps - done) : nsteps - done;
         a.series_row0 = row0 + done;
         a.nlog_chunk = a.log_every > 0 ? (int)((a.t0 + a.nsteps) / a.log_every - a.t0 / a.log_every) : 0;
-        // (the window kernels have the series compiled in, also for a replay without it)
-        const ssk::SmemPlan plan =
-            ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, a.nlog_chunk, corr || win != ssk::kWinOff);
+        const int smem = chunk_smem<T>(e.W, e.B, a.nlog_chunk, flow, heun, series, alt);
         // the attribute belongs to the current device: set it on every launch that
         // needs more than the default 48 KiB (a host call per launch of many steps)
-        if (plan.total > 48 * 1024)
-            SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total));
+        if (smem > 48 * 1024)
+            SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         if (c->timing) {
             SS_CUDA(c, cudaEventCreate(&ev0));
             SS_CUDA(c, cudaEventCreate(&ev1));
             SS_CUDA(c, cudaEventRecord(ev0, st));
         }
-        SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, plan.total, st));
+        SS_CUDA(c, cudaLaunchKernel(kern, dim3(ctas), dim3(kThreads), args, smem, st));
         if (c->timing) {
             SS_CUDA(c, cudaEventRecord(ev1, st));
             c->events.emplace_back(ev0, ev1);
@@ -751,8 +788,7 @@ const void* batched_fn_of(int k) {
 
 template <typename T>
 int batched_smem_bytes(const ss_ctx* c, int k) {
-    const int nlog = c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
-    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog, false).total;
+    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], logs_per_launch(c), 0).total;
 }
 
 template <typename T>
@@ -1188,9 +1224,10 @@ int order_streams(ss_ctx* c, cudaStream_t first, cudaStream_t later) {
 // warps per SM of the chain kernel's launches over an element
 template <typename T>
 int resident_warps(const ss_ctx* c, const Elem& e, bool flow) {
-    const int nlog = c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
-    return std::min(ssk::chunk_warps_per_sm<T>(e.W, e.B, c->P.integrator == SS_HEUN, flow),
-                    ssk::ctas_by_smem(ssk::smem_plan<T>(kWarpsPerCta, e.W, e.B, nlog, c->levels > 0).total));
+    const bool heun = c->P.integrator == SS_HEUN, series = c->levels > 0;
+    const int nlog = logs_per_launch(c);
+    const bool alt = four_bead_alt<T>(e.M, e.W, e.B, c->sms, nlog, flow, heun, series);
+    return chunk_resident<T>(e.W, e.B, nlog, flow, heun, series, alt);
 }
 
 constexpr int kSideStreams = 7;    // beside the context's own
@@ -2024,12 +2061,20 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
         a.series = scr + off_ser;
         a.series_row0 = 0;
     }
-    const void* kern = chunk_fn<T>(W, B, ssk::kWinOff, flow, false, c->levels > 0);
+    bool alt = false;
+    if (W == 16 && B == 4) {
+        int dev = 0, sms = 1;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+            return SS_ECUDA;
+        alt = four_bead_alt<T>(M, W, B, sms, 0, flow, false, c->levels > 0);
+    }
+    const void* kern = chunk_fn<T>(W, B, ssk::kWinOff, flow, false, c->levels > 0, alt);
     if (!kern) return SS_EINVAL;
     const int cpc = chains_per_cta(W);
-    const ssk::SmemPlan plan = ssk::smem_plan<T>(kWarpsPerCta, W, B, 0, c->levels > 0);
-    if (plan.total > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, plan.total) != cudaSuccess)
+    const int smem = chunk_smem<T>(W, B, 0, flow, false, c->levels > 0, alt);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return SS_ECUDA;
     ssk::StepConst<T> sc = step_const<T>(c, N);
     void* args[] = {(void*)&a, (void*)&sc};
@@ -2038,7 +2083,7 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
         const int ns = (int)std::min<int64_t>(n_steps - done, c->levels > 0 ? ser_cap : p.chunk_steps);
         a.t0 = t0 + done;
         a.nsteps = ns;
-        if (cudaLaunchKernel(kern, dim3((M + cpc - 1) / cpc), dim3(kThreads), args, plan.total, st) != cudaSuccess)
+        if (cudaLaunchKernel(kern, dim3((M + cpc - 1) / cpc), dim3(kThreads), args, smem, st) != cudaSuccess)
             return SS_ECUDA;
         if (c->levels > 0 &&
             corr_launches<T>(static_cast<const T*>(a.series), 0, M, ssk::kSliceChains, ns, M, c->levels, done,

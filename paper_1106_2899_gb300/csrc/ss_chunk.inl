@@ -6,31 +6,34 @@
 namespace ssk {
 namespace {
 
-template <typename T, int W, int B, bool FLOW>
+template <typename T, int W, int B, bool FLOW, bool ALT>
 const void* chunk_of(int win, bool heun, bool corr) {
     if constexpr (!FLOW) {
         if (win == kWinRecord) return (const void*)chunk_kernel<T, W, B, kWinRecord, false, false, true>;
         if (win == kWinReplay) return (const void*)chunk_kernel<T, W, B, kWinReplay, false, false, true>;
     }
-    if (heun)
-        return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, true>
-                    : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, false>;
-    return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, true>
-                : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, false>;
+    if (heun)  // (without a flow and a series both forms are the same)
+        return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, true, ALT>
+                    : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, false, ALT && FLOW>;
+    return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, true, ALT>
+                : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, false, ALT>;
 }
 
 template <typename T, bool FLOW>
-const void* chunk_fn(int W, int B, int win, bool heun, bool corr) {
+const void* chunk_fn(int W, int B, int win, bool heun, bool corr, bool alt) {
+    if constexpr (sizeof(T) == 4) {
+        if (alt && W == 16 && B == 4 && win == kWinOff) return chunk_of<T, 16, 4, FLOW, true>(win, heun, corr);
+    }
     switch (W * 16 + B) {
-        case 8 * 16 + 1: return chunk_of<T, 8, 1, FLOW>(win, heun, corr);
-        case 8 * 16 + 2: return chunk_of<T, 8, 2, FLOW>(win, heun, corr);
-        case 8 * 16 + 3: return chunk_of<T, 8, 3, FLOW>(win, heun, corr);
-        case 16 * 16 + 1: return chunk_of<T, 16, 1, FLOW>(win, heun, corr);
-        case 16 * 16 + 2: return chunk_of<T, 16, 2, FLOW>(win, heun, corr);
-        case 16 * 16 + 3: return chunk_of<T, 16, 3, FLOW>(win, heun, corr);
-        case 16 * 16 + 4: return chunk_of<T, 16, 4, FLOW>(win, heun, corr);
-        case 32 * 16 + 3: return chunk_of<T, 32, 3, FLOW>(win, heun, corr);
-        case 32 * 16 + 4: return chunk_of<T, 32, 4, FLOW>(win, heun, corr);
+        case 8 * 16 + 1: return chunk_of<T, 8, 1, FLOW, false>(win, heun, corr);
+        case 8 * 16 + 2: return chunk_of<T, 8, 2, FLOW, false>(win, heun, corr);
+        case 8 * 16 + 3: return chunk_of<T, 8, 3, FLOW, false>(win, heun, corr);
+        case 16 * 16 + 1: return chunk_of<T, 16, 1, FLOW, false>(win, heun, corr);
+        case 16 * 16 + 2: return chunk_of<T, 16, 2, FLOW, false>(win, heun, corr);
+        case 16 * 16 + 3: return chunk_of<T, 16, 3, FLOW, false>(win, heun, corr);
+        case 16 * 16 + 4: return chunk_of<T, 16, 4, FLOW, false>(win, heun, corr);
+        case 32 * 16 + 3: return chunk_of<T, 32, 3, FLOW, false>(win, heun, corr);
+        case 32 * 16 + 4: return chunk_of<T, 32, 4, FLOW, false>(win, heun, corr);
         default: return nullptr;
     }
 }

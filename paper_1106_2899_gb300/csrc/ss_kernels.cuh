@@ -317,17 +317,23 @@ constexpr int kChunkThreads = 32;
 constexpr int kCounterCopies = 64;  // power of two
 // Resident warps per SM the kernels are compiled for.  Two beads per lane fit 96
 // registers; three or more need 128 (N = 40, 65536 chains: 26.4 us per step at 16
-// warps, 28.8 at 20 with the spills of 96 registers).  Sixteen lanes of four beads
-// spill 136-188 bytes at 128 registers and none at 168 (N = 62, 9000 chains, 400
-// steps: 2.97 -> 2.67 ms; N = 56, 16000 chains: 4.62 -> 4.20) and take 254 with Heun
-// and flow (N = 50, 1000 chains: 1.53 -> 1.35 ms); Heun without flow stays at 128,
-// since at 168 the compiler contracts its sums in another order and the results
-// differ in the last bits.  FP64 work is bound by the
+// warps, 28.8 at 20 with the spills of 96 registers).  FP64 work is bound by the
 // FP64 pipe long before twelve warps.
+//
+// Sixteen lanes of four beads (N = 49..64) spill 136-188 bytes at 128 registers and none
+// at 168 (N = 62, 9000 chains, 400 steps: 2.97 -> 2.67 ms; N = 56, 16000 chains: 4.62 ->
+// 4.20), but 12 warps/SM take a second wave for what 16 take in one.  So the chain
+// kernel has two forms there (ALT the second), which give the same bits, and the host
+// takes the better one by the waves of an ensemble (four_bead_alt).
+//   Euler-Maruyama   12 warps, or 16 with reduction batches of two steps
+//   Heun             128 registers, batches of five steps (13 warps by shared memory) or
+//                    of two (16); with 168 registers the compiler contracts its sums in
+//                    another order and the results differ in the last bits
+//   Heun with flow   10 warps (168 registers, of which 12 fit), or 8 without spills
 template <typename T>
-constexpr int chunk_warps_per_sm(int W, int B, bool heun = false, bool flow = false) {
+constexpr int chunk_warps_per_sm(int W, int B, bool heun = false, bool flow = false, bool alt = false) {
     if (sizeof(T) == 8) return heun && flow ? 8 : 12;
-    if (W == 16 && B == 4 && !(heun && !flow)) return heun ? 8 : 12;
+    if (W == 16 && B == 4) return heun && flow ? (alt ? 8 : 10) : (heun || alt ? 16 : 12);
     if (heun && flow) return B == 1 ? 20 : (B == 2 ? 16 : 12);  // both states live at once
     return B == 1 ? 24 : (B == 2 ? 20 : 16);
 }
@@ -353,22 +359,27 @@ struct SmemPlan {
 // with its selects and its five dependent rounds, took 12 instructions per
 // warp-step more.)
 constexpr int kRedSteps = 5;
+// of a chain kernel whose stress series may be written (0: FP64, no batches)
+template <typename T>
+constexpr int red_steps(int W, int B, bool heun, bool flow, bool alt) {
+    return sizeof(T) == 8 ? 0 : (alt && !(heun && flow) ? 2 : kRedSteps);
+}
 // Rows of W + 4 words, so that eight lanes reading 16 bytes of eight rows each
 // cover every bank once; the chains of a warp lie W words (mod 32) apart, so that
 // the 32 lanes writing one value of each do, too.
 __host__ __device__ constexpr int red_row(int W) { return W + 4; }
-__host__ __device__ constexpr int red_chain(int W) {
-    const int n = kRedSteps * 6 * red_row(W), pad = (W - n % 32 + 32) % 32;
+__host__ __device__ constexpr int red_chain(int W, int steps) {
+    const int n = steps * 6 * red_row(W), pad = (W - n % 32 + 32) % 32;
     return n + (W == 32 ? 0 : pad);
 }
 
-// series: a stress series may be written.  Without one nothing touches the reduction
-// buffer, a third of the shared memory of a CTA: left out, the batched kernel and the
+// red: steps of a reduction batch, 0 without a stress series.  Nothing touches the
+// reduction buffer then, a third of the shared memory of a CTA: left out, the batched kernel and the
 // chain kernel without the correlator run the warps their registers are planned for
 // (16 x 2 with 11 log steps: 17 and 18 warps/SM -> 20; 512 elements, 1000 steps: 57.4 ->
 // 52.3 ms, six ensembles of 4096 x 40 under shear: 11.1 -> 10.7 ms).
 template <typename T>
-__host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_chunk, bool series) {
+__host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_chunk, int red) {
     SmemPlan p;
     const int chains = warps * (32 / W), NL = W * B;
     p.off_rec = 0;
@@ -383,7 +394,7 @@ __host__ __device__ inline SmemPlan smem_plan(int warps, int W, int B, int nlog_
     p.off_msk = (sz + 15) & ~15;
     sz = p.off_msk + chains * NL * (int)(NL <= 32 ? sizeof(unsigned) : sizeof(unsigned long long));
     p.off_red = (sz + 15) & ~15;
-    sz = p.off_red + (series && sizeof(T) == 4 ? chains * red_chain(W) * (int)sizeof(T) : 0);
+    sz = p.off_red + (red > 0 ? chains * red_chain(W, red) * (int)sizeof(T) : 0);
     p.off_kap = (sz + 15) & ~15;
     sz = p.off_kap + warps * 3 * (int)sizeof(Pos<T>);
     p.off_log = (sz + 15) & ~15;
@@ -597,11 +608,11 @@ __device__ __forceinline__ KappaState kappa_at(Args& a, int ki, long long t0, in
 // the element described by `a` (all warps of the CTA call this together).
 // FLOW: the velocity-gradient terms are compiled in (without them the launch
 // must have kappa = 0 throughout; recentring is then never needed).  CORR: the
-// stress series is compiled in.  VL = 2: eight lanes do the work of sixteen.
+// stress series is compiled in, its samples reduced RED steps at a time.  VL = 2: eight lanes do the work of sixteen.
 // Sub-slots of even and of odd b are the beads of lanes l and l + 8 of a 16-lane
 // segment; summing them apart and adding the two is the first round of that
 // segment's reduction, so every sum over beads is rounded as there.
-template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, int VL, typename Args>
+template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, int VL, int RED, typename Args>
 __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const int cta_first,
                                            const T NkT, const long long t0_, const int nsteps_,
                                            const long long log_m0_, const int nlog_) {
@@ -637,7 +648,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     const unsigned lt = ((1u << lane) - 1u) & segmask;  // lanes of this segment below this one
 
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemPlan plan = smem_plan<T>(nwarps, W, B, nlog_, CORR);
+    const SmemPlan plan = smem_plan<T>(nwarps, W, B, nlog_, RED);
     // spring records of this chain: [0, NL) the first spring of each bead, [NL, 2 NL)
     // the second (zeros where there is none), [2 NL, 3 NL) by slot: springs beyond
     // the second of a bead, and scratch of the re-indexing
@@ -651,7 +662,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // whose corrector rounds the bond force from it
     Pos<T>* bq = reinterpret_cast<Pos<T>*>(smem + plan.off_bq) + cslot * (NL + 1);
     Mask* msk = reinterpret_cast<Mask*>(smem + plan.off_msk) + cslot * NL;
-    [[maybe_unused]] T* const red = reinterpret_cast<T*>(smem + plan.off_red) + warp * SEGS * red_chain(W);
+    [[maybe_unused]] T* const red = reinterpret_cast<T*>(smem + plan.off_red) + warp * SEGS * red_chain(W, RED);
     double* slog = reinterpret_cast<double*>(smem + plan.off_log);
 
     for (int i = threadIdx.x; i < nlog_ * 14; i += blockDim.x) slog[i] = 0.0;
@@ -757,7 +768,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // chain, W lane parts summed in pairs as the butterflies of seg_reduce6 pair
     // the lanes.
     [[maybe_unused]] int red_n = 0;  // steps waiting
-    [[maybe_unused]] T* red_w = red + seg * red_chain(W) + ll;
+    [[maybe_unused]] T* red_w = red + seg * red_chain(W, RED) + ll;
     [[maybe_unused]] auto red_put = [&](const T (&v)[6]) {
 #pragma unroll
         for (int q = 0; q < 6; ++q) red_w[q * red_row(W)] = v[q];
@@ -767,7 +778,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         const int rows = 6 * red_n;  // of each chain
         for (int r = lane; r < rows * SEGS; r += 32) {
             const int ch = SEGS == 1 ? 0 : r / rows, rr = r - ch * rows;
-            const float4* row = reinterpret_cast<const float4*>(red + ch * red_chain(W) + rr * red_row(W));
+            const float4* row = reinterpret_cast<const float4*>(red + ch * red_chain(W, RED) + rr * red_row(W));
             float4 x[W / 4];
 #pragma unroll
             for (int k = 0; k < W / 4; ++k) x[k] = row[k];
@@ -786,7 +797,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             if (m < a.M) ser[((size_t)(a.series_row0 + s_end - red_n + st) * a.M + m) * 6 + q] = sum;
         }
         red_n = 0;
-        red_w = red + seg * red_chain(W) + ll;
+        red_w = red + seg * red_chain(W, RED) + ll;
     };
     if (nlog_ > 0)
         __syncthreads();  // the CTA's stress-log buffer is zeroed
@@ -1531,7 +1542,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
         }
         __syncwarp();
         if constexpr (sizeof(T) == 4) {
-            if (corr_on && ++red_n == kRedSteps) red_flush(s + 1);
+            if (corr_on && ++red_n == RED) red_flush(s + 1);
         }
     }
     if (!FLOW || s >= nsteps_) break;
@@ -1618,12 +1629,12 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 // velocity-gradient terms are compiled in (launches with kappa = 0 throughout
 // may use the instantiation without them).  HEUN: the stochastic Heun
 // integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
-// be written (without one, its registers are free).
-template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR>
-__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B, HEUN, FLOW))
+// be written (without one, its registers are free).  ALT: the second form of 16 x 4.
+template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, bool ALT = false>
+__global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B, HEUN, FLOW, ALT))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
-    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1>(a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0,
-                                         a.nlog_chunk);
+    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1, CORR ? red_steps<T>(W, B, HEUN, FLOW, ALT) : 0>(
+        a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0, a.nlog_chunk);
 }
 
 // ------------------------------------------------------ batched kernel ------
@@ -1657,8 +1668,8 @@ __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B))
     // The centre of mass, the only sum over beads that enters a state, is the same
     // either way.
     constexpr int VL = W == 8 && B != 2 ? 2 : 1;
-    run_chains<T, W, B, kWinOff, true, false, false, VL>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
-                                                     info.log_m0, nlog);
+    run_chains<T, W, B, kWinOff, true, false, false, VL, 0>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
+                                                        info.log_m0, nlog);
 }
 
 }  // namespace ssk

@@ -7,13 +7,14 @@
 
 namespace ssk {
 
-// chunk_kernel<T, W, B, win, FLOW, heun, corr>, launched with (ChunkArgs,
-// StepConst<T>); null for a layout that is not compiled.  Windows (win != kWinOff)
+// chunk_kernel<T, W, B, win, FLOW, heun, corr, alt>, launched with (ChunkArgs,
+// StepConst<T>); null for a layout that is not compiled, the first form where there is
+// no second.  Windows (win != kWinOff)
 // run the Euler-Maruyama step without flow.
-const void* chunk_fn_f32(int W, int B, int win, bool heun, bool corr);
-const void* chunk_fn_f32_flow(int W, int B, int win, bool heun, bool corr);
-const void* chunk_fn_f64(int W, int B, int win, bool heun, bool corr);
-const void* chunk_fn_f64_flow(int W, int B, int win, bool heun, bool corr);
+const void* chunk_fn_f32(int W, int B, int win, bool heun, bool corr, bool alt);
+const void* chunk_fn_f32_flow(int W, int B, int win, bool heun, bool corr, bool alt);
+const void* chunk_fn_f64(int W, int B, int win, bool heun, bool corr, bool alt);
+const void* chunk_fn_f64_flow(int W, int B, int win, bool heun, bool corr, bool alt);
 // batched_kernel<T, W, B>
 const void* batched_fn_f32(int W, int B);
 const void* batched_fn_f64(int W, int B);

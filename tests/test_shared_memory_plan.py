@@ -22,11 +22,17 @@ int main() {
     const int lay[][2] = {{8, 1}, {8, 2}, {8, 3}, {16, 1}, {16, 2}, {16, 3}, {16, 4}, {32, 1}, {32, 3}, {32, 4}};
     for (auto& l : lay)
         for (int logs : {0, 11, 16})
-            for (int series = 0; series < 2; ++series)
+            for (int series = 0; series < 2; ++series) {
+                const int red = series ? red_steps<float>(l[0], l[1], false, true, false) : 0;
+                const int bytes = smem_plan<float>(1, l[0], l[1], logs, red).total;
                 std::printf("%d %d %d %d %d %d %d\n", l[0], l[1], logs, series,
-                            chunk_warps_per_sm<float>(l[0], l[1], false, true),
-                            ctas_by_smem(smem_plan<float>(1, l[0], l[1], logs, series).total),
-                            ctas_by_smem(smem_plan<float>(1, l[0], l[1], logs, series).total + (int)sizeof(ChunkArgs)));
+                            chunk_warps_per_sm<float>(l[0], l[1], false, true), ctas_by_smem(bytes),
+                            ctas_by_smem(bytes + (int)sizeof(ChunkArgs)));
+            }
+    // the second form of 16 x 4 (Euler-Maruyama, Heun), with a series
+    for (int heun = 0; heun < 2; ++heun)
+        std::printf("16 4 -1 %d %d %d 0\n", heun, chunk_warps_per_sm<float>(16, 4, heun, false, true),
+                    ctas_by_smem(smem_plan<float>(1, 16, 4, 0, red_steps<float>(16, 4, heun, false, true)).total));
 }
 """
 
@@ -44,9 +50,9 @@ def table(tmp_path_factory):
 
 
 def test_without_a_series_registers_decide(table):
-    assert len(table) == 60
+    assert len(table) == 62
     for (w, b, logs, series), (regs, chunk, batched) in table.items():
-        if not series:
+        if logs >= 0 and not series:
             assert chunk >= regs and batched >= regs, (w, b, logs)
 
 
@@ -56,3 +62,5 @@ def test_with_a_series(table):
     for (w, b, logs, series), (regs, chunk, _) in table.items():
         if series and logs == 0:
             assert chunk >= least.get((w, b), regs), (w, b)
+    for heun in (0, 1):
+        assert table[16, 4, -1, heun][:2] == (16, 16)
