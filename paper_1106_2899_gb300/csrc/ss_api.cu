@@ -84,6 +84,7 @@ struct ss_ctx {
     size_t logs_n = 0;
     std::vector<double> logs_host;  // what the last read copied back
     bool logs_read = false;         // logs_host holds the whole block as it is now
+    bool logs_captured = false;     // a graph that writes the logs was captured: its replays are not seen here
     void* stage = nullptr;  // device staging for state uploads and correlator readout
     size_t stage_bytes = 0;
     long long launches = 0;
@@ -187,17 +188,27 @@ void free_logs(ss_ctx* c) {
     if (c->logs) cudaFree(c->logs);
     c->logs = nullptr;
     c->logs_n = 0;
-    c->logs_read = false;
+    c->logs_read = c->logs_captured = false;
     for (Elem& e : c->el) e.logs = nullptr;
+}
+
+// Work that changes the logs is about to be enqueued: what was read of them is out of
+// date, and stays so from read to read once the stream is captured into a graph.
+int logs_change(ss_ctx* c) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (c->logs) SS_CUDA(c, cudaStreamIsCapturing(c->stream, &st));
+    if (st != cudaStreamCaptureStatusNone) c->logs_captured = true;
+    c->logs_read = false;
+    return SS_OK;
 }
 
 // The first n stress logs of an element on the host.  The logs of several elements
 // are usually read one after another, so a block of up to kLogBlockBytes comes over
 // in one copy and stays until the next run or reset (512 elements: 512 copies and
-// synchronisations took 7 ms).
+// synchronisations took 7 ms), but for a context whose runs were captured into a graph.
 constexpr size_t kLogBlockBytes = 4 << 20;
 int read_logs(ss_ctx* c, const Elem& e, int n, const double** out) {
-    const bool all = c->el.size() > 1 && c->logs_n * sizeof(double) <= kLogBlockBytes;
+    const bool all = c->el.size() > 1 && !c->logs_captured && c->logs_n * sizeof(double) <= kLogBlockBytes;
     const size_t first = (size_t)(e.logs - c->logs), count = (size_t)n * e.groups * 14;
     if (!all || !c->logs_read) {
         c->logs_host.resize(all ? c->logs_n : count);
@@ -587,8 +598,8 @@ int zero_observables(ss_ctx* c) {
             SS_CUDA(c, cudaMemsetAsync(e.acc64tt, 0, (size_t)e.slices * e.parts * c->levels * 48 * sizeof(double),
                                        c->stream));
     }
+    if (const int rl = logs_change(c)) return rl;
     if (c->logs) SS_CUDA(c, cudaMemsetAsync(c->logs, 0, c->logs_n * sizeof(double), c->stream));
-    c->logs_read = false;
     c->nsamp = 0;
     c->log_m0 = c->P.log_every > 0 ? c->step / c->P.log_every : 0;
     return SS_OK;
@@ -1466,7 +1477,7 @@ int ss_run(ss_ctx* c, int64_t n_steps) {
         const long long nlog = (c->step + n_steps) / p.log_every - c->log_m0;
         if (nlog > p.max_logs) return fail(c, SS_EINVAL, "stress log capacity (max_logs) exceeded");
     }
-    c->logs_read = false;
+    if (const int rl = logs_change(c)) return rl;
     for (Elem& e : c->el) {
         int rc = upload_flow(c, e);
         if (rc != SS_OK) return rc;
