@@ -7,9 +7,11 @@ namespace {
 
 template <typename T>
 const void* adjoint_fn(int W, int B) {
+    if constexpr (sizeof(T) == 4) {  // FP64 windows of that length run 16 x 2
+        if (W == 8 && B == 3) return (const void*)adjoint_kernel<T, 8, 3>;
+    }
     switch (W * 16 + B) {
         case 8 * 16 + 1: return (const void*)adjoint_kernel<T, 8, 1>;
-        case 8 * 16 + 3: return (const void*)adjoint_kernel<T, 8, 3>;
         case 16 * 16 + 1: return (const void*)adjoint_kernel<T, 16, 1>;
         case 16 * 16 + 2: return (const void*)adjoint_kernel<T, 16, 2>;
         case 16 * 16 + 3: return (const void*)adjoint_kernel<T, 16, 3>;

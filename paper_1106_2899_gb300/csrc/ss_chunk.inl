@@ -6,15 +6,22 @@
 namespace ssk {
 namespace {
 
+// 8 x 2 and 8 x 3 serve FP32 runs of the Euler-Maruyama step alone (layout_for)
+template <int W, int B>
+constexpr bool kNarrow = W == 8 && B > 1;
+
 template <typename T, int W, int B, bool FLOW, bool ALT>
 const void* chunk_of(int win, bool heun, bool corr) {
     if constexpr (!FLOW) {
         if (win == kWinRecord) return (const void*)chunk_kernel<T, W, B, kWinRecord, false, false, true>;
         if (win == kWinReplay) return (const void*)chunk_kernel<T, W, B, kWinReplay, false, false, true>;
     }
-    if (heun)  // (without a flow and a series both forms are the same)
+    if constexpr (kNarrow<W, B>) {
+        if (heun) return nullptr;
+    } else if (heun) {  // (without a flow and a series both forms are the same)
         return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, true, ALT>
                     : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, true, false, ALT && FLOW>;
+    }
     return corr ? (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, true, ALT>
                 : (const void*)chunk_kernel<T, W, B, kWinOff, FLOW, false, false, ALT>;
 }
@@ -23,11 +30,11 @@ template <typename T, bool FLOW>
 const void* chunk_fn(int W, int B, int win, bool heun, bool corr, bool alt) {
     if constexpr (sizeof(T) == 4) {
         if (alt && W == 16 && B == 4 && win == kWinOff) return chunk_of<T, 16, 4, FLOW, true>(win, heun, corr);
+        if (W == 8 && B == 2) return chunk_of<T, 8, 2, FLOW, false>(win, heun, corr);
+        if (W == 8 && B == 3) return chunk_of<T, 8, 3, FLOW, false>(win, heun, corr);
     }
     switch (W * 16 + B) {
         case 8 * 16 + 1: return chunk_of<T, 8, 1, FLOW, false>(win, heun, corr);
-        case 8 * 16 + 2: return chunk_of<T, 8, 2, FLOW, false>(win, heun, corr);
-        case 8 * 16 + 3: return chunk_of<T, 8, 3, FLOW, false>(win, heun, corr);
         case 16 * 16 + 1: return chunk_of<T, 16, 1, FLOW, false>(win, heun, corr);
         case 16 * 16 + 2: return chunk_of<T, 16, 2, FLOW, false>(win, heun, corr);
         case 16 * 16 + 3: return chunk_of<T, 16, 3, FLOW, false>(win, heun, corr);

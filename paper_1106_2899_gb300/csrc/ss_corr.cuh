@@ -28,7 +28,7 @@ namespace ssk {
 // [parts][L][3][32] (component, channel * 16 + lag).  With TT the rows of
 // sigma + sigma^(v) also take their own samples as the later value (channel TT,
 // acc64tt [parts][L][3][16]).
-constexpr int kCorrMaxSteps = 1024;  // samples per launch (the level-sample buffers hold half)
+constexpr int kCorrMaxSteps = 1024;  // samples per launch (the level-sample buffers hold a quarter)
 constexpr int kCorrPartChains = 32;  // chains per CTA at most, but for callers that keep one sum per slice
 
 // Chains per CTA: 32 in seven warps, or, in ensembles too small to fill the chip
