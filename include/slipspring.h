@@ -102,9 +102,9 @@ typedef struct {
     int32_t corr_levels;    /* multiple-tau levels, 1..SS_MAX_LEVELS [24]; < 0: none      */
     int32_t groups;         /* chain groups per element for standard errors [32]         */
     int32_t chunk_steps;    /* steps per kernel launch [1024]; 1 gives the plain
-                               one-step-per-launch form.  The chain kernel takes no more
-                               than 16 log steps per launch and is launched again for
-                               the rest of such a chunk.  With the correlator on, a
+                               one-step-per-launch form.  A chunk with many log steps
+                               may be several launches of the chain kernel (at least 16
+                               log steps each).  With the correlator on, a
                                launch covers at most 1024 steps (larger values are
                                reduced to 1024): the launch's stress series, 24 B per
                                chain and step in FP32, is what the correlator reads.

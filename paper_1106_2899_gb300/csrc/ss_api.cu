@@ -94,6 +94,7 @@ struct ss_ctx {
     bool batched = false;
     bool tuned = false;
     bool graph_dirty = true;
+    int batch_logs = 0;  // log steps of a launch at most
     ssk::ChunkArgs* d_elems = nullptr;
     int2* d_items = nullptr;
     std::vector<BatchedClass> bclasses;
@@ -408,22 +409,37 @@ bool flow_in_window(const Elem& e, long long t0, int nsteps) {
     return false;
 }
 
-// Stress-log steps of one chain-kernel launch at most.  Every CTA keeps 112 bytes per
-// log step of its launch in shared memory, and CTAs are single warps: a launch with
-// many log steps would leave room for few of them on an SM (N = 32: 20 without logs,
-// 17 with 16, 10 with 103, one with 1024).  Such a chunk is split into launches (us per
-// step of 65536 x 32 under shear, log_every 10 / 1: 27.2 / 685 unsplit, 19.3 / 86.1 at
-// 16 log steps, 20.5 / 86.3 at 32; 4096 x 40: 3.7 / 49.6, 2.7 / 6.8, 3.6 / 9.6).  The sums
-// of every warp enter device memory by FP64 atomics, which bound a log at every step.
+// Stress-log steps of one launch of the chain kernel at most.  Every CTA keeps 112 bytes
+// per log step of its launch in shared memory, and CTAs are single warps: a launch with
+// many log steps would leave room for few of them on an SM (N = 32: 20 without logs, 17
+// with 16, 10 with 103, one with 1024).  Where a context's warps do not fit the chip at
+// once, a chunk is split into launches of 16 log steps (us per step of 65536 x 32 under
+// shear, log_every 10 / 1: 27.2 / 685 unsplit, 19.3 / 86.1 at 16 log steps, 20.5 / 86.3 at
+// 32).  A smaller context takes as many as leave room for its warps: it is bound by
+// latency, and a launch costs it some steps' time (256 x 16, log_every 1: 3.25 us per
+// step with 16 log steps per launch, 2.85 with 1024; 4096 x 40: 49.6 unsplit, 6.8 with 16
+// log steps, 6.4 with the 62 that fit).  The sums of every warp enter device
+// memory by FP64 atomics, which bound a log at every step of a large ensemble.
 constexpr int kLaunchLogs = 16;
-// steps from t on, n at most, with no more log steps than that
-int log_bounded_steps(const ss_params& p, long long t, int n) {
-    if (p.log_every <= 0) return n;
-    return (int)std::min<long long>(n, (t / p.log_every + kLaunchLogs + 1) * p.log_every - 1 - t);
+// bytes0: shared memory of a CTA without logs
+int launch_logs(const ss_ctx* c, int bytes0) {
+    long long warps = 0;
+    for (const Elem& e : c->el) warps += ((long long)e.M * e.W + 31) / 32;
+    const long long per_sm = std::max(1ll, (warps + c->sms - 1) / c->sms);
+    const long long room = 228 * 1024 / per_sm / 128 * 128 - 1024 - bytes0;
+    return (int)std::max<long long>(kLaunchLogs, room / 112);
 }
-
-int logs_per_launch(const ss_ctx* c) {
-    return c->P.log_every > 0 ? std::min(kLaunchLogs, c->P.chunk_steps / c->P.log_every + 1) : 0;
+// steps from t on, n at most, with no more than `logs` log steps
+int log_bounded_steps(const ss_params& p, long long t, int n, int logs) {
+    if (p.log_every <= 0) return n;
+    return (int)std::min<long long>(n, (t / p.log_every + logs + 1) * p.log_every - 1 - t);
+}
+// log steps of the longest launch over an element
+template <typename T>
+int logs_per_launch(const ss_ctx* c, const Elem& e, bool flow, bool heun, bool series) {
+    if (c->P.log_every <= 0) return 0;
+    return std::min(launch_logs(c, chunk_smem<T>(e.W, e.B, 0, flow, heun, series, false)),
+                    c->P.chunk_steps / c->P.log_every + 1);
 }
 
 template <typename T>
@@ -491,8 +507,8 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     // (the window kernels have the series compiled in, also for a replay without it)
     const bool flow = flow_in_window(e, t0, nsteps), heun = c->P.integrator == SS_HEUN;
     const bool series = corr || win != ssk::kWinOff;
-    const bool alt =
-        win == ssk::kWinOff && four_bead_alt<T>(e.M, e.W, e.B, c->sms, logs_per_launch(c), flow, heun, series);
+    const int max_logs = logs_per_launch<T>(c, e, flow, heun, series);
+    const bool alt = win == ssk::kWinOff && four_bead_alt<T>(e.M, e.W, e.B, c->sms, max_logs, flow, heun, series);
     const void* kern = chunk_fn<T>(e.W, e.B, win, flow, heun, corr, alt);
     if (!kern) return fail(c, SS_EINVAL, "no chain kernel for this layout");
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
@@ -502,7 +518,7 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     const long long row0 = a.series_row0;
     for (int done = 0; done < nsteps; done += a.nsteps) {
         a.t0 = t0 + done;
-        a.nsteps = a.log_every > 0 ? log_bounded_steps(p, a.t0, nsteps - done) : nsteps - done;
+        a.nsteps = a.log_every > 0 ? log_bounded_steps(p, a.t0, nsteps - done, max_logs) : nsteps - done;
         a.series_row0 = row0 + done;
         a.nlog_chunk = a.log_every > 0 ? (int)((a.t0 + a.nsteps) / a.log_every - a.t0 / a.log_every) : 0;
         const int smem = chunk_smem<T>(e.W, e.B, a.nlog_chunk, flow, heun, series, alt);
@@ -797,9 +813,10 @@ const void* batched_fn_of(int k) {
     return sizeof(T) == 8 ? ssk::batched_fn_f64(kLayoutW[k], kLayoutB[k]) : ssk::batched_fn_f32(kLayoutW[k], kLayoutB[k]);
 }
 
+// shared memory of a class beside the kernel's own copy of an element's arguments
 template <typename T>
-int batched_smem_bytes(const ss_ctx* c, int k) {
-    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], logs_per_launch(c), 0).total;
+int batched_smem_bytes(int k, int nlog) {
+    return ssk::smem_plan<T>(kWarpsPerCta, kLayoutW[k], kLayoutB[k], nlog, 0).total;
 }
 
 template <typename T>
@@ -917,7 +934,7 @@ int autotune(ss_ctx* c) {
                     ssk::ChunkArgs desc = make_desc(c, t);
                     desc.counters = dcnt;
                     desc.status = reinterpret_cast<int32_t*>(dcnt + 8 * ssk::kCounterCopies);
-                    const int smem = batched_smem_bytes<T>(c, k);
+                    const int smem = batched_smem_bytes<T>(k, 0);
                     SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                     smem));
                     SS_CUDA(c, cudaMemcpy(dd, &desc, sizeof(desc), cudaMemcpyHostToDevice));
@@ -983,6 +1000,14 @@ int batched_prepare(ss_ctx* c) {
     SS_CUDA(c, cudaMalloc(&c->d_items, sizeof(int2) * std::max<size_t>(1, total)));
     SS_CUDA(c, cudaMemcpy(c->d_elems, descs.data(), sizeof(ssk::ChunkArgs) * descs.size(), cudaMemcpyHostToDevice));
     SS_CUDA(c, cudaGraphCreate(&c->graph, 0));
+    c->batch_logs = 0;
+    if (c->P.log_every > 0) {
+        c->batch_logs = c->P.chunk_steps / c->P.log_every + 1;
+        for (int k = 0; k < kBatchedLayouts; ++k)
+            if (!cls[k].empty())
+                c->batch_logs = std::min(
+                    c->batch_logs, launch_logs(c, batched_smem_bytes<T>(k, 0) + (int)sizeof(ssk::ChunkArgs)));
+    }
     size_t off = 0;
     for (int k = 0; k < kBatchedLayouts; ++k) {
         if (cls[k].empty()) continue;
@@ -991,7 +1016,7 @@ int batched_prepare(ss_ctx* c) {
         bc.k = k;
         bc.items = c->d_items + off;
         bc.n_items = (int)cls[k].size();
-        bc.smem = batched_smem_bytes<T>(c, k);
+        bc.smem = batched_smem_bytes<T>(k, c->batch_logs);
         SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, bc.smem));
         ssk::RunInfo info{0, 1, 0};
         ssk::StepConst<T> sc = step_const<T>(c, 32);
@@ -1046,7 +1071,8 @@ int batched_run(ss_ctx* c, long long n_steps) {
     }
     long long left = n_steps;
     while (left > 0) {
-        const int ns = log_bounded_steps(c->P, c->step, (int)std::min<long long>(left, c->P.chunk_steps));
+        const int ns =
+            log_bounded_steps(c->P, c->step, (int)std::min<long long>(left, c->P.chunk_steps), c->batch_logs);
         int rc = batched_chunk<T>(c, c->step, ns);
         if (rc != SS_OK) return rc;
         c->step += ns;
@@ -1236,7 +1262,7 @@ int order_streams(ss_ctx* c, cudaStream_t first, cudaStream_t later) {
 template <typename T>
 int resident_warps(const ss_ctx* c, const Elem& e, bool flow) {
     const bool heun = c->P.integrator == SS_HEUN, series = c->levels > 0;
-    const int nlog = logs_per_launch(c);
+    const int nlog = logs_per_launch<T>(c, e, flow, heun, series);
     const bool alt = four_bead_alt<T>(e.M, e.W, e.B, c->sms, nlog, flow, heun, series);
     return chunk_resident<T>(e.W, e.B, nlog, flow, heun, series, alt);
 }

@@ -47,3 +47,42 @@ def test_first_chains_are_the_same_in_any_ensemble(cuda_ok, N, flow, integrator,
         if levels > 0:  # FP64 sums of a slice's parts, 16 or 32 chains each
             assert np.allclose(a, acc, rtol=1e-13, atol=1e-13 * np.abs(acc).max())
         assert np.allclose(lg, log, rtol=1e-12, atol=1e-9)
+
+
+@pytest.mark.parametrize("flow", [False, True])
+@pytest.mark.parametrize("levels", [-1, 2])
+def test_allocation_free_call(cuda_ok, flow, levels):
+    import ctypes
+
+    import torch
+    from paper_1106_2899_gb300 import _native as nat
+    from test_zz_no_alloc import _from_device_layout, _to_device_layout
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    M, N, n = 28 * sms, 61, 33
+    zm = N
+    st0 = synth.random_state(M, N, zm, seed=3, z_mean=N / 4)
+    kappa = np.ascontiguousarray(synth.shear_kappa(0.05 if flow else 0.0))
+    g = SlipSpring([(M, N)], precision="fp32", seed=8)
+    g.set_params(**synth.PAPER, corr_levels=levels)
+    g.set_state(st0)
+    if flow:
+        g.set_flow(kappa, 0)
+    g.run(n)
+    ref = g.get_state()
+    g.close()
+    p = nat.ss_params()
+    for k, v in synth.PAPER.items():
+        setattr(p, k, v)
+    p.corr_levels = levels
+    dev = [torch.from_numpy(x).cuda() for x in _to_device_layout(st0, N, zm, np.float32)]
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ptr = [ctypes.c_void_p(x.data_ptr()) for x in dev]
+    rc = nat.load().ss_run_noalloc(ctypes.byref(p), nat.SS_FP32, 8, M, N, 0, 0, n,
+                                   kappa.ctypes.data_as(ctypes.POINTER(ctypes.c_double)), *ptr, None,
+                                   ctypes.c_void_p(status.data_ptr()),
+                                   ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    torch.cuda.synchronize()
+    assert rc == 0 and int(status.item()) == 0
+    got = _from_device_layout(*[x.cpu().numpy() for x in dev], N, zm)
+    for k in ("Z", "S", "R", "A"):
+        assert np.array_equal(got[k], ref[k]), k
