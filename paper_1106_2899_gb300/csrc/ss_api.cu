@@ -274,23 +274,25 @@ int chunk_resident(int W, int B, int nlog, bool flow, bool heun, bool series, bo
     return std::min(ssk::chunk_warps_per_sm<T>(W, B, heun, flow, alt),
                     ssk::ctas_by_smem(chunk_smem<T>(W, B, nlog, flow, heun, series, alt)));
 }
-// Whether M chains of 49..64 beads (16 x 4) run the second form of the chain kernel.
-// Euler-Maruyama and Heun without a flow: more warps per SM do the same work per time,
-// or a little less, but may save a wave (us of 400 steps, first / second form: 4000 x 60,
-// 13.2 warps per SM, Euler-Maruyama 1516 / 1335, with shear 1592 / 1355, Heun 2104 /
-// 1740; 9000 x 62, 29.6 per SM: 2578 / 2640, 2718 / 2680, 3852 / 3490; 2500 x 52: 951 / 1079,
-// 1001 / 1145, 1376 / 1420).  Heun with flow: the first form does more per time (30000 x
-// 60: 15.1 / 17.4 ms; 3000 x 60: 1.87 / 2.53), the second is faster in one wave of its
-// own and in two where the first, of whose warps 12 fit an SM, takes two as well
-// (2300 x 60: 1.67 / 1.59; 3500 x 60: 1.97 / 2.69; 4000 x 60: 2.98 / 2.77).
+// Whether M chains of a layout run the second form of the chain kernel: by the waves of
+// warps that each form takes.  More warps per SM do the same work per time, or a little
+// less, but may save a wave (first / second form, N = 49..64, us of 400 steps: 4000 x 60,
+// 13.2 warps per SM, Euler-Maruyama 1516 / 1335, with shear 1592 / 1355, Heun 2104 / 1740;
+// 9000 x 62, 29.6 per SM: 2578 / 2640, 2718 / 2680, 3852 / 3490; 2500 x 52: 951 / 1079, 1001 /
+// 1145, 1376 / 1420; 300 steps with shear: 6000 x 48, 19.7 per SM, 1147 / 948; 10200 x 24
+// 1034 / 892; Heun 6000 x 32 985 / 884, 4400 x 48 1642 / 1319).  At N = 49..64 Heun with flow
+// has more warps in the first form, which does more per time (30000 x 60: 15.1 / 17.4 ms;
+// 3000 x 60: 1.87 / 2.53); the second is faster in one wave of its own and in two where the
+// first, of whose warps 12 fit an SM, takes two as well (2300 x 60: 1.67 / 1.59; 3500 x 60:
+// 1.97 / 2.69; 4000 x 60: 2.98 / 2.77).
 template <typename T>
-bool four_bead_alt(int M, int W, int B, int sms, int nlog, bool flow, bool heun, bool series) {
-    if (sizeof(T) == 8 || W != 16 || B != 4) return false;
-    const int warps = (M + 1) / 2;
+bool second_form(int M, int W, int B, int sms, int nlog, bool flow, bool heun, bool series) {
+    if (sizeof(T) == 8 || !ssk::has_second_form(W, B, heun, flow)) return false;
+    const long long warps = ((long long)M * W + 31) / 32;
     const int a = sms * chunk_resident<T>(W, B, nlog, flow, heun, series, false);
     const int b = sms * chunk_resident<T>(W, B, nlog, flow, heun, series, true);
-    if (heun && flow) return warps <= b || (warps > 12 * sms && warps <= 2 * b);
-    const auto cost = [&](int slots) { return (long long)((warps + slots - 1) / slots) * slots; };
+    if (B == 4 && heun && flow) return warps <= b || (warps > 12 * sms && warps <= 2 * b);
+    const auto cost = [&](int slots) { return (warps + slots - 1) / slots * slots; };
     return cost(b) * 23 < cost(a) * 20;
 }
 
@@ -508,7 +510,9 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
     const bool flow = flow_in_window(e, t0, nsteps), heun = c->P.integrator == SS_HEUN;
     const bool series = corr || win != ssk::kWinOff;
     const int max_logs = logs_per_launch<T>(c, e, flow, heun, series);
-    const bool alt = win == ssk::kWinOff && four_bead_alt<T>(e.M, e.W, e.B, c->sms, max_logs, flow, heun, series);
+    // (elements beside one another fill each other's waves: the first form)
+    const bool alt = win == ssk::kWinOff && c->el.size() == 1 &&
+                     second_form<T>(e.M, e.W, e.B, c->sms, max_logs, flow, heun, series);
     const void* kern = chunk_fn<T>(e.W, e.B, win, flow, heun, corr, alt);
     if (!kern) return fail(c, SS_EINVAL, "no chain kernel for this layout");
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
@@ -1263,7 +1267,7 @@ template <typename T>
 int resident_warps(const ss_ctx* c, const Elem& e, bool flow) {
     const bool heun = c->P.integrator == SS_HEUN, series = c->levels > 0;
     const int nlog = logs_per_launch<T>(c, e, flow, heun, series);
-    const bool alt = four_bead_alt<T>(e.M, e.W, e.B, c->sms, nlog, flow, heun, series);
+    const bool alt = second_form<T>(e.M, e.W, e.B, c->sms, nlog, flow, heun, series);
     return chunk_resident<T>(e.W, e.B, nlog, flow, heun, series, alt);
 }
 
@@ -2099,12 +2103,12 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
         a.series_row0 = 0;
     }
     bool alt = false;
-    if (W == 16 && B == 4) {
+    if (sizeof(T) == 4 && ssk::has_second_form(W, B, false, flow)) {
         int dev = 0, sms = 1;
         if (cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
             return SS_ECUDA;
-        alt = four_bead_alt<T>(M, W, B, sms, 0, flow, false, c->levels > 0);
+        alt = second_form<T>(M, W, B, sms, 0, flow, false, c->levels > 0);
     }
     const void* kern = chunk_fn<T>(W, B, ssk::kWinOff, flow, false, c->levels > 0, alt);
     if (!kern) return SS_EINVAL;

@@ -320,22 +320,29 @@ constexpr int kCounterCopies = 64;  // power of two
 // warps, 28.8 at 20 with the spills of 96 registers).  FP64 work is bound by the
 // FP64 pipe long before twelve warps.
 //
-// Sixteen lanes of four beads (N = 49..64) spill 136-188 bytes at 128 registers and none
-// at 168 (N = 62, 9000 chains, 400 steps: 2.97 -> 2.67 ms; N = 56, 16000 chains: 4.62 ->
-// 4.20), but 12 warps/SM take a second wave for what 16 take in one.  So the chain
-// kernel has two forms there (ALT the second), which give the same bits, and the host
-// takes the better one by the waves of an ensemble (four_bead_alt).
-//   Euler-Maruyama   12 warps, or 16 with reduction batches of two steps
-//   Heun             128 registers, batches of five steps (13 warps by shared memory) or
-//                    of two (16); with 168 registers the compiler contracts its sums in
-//                    another order and the results differ in the last bits
-//   Heun with flow   10 warps (168 registers, of which 12 fit), or 8 without spills
+// A kernel of fewer warps with more registers does as much per time or more, but takes a
+// second wave for what more warps take in one.  Some layouts therefore have two forms
+// (ALT the second), which give the same bits, and the host takes the better one by the
+// waves of an ensemble (second_form):
+//   16 x 4 (N = 49..64), Euler-Maruyama: 168 registers without spills, 12 warps, or 128
+//     with 130-190 bytes of spills, 16 warps (N = 62, 9000 chains, 400 steps: 2.97 -> 2.67
+//     ms at 12; N = 56, 16000 chains: 4.62 -> 4.20)
+//   16 x 4, Heun: 128 registers, 13 warps by shared memory with reduction batches of five
+//     steps, 16 with two; with 168 registers the compiler contracts its sums in another
+//     order and the results differ in the last bits
+//   16 x 4, Heun with flow: 10 warps (168 registers, of which 12 fit), or 8 without spills
+//   16 x 3 and 8 x 3 with flow: 16 or 20 warps; with Heun 12 or 16
+//   16 x 2, Heun with flow: 16 or 20 warps
+constexpr bool has_second_form(int W, int B, bool heun, bool flow) {
+    return (W == 16 && B == 4) || (W <= 16 && B == 3 && flow) || (W == 16 && B == 2 && heun && flow);
+}
 template <typename T>
 constexpr int chunk_warps_per_sm(int W, int B, bool heun = false, bool flow = false, bool alt = false) {
     if (sizeof(T) == 8) return heun && flow ? 8 : 12;
     if (W == 16 && B == 4) return heun && flow ? (alt ? 8 : 10) : (heun || alt ? 16 : 12);
-    if (heun && flow) return B == 1 ? 20 : (B == 2 ? 16 : 12);  // both states live at once
-    return B == 1 ? 24 : (B == 2 ? 20 : 16);
+    const int more = alt ? 4 : 0;
+    if (heun && flow) return B == 1 ? 20 : (B == 2 ? 16 : 12) + more;  // both states live at once
+    return B == 1 ? 24 : (B == 2 ? 20 : 16) + more;
 }
 
 // Columns of a chain's row in device memory (R, A [3][NP], S, tape [NP]): a
@@ -362,7 +369,10 @@ constexpr int kRedSteps = 5;
 // of a chain kernel whose stress series may be written (0: FP64, no batches)
 template <typename T>
 constexpr int red_steps(int W, int B, bool heun, bool flow, bool alt) {
-    return sizeof(T) == 8 ? 0 : (alt && !(heun && flow) ? 2 : kRedSteps);
+    if (sizeof(T) == 8) return 0;
+    // a second form of more warps: as many as leave room for them
+    if (alt && heun && flow) return B == 3 ? 4 : kRedSteps;
+    return alt ? 2 : kRedSteps;
 }
 // Rows of W + 4 words, so that eight lanes reading 16 bytes of eight rows each
 // cover every bank once; the chains of a warp lie W words (mod 32) apart, so that
@@ -1629,7 +1639,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 // velocity-gradient terms are compiled in (launches with kappa = 0 throughout
 // may use the instantiation without them).  HEUN: the stochastic Heun
 // integrator instead of Euler-Maruyama for substep 1.  CORR: a stress series may
-// be written (without one, its registers are free).  ALT: the second form of 16 x 4.
+// be written (without one, its registers are free).  ALT: the second form of a layout.
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, bool ALT = false>
 __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B, HEUN, FLOW, ALT))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {

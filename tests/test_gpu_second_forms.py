@@ -1,7 +1,7 @@
-"""The two forms of the chain kernel for N = 49..64, bit for bit.
+"""The two forms of the chain kernel in layouts that have them, bit for bit.
 
-Which form runs follows the number of chains: the first up to 12 warps per SM (13 with
-Heun, eight of the second with Heun and a flow), the second where that saves a wave.
+Which form runs follows the number of chains: the second where that saves a wave of
+warps (at N = 49..64 with Heun and a flow in small ensembles, too).
 Chains of one seed and global id draw the same numbers in any ensemble, and both forms
 round alike, so the first 64 chains are equal in states and correlator sums whatever
 ensemble they are part of.
@@ -31,22 +31,36 @@ def _run(M, N, flow, integrator, levels):
     return out
 
 
-@pytest.mark.parametrize("N", [49, 62])
-@pytest.mark.parametrize("flow", [False, True])
-@pytest.mark.parametrize("integrator", [0, 1])
-@pytest.mark.parametrize("levels", [-1, 4])
-def test_first_chains_are_the_same_in_any_ensemble(cuda_ok, N, flow, integrator, levels):
+def _check(N, flow, integrator, levels, per_sm):
     import torch
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     ref, acc, log = _run(64, N, flow, integrator, levels)
-    # two chains per warp: 9, 14 and 29 warps per SM
-    for M in (18 * sms + 1, 28 * sms, 58 * sms):
+    for chains in per_sm:
+        M = chains * sms + 1
         st, a, lg = _run(M, N, flow, integrator, levels)
         for k in ("Z", "S", "R", "A"):
             assert np.array_equal(st[k][:64], ref[k]), (M, k)
         if levels > 0:  # FP64 sums of a slice's parts, 16 or 32 chains each
             assert np.allclose(a, acc, rtol=1e-13, atol=1e-13 * np.abs(acc).max())
         assert np.allclose(lg, log, rtol=1e-12, atol=1e-9)
+
+
+# two chains per warp: 9, 14 and 29 warps per SM
+@pytest.mark.parametrize("N", [49, 62])
+@pytest.mark.parametrize("flow", [False, True])
+@pytest.mark.parametrize("integrator", [0, 1])
+@pytest.mark.parametrize("levels", [-1, 4])
+def test_four_beads_per_lane(cuda_ok, N, flow, integrator, levels):
+    _check(N, flow, integrator, levels, (18, 28, 58))
+
+
+# with a flow: 18 warps per SM of sixteen lanes (14 with Heun at three beads) and, from
+# 8192 chains on, of eight
+@pytest.mark.parametrize("N,integrator,per_sm", [(33, 0, 36), (48, 0, 36), (24, 0, 72), (17, 0, 72), (18, 1, 36),
+                                                 (32, 1, 36), (35, 1, 28), (48, 1, 28)])
+@pytest.mark.parametrize("levels", [-1, 4])
+def test_flow_at_two_and_three_beads(cuda_ok, N, integrator, per_sm, levels):
+    _check(N, True, integrator, levels, (per_sm,))
 
 
 @pytest.mark.parametrize("flow", [False, True])
