@@ -172,8 +172,9 @@ int ss_set_flow_table(ss_ctx* ctx, int n, const int32_t* elem, const int64_t* fr
  * length, precision and default).  Batched mode keeps the stress logs, not the
  * correlator: ss_run fails with SS_EINVAL unless corr_levels < 0.  The
  * numbers drawn, the states and the event counts are those of the per-element
- * path bit for bit, the stress logs those up to the rounding of sums over the
- * beads of a chain and over chains.  enable = 0 returns to the per-element path and its default
+ * path bit for bit, whatever their layouts, and the stress logs do not depend on
+ * the layout; they differ from the per-element path's by the rounding of sums
+ * over the beads of a chain and over chains.  enable = 0 returns to the per-element path and its default
  * layouts. */
 int ss_set_batched(ss_ctx* ctx, int enable);
 

@@ -961,8 +961,7 @@ int autotune(ss_ctx* c) {
                 // the default layout (the first candidate) gives way only to one
                 // at least a quarter faster: the candidates are within a few percent
                 // of one another near the lines of the default, and a choice by
-                // timing noise would change the rounding of the stress from one
-                // process to the next
+                // timing noise would differ from one process to the next
                 size_t pick = 0;
                 for (size_t ci = 1; ci < cand.size(); ++ci)
                     if (cand_ms[ci] < 0.75f * cand_ms[0] && cand_ms[ci] < cand_ms[pick]) pick = ci;

@@ -622,7 +622,9 @@ __device__ __forceinline__ KappaState kappa_at(Args& a, int ki, long long t0, in
 // Sub-slots of even and of odd b are the beads of lanes l and l + 8 of a 16-lane
 // segment; summing them apart and adding the two is the first round of that
 // segment's reduction, so every sum over beads is rounded as there.
-template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, int VL, int RED, typename Args>
+// PAIR (one bead per lane): the stress of a log step is summed as with two beads per
+// lane, those of lanes l and l + W/2 in one fused sum.
+template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, int VL, int RED, bool PAIR, typename Args>
 __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const int cta_first,
                                            const T NkT, const long long t0_, const int nsteps_,
                                            const long long log_m0_, const int nlog_) {
@@ -1496,6 +1498,26 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             // again with its diagonal, kept out of the every-step path
             T v[6], dgp[3];
             stress_parts(v, dgp, true);
+            if constexpr (PAIR) {
+                static_assert(B == 1 && VL == 1, "lanes of one bead");
+                constexpr int H = W / 2;
+                const T ks_h = ll + H < Z ? c.k_s : T(0);  // stiffness of the upper lane's slot
+                T q[3], d[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    q[k] = __shfl_down_sync(kFull, Q[0][k], H, W);
+                    d[k] = __shfl_down_sync(kFull, dd[0][k], H, W);
+                }
+                const bool low = ll < H;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {  // xy, xz, yz
+                    const int a0 = k == 2 ? 1 : 0, a1 = k == 0 ? 1 : 2;
+                    const T b = fma(c.k_b * q[a0], q[a1], v[k]);
+                    v[k] = low ? b : T(0);
+                    v[3 + k] = low ? fma(ks_h * d[a0], d[a1], sv[0][k]) + b : T(0);
+                    dgp[k] = low ? fma(c.k_b * q[k], q[k], dgp[k]) : T(0);
+                }
+            }
             const T r6 = seg_reduce6<T, W>(v, ll);
             T sig[3], dg[3];
 #pragma unroll
@@ -1643,7 +1665,7 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
 template <typename T, int W, int B, int WIN, bool FLOW, bool HEUN, bool CORR, bool ALT = false>
 __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B, HEUN, FLOW, ALT))
     chunk_kernel(const ChunkArgs a, const StepConst<T> c) {
-    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1, CORR ? red_steps<T>(W, B, HEUN, FLOW, ALT) : 0>(
+    run_chains<T, W, B, WIN, FLOW, HEUN, CORR, W == 8 ? 2 : 1, CORR ? red_steps<T>(W, B, HEUN, FLOW, ALT) : 0, false>(
         a, c, (blockIdx.x + a.cta0) * (blockDim.x / W), c.NkT, a.t0, a.nsteps, a.log_m0, a.nlog_chunk);
 }
 
@@ -1673,12 +1695,14 @@ __global__ void __launch_bounds__(kChunkThreads, chunk_warps_per_sm<T>(W, B))
         args_s[i] = reinterpret_cast<const unsigned long long*>(elems + wi.x)[i];
     __syncthreads();
     const int nlog = a.log_every > 0 ? (int)((info.t0 + info.nsteps) / a.log_every - info.t0 / a.log_every) : 0;
-    // 8 x 2 adds the stress of a lane's two beads in one fused sum here and in two
-    // in chunk_kernel: the stress logs of the two paths differ by FP32 rounding there.
-    // The centre of mass, the only sum over beads that enters a state, is the same
-    // either way.
+    // 8 x 2 adds the stress of a lane's two beads in one fused sum here and in two in
+    // chunk_kernel: the stress logs of the two paths differ by FP32 rounding there.  (The
+    // centre of mass, the only sum over beads that enters a state, is the same either
+    // way.)  16 x 1 and 32 x 1 sum as 8 x 2 and 16 x 2 do, so that the logs of a length
+    // are the same in every layout it may run in.
+    constexpr bool PAIR = B == 1 && W > 8;
     constexpr int VL = W == 8 && B != 2 ? 2 : 1;
-    run_chains<T, W, B, kWinOff, true, false, false, VL, 0>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
+    run_chains<T, W, B, kWinOff, true, false, false, VL, 0, PAIR>(a, c, wi.y, T((double)a.N) * c.kT, info.t0, info.nsteps,
                                                         info.log_m0, nlog);
 }
 
