@@ -263,6 +263,14 @@ const void* chunk_fn(int W, int B, int win, bool flow, bool heun, bool corr, boo
         return flow ? ssk::chunk_fn_f64_flow(W, B, win, heun, corr, alt) : ssk::chunk_fn_f64(W, B, win, heun, corr, alt);
     return flow ? ssk::chunk_fn_f32_flow(W, B, win, heun, corr, alt) : ssk::chunk_fn_f32(W, B, win, heun, corr, alt);
 }
+// Lets a kernel be launched with more than the default 48 KiB of dynamic shared memory
+// (fixed: its static shared memory).  The limit belongs to the function on the current
+// device, not to a context: it is always set to all that an SM offers a CTA, so that no
+// context or thread lowers what another one's launches or graphs need.
+cudaError_t allow_smem(const void* fn, int bytes, int fixed = 0) {
+    if (bytes <= 48 * 1024 - fixed) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - fixed);
+}
 // its shared memory with nlog log steps; series: a stress series may be written
 template <typename T>
 int chunk_smem(int W, int B, int nlog, bool flow, bool heun, bool series, bool alt) {
@@ -526,10 +534,7 @@ int launch_chunk(ss_ctx* c, Elem& e, int m0, int m1, long long t0, int nsteps, c
         a.series_row0 = row0 + done;
         a.nlog_chunk = a.log_every > 0 ? (int)((a.t0 + a.nsteps) / a.log_every - a.t0 / a.log_every) : 0;
         const int smem = chunk_smem<T>(e.W, e.B, a.nlog_chunk, flow, heun, series, alt);
-        // the attribute belongs to the current device: set it on every launch that
-        // needs more than the default 48 KiB (a host call per launch of many steps)
-        if (smem > 48 * 1024)
-            SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        SS_CUDA(c, allow_smem(kern, smem));
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         if (c->timing) {
             SS_CUDA(c, cudaEventCreate(&ev0));
@@ -939,8 +944,7 @@ int autotune(ss_ctx* c) {
                     desc.counters = dcnt;
                     desc.status = reinterpret_cast<int32_t*>(dcnt + 8 * ssk::kCounterCopies);
                     const int smem = batched_smem_bytes<T>(k, 0);
-                    SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    smem));
+                    SS_CUDA(c, allow_smem(batched_fn_of<T>(k), smem, sizeof(ssk::ChunkArgs)));
                     SS_CUDA(c, cudaMemcpy(dd, &desc, sizeof(desc), cudaMemcpyHostToDevice));
                     SS_CUDA(c, cudaMemcpy(di, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice));
                     cudaEvent_t e0, e1;
@@ -1020,7 +1024,7 @@ int batched_prepare(ss_ctx* c) {
         bc.items = c->d_items + off;
         bc.n_items = (int)cls[k].size();
         bc.smem = batched_smem_bytes<T>(k, c->batch_logs);
-        SS_CUDA(c, cudaFuncSetAttribute(batched_fn_of<T>(k), cudaFuncAttributeMaxDynamicSharedMemorySize, bc.smem));
+        SS_CUDA(c, allow_smem(batched_fn_of<T>(k), bc.smem, sizeof(ssk::ChunkArgs)));
         ssk::RunInfo info{0, 1, 0};
         ssk::StepConst<T> sc = step_const<T>(c, 32);
         const ssk::ChunkArgs* pe = c->d_elems;
@@ -1142,8 +1146,7 @@ int launch_adjoint(ss_ctx* c, Elem& e, int seg) {
     const int smem = kWarpsPerCta * 32 * B * (int)(2 * sizeof(ssk::Pos<T>) + sizeof(ssk::SlotRec<T>) + 8);
     const void* kern = sizeof(T) == 8 ? ssk::adjoint_fn_f64(W, B) : ssk::adjoint_fn_f32(W, B);
     if (!kern) return fail(c, SS_EINVAL, "no adjoint kernel for this layout");
-    if (smem > 48 * 1024)
-        SS_CUDA(c, cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    SS_CUDA(c, allow_smem(kern, smem));
     const int ctas = (e.M + chains_per_cta(W) - 1) / chains_per_cta(W);
     ssk::StepConst<T> sc = step_const<T>(c, e.N);
     void* args[] = {(void*)&a, (void*)&sc};
@@ -2113,9 +2116,7 @@ int noalloc_launches(ss_ctx* c, int W, int B, const ss_params& p, int M, int N, 
     if (!kern) return SS_EINVAL;
     const int cpc = chains_per_cta(W);
     const int smem = chunk_smem<T>(W, B, 0, flow, false, c->levels > 0, alt);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return SS_ECUDA;
+    if (allow_smem(kern, smem) != cudaSuccess) return SS_ECUDA;
     ssk::StepConst<T> sc = step_const<T>(c, N);
     void* args[] = {(void*)&a, (void*)&sc};
     int64_t done = 0;
