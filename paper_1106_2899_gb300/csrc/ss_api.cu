@@ -144,9 +144,11 @@ int fail(ss_ctx* c, int code, const std::string& msg) {
 #define SS_CUDA(ctx, call)                                                                  \
     do {                                                                                    \
         cudaError_t e_ = (call);                                                            \
-        if (e_ != cudaSuccess)                                                              \
+        if (e_ != cudaSuccess) {                                                            \
+            cudaGetLastError(); /* reported here: not to be found again by a later call */  \
             return fail((ctx), e_ == cudaErrorMemoryAllocation ? SS_ENOMEM : SS_ECUDA,      \
                         std::string(#call) + ": " + cudaGetErrorString(e_));                 \
+        }                                                                                   \
     } while (0)
 
 size_t tsize(const ss_ctx* c) { return c->prec == SS_FP64 ? sizeof(double) : sizeof(float); }

@@ -69,3 +69,15 @@ def test_contexts_in_threads(cuda_ok):
     for t in threads:
         t.join()
     assert not errors, errors
+
+
+def test_an_error_is_reported_once(cuda_ok):
+    """A context too large for the device fails, and the next one does not."""
+    big = SlipSpring([(1 << 30, 128)], precision="fp32", seed=1)
+    with pytest.raises(Exception, match="ENOMEM"):
+        big.set_params(**synth.PAPER, corr_levels=-1)
+    big.close()
+    g = _ctx([(64, 16)], 0, False)
+    g.run(5)
+    assert g.status() == 0 and g.step == 5
+    g.close()
