@@ -302,6 +302,8 @@ int ss_synchronize(ss_ctx* ctx);
  * (enable = 1), every launch of the chain kernel is bracketed by CUDA events on
  * the context's stream.  ss_kernel_time synchronises and returns the summed
  * event time of those launches and their number, then clears them.
+ * Timed launches follow one another on that stream: elements and parts of an
+ * element do not run side by side meanwhile.
  * enable = 0 stops recording. */
 int ss_kernel_timing(ss_ctx* ctx, int enable);
 int ss_kernel_time(ss_ctx* ctx, double* chain_kernel_ms, int64_t* chain_launches);

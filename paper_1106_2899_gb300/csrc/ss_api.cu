@@ -847,7 +847,10 @@ int batched_launch_direct(ss_ctx* c, int k, const ssk::ChunkArgs* d_elems, const
 // then 8 x 2, which does less per chain (us per step at 4096 / 16384 / 65536 chains:
 // 16 x 1 0.99 / 2.89 / 10.4, 8 x 2 1.35 / 3.10 / 10.0).  N = 17..32: 32 x 1 for
 // ensembles of one wave (1024 chains: 1.27 us per step, 16 x 2 1.5), then 16 x 2, or
-// 8 x 3 as in layout_for.
+// 8 x 3 as in layout_for.  FP64 takes the same lines (us per step: N = 24, 16 x 2 / 8 x 3,
+// 1000 chains 8.4 / 13.0, 9000 57.0 / 53.9, 20000 121 / 98.8; N = 32, 32 x 1 / 16 x 2, 1000
+// 7.05 / 8.9, 20000 126 / 121; N = 16, 16 x 1 / 8 x 2, 1000 4.85 / 9.1, 9000 33.7 / 35.6, 30000
+// 100.9 / 98.0).
 std::vector<std::pair<int, int>> layout_candidates(int N, long long total, long long sms) {
     using L = std::vector<std::pair<int, int>>;
     if (N <= 8) return {{8, 1}};

@@ -516,8 +516,8 @@ __device__ __forceinline__ float trunc_f32(double x, bool& odd) {
 // the bead, the one above and the one below, the 24-bit uniform k.  With vectors
 // truncated to 23 bits a squared length is off by less than 4.2e-7 of itself, the
 // exponent by less than 6e-7 c2 (sum of two squared lengths), a probability by
-// less than 1.1e-7 two_pref times that plus 6e-7 two_pref; the margin is ten times
-// as wide.  Returns false if the uniform lies within it (about 1e-5 of all hops):
+// less than 1.1e-7 two_pref times that plus 6e-7 two_pref; the margin is nine
+// times as wide in the first part and six times in the second.  Returns false if the uniform lies within it (about 1e-5 of all hops):
 // the FP64 probabilities then decide.  These are 70 FP64 instructions (two
 // exponentials, two divisions) of 64 cycles each.
 __device__ __forceinline__ bool hop_filter(const StepConst<double>& c, const double (&r0)[3], const double (&rp)[3],
