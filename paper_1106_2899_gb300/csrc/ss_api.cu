@@ -294,7 +294,8 @@ int chunk_resident(int W, int B, int nlog, bool flow, bool heun, bool series, bo
 // has more warps in the first form, which does more per time (30000 x 60: 15.1 / 17.4 ms;
 // 3000 x 60: 1.87 / 2.53); the second is faster in one wave of its own and in two where the
 // first, of whose warps 12 fit an SM, takes two as well (2300 x 60: 1.67 / 1.59; 3500 x 60:
-// 1.97 / 2.69; 4000 x 60: 2.98 / 2.77).
+// 1.97 / 2.69; 4000 x 60: 2.98 / 2.77).  (Heun figures before its records by slot, which took
+// 4-9% off both forms.)
 template <typename T>
 bool second_form(int M, int W, int B, int sms, int nlog, bool flow, bool heun, bool series) {
     if (sizeof(T) == 8 || !ssk::has_second_form(W, B, heun, flow)) return false;

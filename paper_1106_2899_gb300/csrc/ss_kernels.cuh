@@ -833,12 +833,19 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
     // bead of three or more can add them in slot order.  The masks and the records
     // of beads 0 .. NL - 1 are zero before: each slot clears what it wrote before
     // it moves.  loc: this slot's record; more3: some bead of the warp has three.
+    // With BY_SLOT (Heun at three and four beads per lane) every record is written by
+    // slot as well while some bead has three, so that the sums in slot order read them
+    // without a search: that kernel gathers twice a step with a flow and is short of
+    // registers (us of 200 steps, before / with: 16000 x 60 3122 / 2927, with shear 4185 /
+    // 3997, 16000 x 48 with shear 2810 / 2517, 16000 x 128 4764 / 4369; in the Euler-Maruyama
+    // step, which gathers once, it cost 2.4% at N = 32).
     // The slots of an idle lane (no spring) do the same work without a branch: a
     // stale S is a valid bead, and their record is their own slot's, which nothing
     // reads.  Sub-slots at or above every Z of the warp are skipped (the first
     // never is).
     int loc[SB];
     bool more3 = false;
+    constexpr bool BY_SLOT = HEUN && B >= 3;
     auto skip = [&](int b, int z) { return b > 0 && b * W >= z; };
     auto register_springs = [&](const T (&d)[SB][3]) {
         bool third = false;
@@ -863,6 +870,22 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
             }
         }
         more3 = __any_sync(kFull, third);
+        if constexpr (BY_SLOT) {
+            if (more3) {
+#pragma unroll
+                for (int b = 0; b < SB; ++b) {
+                    const int i = ll + b * W;
+                    if (!skip(b, z_w)) {
+                        SlotRec<T> r;
+                        r.x = d[b][0];
+                        r.y = d[b][1];
+                        r.z = d[b][2];
+                        r.s = i;
+                        tab[i] = r;
+                    }
+                }
+            }
+        }
     };
     auto spring_vectors = [&](T (&d)[SB][3]) {
 #pragma unroll
@@ -885,6 +908,9 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                 r.x = ps.x - A[b][0];
                 r.y = ps.y - A[b][1];
                 r.z = ps.z - A[b][2];
+                if constexpr (BY_SLOT) {
+                    if (more3) tab[ll + b * W] = r;
+                }
             }
         }
     };
@@ -1037,11 +1063,12 @@ __device__ __forceinline__ void run_chains(Args& a, const StepConst<T>& c, const
                     Mask mb = msk[ll + b * W];
                     if (mask_popc(mb) > 2) {
                         // the springs of the mask in slot order: the first two, then the rest
-                        const int j0 = rec[ll + b * W].s, j1 = rec[NL + ll + b * W].s;
+                        const int j0 = BY_SLOT ? 0 : rec[ll + b * W].s, j1 = BY_SLOT ? 0 : rec[NL + ll + b * W].s;
                         auto take = [&]() {
                             const int j = mask_ffs(mb) - 1;
                             mb &= mb - Mask(1);
-                            return rec[j == j0 ? ll + b * W : (j == j1 ? NL + ll + b * W : 2 * NL + j)];
+                            if constexpr (BY_SLOT) return tab[j];
+                            else return rec[j == j0 ? ll + b * W : (j == j1 ? NL + ll + b * W : 2 * NL + j)];
                         };
                         const SlotRec<T> q0 = take(), q1 = take();
                         Fo[b][0] -= c.k_s * (q0.x + q1.x);
